@@ -1,0 +1,225 @@
+// FP64 states as zone-scaled 64-bit integers.
+//
+// Most FP64 instructions of the predictor and face kernels were linear algebra: node states are fixed linear
+// combinations of a zone's modes.  GB300 executes 1.7 FP64 additions per clock and SM, but 58 64-bit integer
+// additions (measured, independent chains on every SM), so these combinations run on integers: a zone's modes
+// of one variable share the exponent of the largest of them, q = mode * 2^s, and sums and differences of q are
+// exact.  Only the products and quotients of the fluxes stay FP64.
+//
+// Precision.  The largest mode keeps all its 53 bits and LSH more below them; the others are cut at the same
+// unit, 2^-(53 + LSH) of the largest.  A node state then carries an error of a few such units before it is
+// rounded once to FP64, where the FP64 sum rounds at every operation to 2^-53 of its partial sums.
+//
+// Measured (FP64, face states): the third-order tile kernel of 64 x 128 x 128 zones 6.28 -> 4.71 ms, 3224 -> 2116
+// FP64 instructions a zone; the step of 256^3 zones 147.7 -> 124.7 ms, of 93 x 75 x 110 zones at second order
+// 3.10 -> 2.74 ms.
+//
+// Range.  HEADROOM = 10 - LSH bits are left above the largest mode for sums; intermediate sums may wrap (the
+// arithmetic is modulo 2^64) as long as no wrapped value is shifted or scaled by a fraction.  Modes of magnitude
+// below 2^-959 count as zero; a variable with a mode that is not finite, or within 2^16 of the largest FP64
+// number, leaves as NaN at every node.
+#pragma once
+#include "common.cuh"
+
+namespace ader {
+
+struct Fix {
+    long long q;
+};
+
+ADER_DEV Fix fix_wrap(unsigned long long q) {
+    Fix r;
+    r.q = (long long)q;
+    return r;
+}
+ADER_DEV Fix operator+(Fix a, Fix b) { return fix_wrap((unsigned long long)a.q + (unsigned long long)b.q); }
+ADER_DEV Fix operator-(Fix a, Fix b) { return fix_wrap((unsigned long long)a.q - (unsigned long long)b.q); }
+ADER_DEV Fix operator-(Fix a) { return fix_wrap(0ull - (unsigned long long)a.q); }
+
+// the upper 64 bits of the 128-bit product
+ADER_DEV long long fix_mulhi(long long a, long long b) {
+#ifdef __CUDA_ARCH__
+    return __mul64hi(a, b);
+#else
+    return (long long)(((__int128)a * b) >> 64);
+#endif
+}
+
+// c a for a literal c (folded at compile time): the nearest integer by a multiplication, a fractional power of
+// two by a shift, any other fraction by the upper half of a product with its 64-bit expansion
+ADER_DEV Fix fix_times(double c, Fix a) {          // c >= 0
+    const long long i = (long long)(c + 0.49999999);
+    const double f = c - (double)i;                 // in (-1/2, 1/2]
+    const double g = f < 0.0 ? -f : f;
+    Fix r = fix_wrap((unsigned long long)a.q * (unsigned long long)i);
+    if (g == 0.0) return r;
+    Fix p;
+    if (g == 0.5) p.q = a.q >> 1;
+    else if (g == 0.25) p.q = a.q >> 2;
+    else if (g == 0.125) p.q = a.q >> 3;
+    else if (g == 0.0625) p.q = a.q >> 4;
+    else if (g == 0.03125) p.q = a.q >> 5;
+    else if (g == 0.015625) p.q = a.q >> 6;
+    else p.q = fix_mulhi(a.q, (long long)(g * 18446744073709551616.0));
+    return f < 0.0 ? r - p : r + p;
+}
+ADER_DEV Fix operator*(double c, Fix a) { return c < 0.0 ? -fix_times(-c, a) : fix_times(c, a); }
+
+template <int NV>
+ADER_DEV Vec<NV, Fix> operator*(double s, const Vec<NV, Fix>& a) {
+    Vec<NV, Fix> r;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) r.v[i] = s * a.v[i];
+    return r;
+}
+
+ADER_DEV long long bits_of(double x) {
+#ifdef __CUDA_ARCH__
+    return __double_as_longlong(x);
+#else
+    long long b;
+    __builtin_memcpy(&b, &x, 8);
+    return b;
+#endif
+}
+ADER_DEV double of_bits(long long b) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double(b);
+#else
+    double x;
+    __builtin_memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+
+// What a zone's node states are built in: the scalar S, and the way in and out.  In general S is the bulk
+// precision R itself and both ways are the identity; FP64 takes Fix with one exponent per variable.
+// Use: include() every mode, close(), then enter() the modes and leave() with the states.
+template <int NV, class R>
+struct PlainFrame {
+    using S = R;
+    ADER_DEV void include(const Vec<NV, R>&) {}
+    ADER_DEV void close() {}
+    ADER_DEV Vec<NV, S> enter(const Vec<NV, R>& m) const { return m; }
+    ADER_DEV Vec<NV, R> leave(const Vec<NV, S>& u) const { return u; }
+};
+
+template <int NV, int LSH>
+struct FixFrame {
+    using S = Fix;
+    unsigned e[NV];       // biased exponent of the largest mode
+    unsigned bad[NV];     // bits that make a value NaN, or none
+
+    ADER_DEV FixFrame() {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) e[v] = 0;
+    }
+    ADER_DEV void include(const Vec<NV, double>& m) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const unsigned h = (unsigned)((unsigned long long)bits_of(m[v]) >> 32) & 0x7ff00000u;
+            e[v] = h > e[v] ? h : e[v];
+        }
+    }
+    ADER_DEV void close() {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            e[v] >>= 20;
+            bad[v] = e[v] > 2046u - 16u ? 0x7ff80000u : 0u;
+            e[v] = e[v] < 64u ? 64u : e[v];
+        }
+    }
+    ADER_DEV Vec<NV, Fix> enter(const Vec<NV, double>& m) const {
+        Vec<NV, Fix> r;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const long long b = bits_of(m[v]);
+            const unsigned long long mant = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
+            const unsigned d = e[v] - ((unsigned)((unsigned long long)b >> 52) & 0x7ffu);
+            const unsigned long long q = (mant << LSH) >> (d < 63u ? d : 63u);
+            const unsigned long long s = (unsigned long long)(b >> 63);
+            r[v] = fix_wrap((q ^ s) - s);
+        }
+        return r;
+    }
+    // the nearest FP64 value (ties away from zero)
+    ADER_DEV double leave_one(int v, Fix u) const {
+        const unsigned long long s = (unsigned long long)(u.q >> 63);
+        const unsigned long long a = ((unsigned long long)u.q ^ s) - s;
+        const unsigned hi = (unsigned)(a >> 32), lo = (unsigned)a;
+        const unsigned top = hi ? hi : lo;
+#ifdef __CUDA_ARCH__
+        const unsigned lz = (unsigned)__clz((int)top) + (hi ? 0u : 32u);
+#else
+        const unsigned lz = (top ? (unsigned)__builtin_clz(top) : 32u) + (hi ? 0u : 32u);
+#endif
+        const unsigned long long n = ((a << (lz - 1u & 63u)) + 0x200ull) >> 10;       // bit 52 is the leading one
+        const unsigned ex = e[v] + (unsigned)(11 - LSH) - lz - 1u;                     // its place adds one
+        unsigned h = (unsigned)(n >> 32) + (ex << 20);
+        h = a ? h : 0u;
+        h |= ((unsigned)s & 0x80000000u) | bad[v];
+        return of_bits((long long)(((unsigned long long)h << 32) | (unsigned)n));
+    }
+    ADER_DEV Vec<NV, double> leave(const Vec<NV, Fix>& u) const {
+        Vec<NV, double> r;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) r[v] = leave_one(v, u[v]);
+        return r;
+    }
+};
+
+// Sum of the Euler flux of direction D over face nodes, kept by its factors so that a node costs few FP64
+// instructions: with r = 1 / rho, v = m_D r and w = |m|^2 r (twice the kinetic energy) the node adds m_i v to the
+// momentum products, E v and w v to the energy's and w to the pressure's.  The pressure P = (gamma - 1)(E - w / 2)
+// is applied to the sums, and the weighted sums of m_D and E themselves are the face averages of the state (the
+// facial quadrature is exact on its basis).  14 FP64 instructions a node where the flux and its addition took 22.
+template <int D, class R>
+struct FluxSum {
+    R p[3] = {R(0), R(0), R(0)}, w = R(0), ev = R(0), wv = R(0);
+
+    template <int SIGN = 1>
+    ADER_DEV void add(const Vec<5, R>& u) {
+        const R r = rcp(u[0]);
+        const R v = SIGN > 0 ? u[1 + D] * r : -(u[1 + D] * r);
+        const R k = (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * r;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) p[c] += u[1 + c] * v;
+        w = SIGN > 0 ? w + k : w - k;
+        ev += u[4] * v;
+        wv += k * v;
+    }
+    ADER_DEV void scale(R c) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) p[i] = c * p[i];
+        w = c * w;
+        ev = c * ev;
+        wv = c * wv;
+    }
+    ADER_DEV void merge(R c, const FluxSum& o) {      // this + c o
+#pragma unroll
+        for (int i = 0; i < 3; ++i) p[i] += c * o.p[i];
+        w += c * o.w;
+        ev += c * o.ev;
+        wv += c * o.wv;
+    }
+    // c times the sum; avg the face average of the state
+    ADER_DEV Vec<5, R> mean(const Vec<5, R>& avg, R gm1, R c) const {
+        Vec<5, R> f;
+        f[0] = avg[1 + D];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) f[1 + i] = c * p[i];
+        f[1 + D] += gm1 * (avg[4] - (R(0.5) * c) * w);
+        f[4] = c * (ev + gm1 * (ev - R(0.5) * wv));
+        return f;
+    }
+};
+
+// The frame of an order: integers for FP64 at orders 2 and 3, with 5 of the 10 bits below the mantissa.  The
+// fourth order keeps FP64 states: its 35 modes and the wider node formulas do not fit the registers, and the integer
+// form only added to what they spill (30.2 -> 31.5 ms for the step of 96^3 zones).
+template <int ORDER, int NV, class R> struct FrameSelect { using T = PlainFrame<NV, R>; };
+template <int NV> struct FrameSelect<2, NV, double> { using T = FixFrame<NV, 5>; };
+template <int NV> struct FrameSelect<3, NV, double> { using T = FixFrame<NV, 5>; };
+template <int ORDER, int NV, class R> using FrameOf = typename FrameSelect<ORDER, NV, R>::T;
+
+}  // namespace ader

@@ -18,9 +18,10 @@ namespace ader {
         template <int NV, class R> static ADER_DEV void predict_nodal(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& n) { \
             o##O::predict_nodal(m, gm1, cx, cy, cz, n);                                                              \
         }                                                                                                            \
-        template <int D, int NV, class R>                                                                            \
-        static ADER_DEV void face(const Vec<NV, R>* p, R gm1, Vec<NV, R>& ub, Vec<NV, R>& avg, Vec<NV, R>& Fa) {     \
-            o##O::face<D>(p, gm1, ub, avg, Fa);                                                                       \
+        template <int D, int NV, class R, class FR>                                                                  \
+        static ADER_DEV void face(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>& ub,             \
+                                  Vec<NV, R>& avg, Vec<NV, R>& Fa) {                                                 \
+            o##O::face<D>(fr, p, gm1, ub, avg, Fa);                                                                   \
         }                                                                                                            \
         template <int D, class R>                                                                                    \
         static ADER_DEV void face_mhd(const Vec<8, R>* p, R gm1, Vec<8, R>& ub, Vec<8, R>& avg, Vec<8, R>& Fa, R* eu, \
@@ -40,9 +41,10 @@ namespace ader {
             o##O::predict_nodal_src(m, gm1, cx, cy, cz, n, s, sdt);                                                  \
         }                                                                                                            \
         static constexpr bool HAS_FACE_PAIR = o##O::HAS_FACE_PAIR;                                                   \
-        template <int D, int NV, class R>                                                                            \
-        static ADER_DEV void face_pair(const Vec<NV, R>* p, R gm1, Vec<NV, R>* ub, Vec<NV, R>* avg, Vec<NV, R>* Fa) {  \
-            o##O::face_pair<D>(p, gm1, ub, avg, Fa);                                                                  \
+        template <int D, int NV, class R, class FR>                                                                  \
+        static ADER_DEV void face_pair(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>* ub,        \
+                                       Vec<NV, R>* avg, Vec<NV, R>* Fa) {                                            \
+            o##O::face_pair<D>(fr, p, gm1, ub, avg, Fa);                                                              \
         }                                                                                                            \
         template <int D, class R>                                                                                    \
         static ADER_DEV void edge_states(const Vec<8, R>* p, const Vec<8, R>& ub, const Vec<8, R>& avg, Vec<8, R>* e) { \

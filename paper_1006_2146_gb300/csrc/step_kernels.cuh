@@ -11,6 +11,7 @@
 // component c = 5 + t the edge's EMF needs.
 #pragma once
 #include "common.cuh"
+#include "fixed.cuh"
 #include "kernels.cuh"
 #include "modes.cuh"
 #include "riemann.cuh"
@@ -75,10 +76,7 @@ ADER_DEV void store_face(const StepArgs& a, long long z, const Vec<NV, R>* m, R 
     to_face_frame<ORDER, D, S>(m, p);
     Vec<NV, R> ub, avg, Fa;
     R eu[4], ef[4];
-    if constexpr (NV == 8)
-        ZoneOps<ORDER>::template face_mhd<D>(p, gm1, ub, avg, Fa, eu, ef);
-    else
-        ZoneOps<ORDER>::template face<D>(p, gm1, ub, avg, Fa);
+    ZoneOps<ORDER>::template face_mhd<D>(p, gm1, ub, avg, Fa, eu, ef);
     write_side<D, S>(a, z, m[1], ub, avg, Fa, gm1);
     if constexpr (NV == 8) {
         constexpr int side = 2 * D + (S < 0 ? 1 : 0);
@@ -101,21 +99,42 @@ ADER_DEV void store_face(const StepArgs& a, long long z, const Vec<NV, R>* m, R 
     }
 }
 
-// both faces of direction D: the paired form where the order has one (Euler), else one face at a time
-template <int ORDER, int D, int NV, class R>
-ADER_DEV void store_faces(const StepArgs& a, long long z, const Vec<NV, R>* m, R gm1) {
-    if constexpr (NV == 5 && ZoneOps<ORDER>::HAS_FACE_PAIR) {
-        constexpr int L = ModeCount<ORDER>::L;
-        Vec<NV, R> p[L + 1];
-        to_face_frame<ORDER, D, +1>(m, p);
-        Vec<NV, R> ub[2], avg[2], Fa[2];
-        ZoneOps<ORDER>::template face_pair<D>(p, gm1, ub, avg, Fa);
-        write_side<D, +1>(a, z, m[1], ub[0], avg[0], Fa[0], gm1);
-        write_side<D, -1>(a, z, m[1], ub[1], avg[1], Fa[1], gm1);
+// ------------------------------------------------------------------ Euler faces from zone-framed states
+// the zone's modes in the state scalar of its frame (fixed.cuh)
+template <int ORDER, int NV, class R>
+ADER_DEV void enter_frame(const Vec<NV, R>* m, FrameOf<ORDER, NV, R>& fr,
+                          Vec<NV, typename FrameOf<ORDER, NV, R>::S>* s) {
+    constexpr int L = ModeCount<ORDER>::L;
+#pragma unroll
+    for (int k = 1; k <= L; ++k) fr.include(m[k]);
+    fr.close();
+#pragma unroll
+    for (int k = 1; k <= L; ++k) s[k] = fr.enter(m[k]);
+}
+
+// the two faces of direction D (index 0 upper, 1 lower): the paired form where the order has one
+template <int ORDER, int D, class R>
+ADER_DEV void both_faces(const FrameOf<ORDER, 5, R>& fr, const Vec<5, typename FrameOf<ORDER, 5, R>::S>* s, R gm1,
+                         Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
+    constexpr int L = ModeCount<ORDER>::L;
+    Vec<5, typename FrameOf<ORDER, 5, R>::S> p[L + 1];
+    to_face_frame<ORDER, D, +1>(s, p);
+    if constexpr (ZoneOps<ORDER>::HAS_FACE_PAIR) {
+        ZoneOps<ORDER>::template face_pair<D>(fr, p, gm1, ub, avg, Fa);
     } else {
-        store_face<ORDER, D, +1>(a, z, m, gm1);
-        store_face<ORDER, D, -1>(a, z, m, gm1);
+        ZoneOps<ORDER>::template face<D>(fr, p, gm1, ub[0], avg[0], Fa[0]);
+        to_face_frame<ORDER, D, -1>(s, p);
+        ZoneOps<ORDER>::template face<D>(fr, p, gm1, ub[1], avg[1], Fa[1]);
     }
+}
+
+template <int ORDER, int D, class R>
+ADER_DEV void store_faces(const StepArgs& a, long long z, const Vec<5, R>& mean, const FrameOf<ORDER, 5, R>& fr,
+                          const Vec<5, typename FrameOf<ORDER, 5, R>::S>* s, R gm1) {
+    Vec<5, R> ub[2], avg[2], Fa[2];
+    both_faces<ORDER, D, R>(fr, s, gm1, ub, avg, Fa);
+    write_side<D, +1>(a, z, mean, ub[0], avg[0], Fa[0], gm1);
+    write_side<D, -1>(a, z, mean, ub[1], avg[1], Fa[1], gm1);
 }
 
 // Iteration statistics of the converged predictor: sum, maximum and capped zones.
@@ -197,9 +216,21 @@ ADER_DEV void zone_predict_faces(const StepArgs& a, const double* __restrict__ U
     Vec<NV, R> m[ModeCount<ORDER>::L + 1];
     zone_predict<ORDER, FORM, NV, R, SRC>(a, U, z, m, bulk_arg<R>(a.dt_dev ? *a.dt_dev : a.dt));
     const R gm1 = arg_gm1<R>(a);
-    store_faces<ORDER, 0>(a, z, m, gm1);
-    store_faces<ORDER, 1>(a, z, m, gm1);
-    store_faces<ORDER, 2>(a, z, m, gm1);
+    if constexpr (NV == 5) {
+        FrameOf<ORDER, 5, R> fr;
+        Vec<5, typename FrameOf<ORDER, 5, R>::S> s[ModeCount<ORDER>::L + 1];
+        enter_frame<ORDER>(m, fr, s);
+        store_faces<ORDER, 0>(a, z, m[1], fr, s, gm1);
+        store_faces<ORDER, 1>(a, z, m[1], fr, s, gm1);
+        store_faces<ORDER, 2>(a, z, m[1], fr, s, gm1);
+    } else {
+        store_face<ORDER, 0, +1>(a, z, m, gm1);
+        store_face<ORDER, 0, -1>(a, z, m, gm1);
+        store_face<ORDER, 1, +1>(a, z, m, gm1);
+        store_face<ORDER, 1, -1>(a, z, m, gm1);
+        store_face<ORDER, 2, +1>(a, z, m, gm1);
+        store_face<ORDER, 2, -1>(a, z, m, gm1);
+    }
 }
 
 // FP32 bulk asks for three 128-thread blocks per SM at orders 2-3 (at most 168 registers, a few hundred
@@ -508,31 +539,12 @@ ADER_DEV void pt_side(R* dst, const Vec<5, R>& mean, Vec<5, R> ub, const Vec<5, 
 }
 
 template <int ORDER, int D, class R>
-ADER_DEV void pt_sides(R* sh, int tid, int slot_plus, int slot_minus, const Vec<5, R>* m, R gm1) {
-    constexpr int L = ModeCount<ORDER>::L;
-    if constexpr (ZoneOps<ORDER>::HAS_FACE_PAIR) {
-        Vec<5, R> p[L + 1];
-        to_face_frame<ORDER, D, +1>(m, p);
-        Vec<5, R> ub[2], avg[2], Fa[2];
-        ZoneOps<ORDER>::template face_pair<D>(p, gm1, ub, avg, Fa);
-        pt_side(pt_slot(sh, slot_plus, tid), m[1], ub[0], avg[0], Fa[0], gm1);
-        pt_side(pt_slot(sh, slot_minus, tid), m[1], ub[1], avg[1], Fa[1], gm1);
-    } else {
-        {
-            Vec<5, R> p[L + 1];
-            to_face_frame<ORDER, D, +1>(m, p);
-            Vec<5, R> ub, avg, Fa;
-            ZoneOps<ORDER>::template face<D>(p, gm1, ub, avg, Fa);
-            pt_side(pt_slot(sh, slot_plus, tid), m[1], ub, avg, Fa, gm1);
-        }
-        {
-            Vec<5, R> p[L + 1];
-            to_face_frame<ORDER, D, -1>(m, p);
-            Vec<5, R> ub, avg, Fa;
-            ZoneOps<ORDER>::template face<D>(p, gm1, ub, avg, Fa);
-            pt_side(pt_slot(sh, slot_minus, tid), m[1], ub, avg, Fa, gm1);
-        }
-    }
+ADER_DEV void pt_sides(R* sh, int tid, int slot_plus, int slot_minus, const Vec<5, R>& mean,
+                       const FrameOf<ORDER, 5, R>& fr, const Vec<5, typename FrameOf<ORDER, 5, R>::S>* s, R gm1) {
+    Vec<5, R> ub[2], avg[2], Fa[2];
+    both_faces<ORDER, D, R>(fr, s, gm1, ub, avg, Fa);
+    pt_side(pt_slot(sh, slot_plus, tid), mean, ub[0], avg[0], Fa[0], gm1);
+    pt_side(pt_slot(sh, slot_minus, tid), mean, ub[1], avg[1], Fa[1], gm1);
 }
 
 template <class R>
@@ -629,9 +641,12 @@ __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 3 : 1)
         if (valid) {
             Vec<5, R> m[ModeCount<ORDER>::L + 1];
             zone_predict<ORDER, FORM, 5, R, SRC>(a, U, z, m, dt);
-            pt_sides<ORDER, 0>(sh, tid, 0, 1, m, gm1);
-            pt_sides<ORDER, 1>(sh, tid, 2, 3, m, gm1);
-            pt_sides<ORDER, 2>(sh, tid, zp_slot, 5, m, gm1);
+            FrameOf<ORDER, 5, R> fr;
+            Vec<5, typename FrameOf<ORDER, 5, R>::S> s[ModeCount<ORDER>::L + 1];
+            enter_frame<ORDER>(m, fr, s);
+            pt_sides<ORDER, 0>(sh, tid, 0, 1, m[1], fr, s, gm1);
+            pt_sides<ORDER, 1>(sh, tid, 2, 3, m[1], fr, s, gm1);
+            pt_sides<ORDER, 2>(sh, tid, zp_slot, 5, m[1], fr, s, gm1);
         }
         __syncthreads();
         if (valid) {

@@ -2,6 +2,7 @@
 // face quantities (Sec. V.1, App. D).  Modes m[1..5] (Eq. 14).
 #pragma once
 #include "common.cuh"
+#include "fixed.cuh"
 #include "modes.cuh"
 
 namespace ader {
@@ -120,13 +121,19 @@ ADER_DEV void predict_nodal_src(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl&
 
 // Eqs. 58-59 and D.3-D.5: composing D.4 with D.5, <F> is the mean of the flux
 // at the four tau = 1/2 facial nodes (node 5 enters only through the time mode).
-template <int D, int NV, class R>
-ADER_DEV void face(const Vec<NV, R>* p, R gm1, Vec<NV, R>& ub, Vec<NV, R>& avg, Vec<NV, R>& Fa) {
-    ub = p[1] + 0.5 * (p[2] + p[5]);
+template <int D, int NV, class R, class FR>
+ADER_DEV void face(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>& ub, Vec<NV, R>& avg,
+                   Vec<NV, R>& Fa) {
+    using V = Vec<NV, typename FR::S>;
+    const V q1 = p[1] + 0.5 * (p[2] + p[5]), h3 = 0.5 * p[3], h4 = 0.5 * p[4];
+    ub = fr.leave(q1);
     avg = ub;
-    const Vec<NV, R> q1 = ub;
-    Fa = 0.25 * (flux<D>(q1 + 0.5 * p[3], gm1) + flux<D>(q1 - 0.5 * p[3], gm1) + flux<D>(q1 + 0.5 * p[4], gm1) +
-                 flux<D>(q1 - 0.5 * p[4], gm1));
+    FluxSum<D, R> sum;
+    sum.add(fr.leave(q1 + h3));
+    sum.add(fr.leave(q1 - h3));
+    sum.add(fr.leave(q1 + h4));
+    sum.add(fr.leave(q1 - h4));
+    Fa = sum.mean(avg, gm1, R(0.25));
 }
 
 // MHD face: also the edge averages (Eq. 60 for <u>, Eqs. D.4-D.5 for <F>) of
@@ -171,8 +178,8 @@ ADER_DEV void edge_states(const Vec<8, R>* p, const Vec<8, R>& ub, const Vec<8, 
 
 // No paired-face form at this order: the faces are evaluated one at a time.
 constexpr bool HAS_FACE_PAIR = false;
-template <int D, int NV, class R>
-ADER_DEV void face_pair(const Vec<NV, R>*, R, Vec<NV, R>*, Vec<NV, R>*, Vec<NV, R>*) {}
+template <int D, int NV, class R, class FR>
+ADER_DEV void face_pair(const FR&, const Vec<NV, typename FR::S>*, R, Vec<NV, R>*, Vec<NV, R>*, Vec<NV, R>*) {}
 
 }  // namespace o2
 }  // namespace ader

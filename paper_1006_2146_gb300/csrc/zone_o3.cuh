@@ -7,6 +7,7 @@
 // to the extracted flux modes.
 #pragma once
 #include "common.cuh"
+#include "fixed.cuh"
 #include "modes.cuh"
 
 namespace ader {
@@ -284,86 +285,74 @@ constexpr bool HAS_SOURCE = true;
 constexpr bool HAS_SOURCE_MODAL = true;
 
 // ------------------------------------------------------------------ x+ face, Sec. V.2 and App. D
-// p = the zone's modes in the face's x-frame (modes.cuh).  Outputs the
+// p = the zone's modes in the face's x-frame (modes.cuh), in the state scalar of the frame fr (fixed.cuh).
+// Outputs the
 // barycentre state (Eq. 61), the face average of u (Eq. 62) and the face
 // average of the physical normal flux: composing Eq. D.9 with D.10 gives
 // <F> = (F1 + F6 + F7 + F8 + F9 + F10) / 6 over the facial nodes of Eq. D.6
 // (the four corner nodes enter only the edge averages).
-template <int D, int NV, class R>
-ADER_DEV void face(const Vec<NV, R>* p, R gm1, Vec<NV, R>& ub, Vec<NV, R>& avg, Vec<NV, R>& Fa) {
-    ub = p[1] + 0.5 * (p[2] + p[11]) + 0.25 * (p[12] + p[13]) + (2.0 * p[5] - p[6] - p[7]) / 12.0;
-    avg = ub + (p[6] + p[7] + p[12]) / 12.0;
-    // Eq. D.8
-    const Vec<NV, R> q1 = 0.5 * p[11] + 0.25 * (p[12] + p[13]);
-    const Vec<NV, R> t1 = p[1] + 0.5 * p[2] + (2.0 * p[5] - p[6] - p[7]) / 12.0;
-    const Vec<NV, R> t2 = t1 + 0.5 * (p[3] + p[4]) + 0.25 * (p[6] + p[7] + p[8] + p[9] + p[10]);
-    const Vec<NV, R> t3 = t2 - p[3] - 0.5 * (p[8] + p[9]);
-    const Vec<NV, R> t4 = t2 - p[4] - 0.5 * (p[9] + p[10]);
-    const Vec<NV, R> t5 = t4 - p[3] - 0.5 * (p[8] - p[9]);
-    const Vec<NV, R> t6 = 0.5 * (t2 + t4) + q1 + 0.25 * (p[14] - p[7]);
-    const Vec<NV, R> t7 = 0.5 * (t3 + t5) + q1 - 0.25 * (p[7] + p[14]);
-    const Vec<NV, R> t8 = 0.5 * (t2 + t3) + q1 + 0.25 * (p[15] - p[6]);
-    const Vec<NV, R> t9 = 0.5 * (t4 + t5) + q1 - 0.25 * (p[6] + p[15]);
-    const Vec<NV, R> t10 = t1 + p[11] + p[12] + 0.5 * p[13];
-    Fa = (flux<D>(t1, gm1) + flux<D>(t6, gm1) + flux<D>(t7, gm1) + flux<D>(t8, gm1) + flux<D>(t9, gm1) +
-          flux<D>(t10, gm1)) / 6.0;
-}
-
 // Both x-faces of one direction at once (Euler).  p is the zone's modes in
 // the frame of the upper face; the lower face's frame differs only in the
 // sign of the modes odd in the normal coordinate (2, 8, 10, 13), so each of
-// face()'s node states is E + O on the upper face and E - O on the lower one,
-// with E its part from the even modes and O from the odd ones.  E and O are
-// face()'s own linear combinations split by parity, each computed once; the
+// the node states of Eq. D.8 is E + O on the upper face and E - O on the lower one,
+// with E its part from the even modes and O from the odd ones, each computed once; the
 // nodes are taken in an order that keeps few of them alive at a time.
 // Index 0 of ub, avg, Fa is the upper face (S = +1), index 1 the lower.
 constexpr bool HAS_FACE_PAIR = true;
 
-template <int D, int NV, class R>
-ADER_DEV void face_pair(const Vec<NV, R>* p, R gm1, Vec<NV, R>* ub, Vec<NV, R>* avg, Vec<NV, R>* Fa) {
-    const Vec<NV, R> t1e = p[1] + (2.0 * p[5] - p[6] - p[7]) / 12.0, t1o = 0.5 * p[2];
-    const Vec<NV, R> q1e = 0.5 * p[11] + 0.25 * p[12], q1o = 0.25 * p[13];
+template <int D, int NV, class R, class FR>
+ADER_DEV void face_pair(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>* ub, Vec<NV, R>* avg,
+                        Vec<NV, R>* Fa) {
+    using V = Vec<NV, typename FR::S>;
+    const V t1e = p[1] + (2.0 * p[5] - p[6] - p[7]) / 12.0, t1o = 0.5 * p[2];
+    const V q1e = 0.5 * p[11] + 0.25 * p[12], q1o = 0.25 * p[13];
     {
-        const Vec<NV, R> ube = t1e + q1e, ubo = t1o + q1o;
-        const Vec<NV, R> avge = ube + (p[6] + p[7] + p[12]) / 12.0;
-        ub[0] = ube + ubo;
-        ub[1] = ube - ubo;
-        avg[0] = avge + ubo;
-        avg[1] = avge - ubo;
+        const V ube = t1e + q1e, ubo = t1o + q1o;
+        const V avge = ube + (p[6] + p[7] + p[12]) / 12.0;
+        ub[0] = fr.leave(ube + ubo);
+        ub[1] = fr.leave(ube - ubo);
+        avg[0] = fr.leave(avge + ubo);
+        avg[1] = fr.leave(avge - ubo);
     }
-    Vec<NV, R> up = flux<D>(t1e + t1o, gm1), lo = flux<D>(t1e - t1o, gm1);       // node 1
+    FluxSum<D, R> up, lo;
+    up.add(fr.leave(t1e + t1o));                                                        // node 1
+    lo.add(fr.leave(t1e - t1o));
     {
-        const Vec<NV, R> e = t1e + p[11] + p[12], o = t1o + 0.5 * p[13];          // node 10
-        up += flux<D>(e + o, gm1);
-        lo += flux<D>(e - o, gm1);
+        const V e = t1e + p[11] + p[12], o = t1o + 0.5 * p[13];                   // node 10
+        up.add(fr.leave(e + o));
+        lo.add(fr.leave(e - o));
     }
-    const Vec<NV, R> t2e = t1e + 0.5 * (p[3] + p[4]) + 0.25 * (p[6] + p[7] + p[9]), t2o = t1o + 0.25 * (p[8] + p[10]);
-    const Vec<NV, R> t3e = t2e - p[3] - 0.5 * p[9], t3o = t2o - 0.5 * p[8];
-    const Vec<NV, R> t4e = t2e - p[4] - 0.5 * p[9], t4o = t2o - 0.5 * p[10];
+    const V t2e = t1e + 0.5 * (p[3] + p[4]) + 0.25 * (p[6] + p[7] + p[9]), t2o = t1o + 0.25 * (p[8] + p[10]);
+    const V t3e = t2e - p[3] - 0.5 * p[9], t3o = t2o - 0.5 * p[8];
+    const V t4e = t2e - p[4] - 0.5 * p[9], t4o = t2o - 0.5 * p[10];
     {
-        const Vec<NV, R> e = 0.5 * (t2e + t4e) + q1e + 0.25 * (p[14] - p[7]), o = 0.5 * (t2o + t4o) + q1o;   // 6
-        up += flux<D>(e + o, gm1);
-        lo += flux<D>(e - o, gm1);
-    }
-    {
-        const Vec<NV, R> e = 0.5 * (t2e + t3e) + q1e + 0.25 * (p[15] - p[6]), o = 0.5 * (t2o + t3o) + q1o;   // 8
-        up += flux<D>(e + o, gm1);
-        lo += flux<D>(e - o, gm1);
-    }
-    const Vec<NV, R> t5e = t4e - p[3] + 0.5 * p[9], t5o = t4o - 0.5 * p[8];
-    {
-        const Vec<NV, R> e = 0.5 * (t4e + t5e) + q1e - 0.25 * (p[6] + p[15]), o = 0.5 * (t4o + t5o) + q1o;   // 9
-        up += flux<D>(e + o, gm1);
-        lo += flux<D>(e - o, gm1);
+        const V e = 0.5 * (t2e + t4e) + q1e + 0.25 * (p[14] - p[7]), o = 0.5 * (t2o + t4o) + q1o;   // 6
+        up.add(fr.leave(e + o));
+        lo.add(fr.leave(e - o));
     }
     {
-        const Vec<NV, R> e = 0.5 * (t3e + t5e) + q1e - 0.25 * (p[7] + p[14]), o = 0.5 * (t3o + t5o) + q1o;   // 7
-        up += flux<D>(e + o, gm1);
-        lo += flux<D>(e - o, gm1);
+        const V e = 0.5 * (t2e + t3e) + q1e + 0.25 * (p[15] - p[6]), o = 0.5 * (t2o + t3o) + q1o;   // 8
+        up.add(fr.leave(e + o));
+        lo.add(fr.leave(e - o));
     }
-    Fa[0] = up / 6.0;
-    Fa[1] = lo / 6.0;
+    const V t5e = t4e - p[3] + 0.5 * p[9], t5o = t4o - 0.5 * p[8];
+    {
+        const V e = 0.5 * (t4e + t5e) + q1e - 0.25 * (p[6] + p[15]), o = 0.5 * (t4o + t5o) + q1o;   // 9
+        up.add(fr.leave(e + o));
+        lo.add(fr.leave(e - o));
+    }
+    {
+        const V e = 0.5 * (t3e + t5e) + q1e - 0.25 * (p[7] + p[14]), o = 0.5 * (t3o + t5o) + q1o;   // 7
+        up.add(fr.leave(e + o));
+        lo.add(fr.leave(e - o));
+    }
+    Fa[0] = up.mean(avg[0], gm1, R(1.0 / 6.0));
+    Fa[1] = lo.mean(avg[1], gm1, R(1.0 / 6.0));
 }
+
+// One face at a time: not used at this order.
+template <int D, int NV, class R, class FR>
+ADER_DEV void face(const FR&, const Vec<NV, typename FR::S>*, R, Vec<NV, R>&, Vec<NV, R>&, Vec<NV, R>&) {}
 
 // MHD face: all ten facial nodes of Eq. D.6; edge averages by Eq. 63 (<u>)
 // and Eqs. D.9-D.10 (<F>) for the field component of each edge's EMF

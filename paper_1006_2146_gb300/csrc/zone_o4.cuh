@@ -2,6 +2,7 @@
 // face quantities (Sec. V.3, App. D).  Modes m[1..35] (Eq. 16).
 #pragma once
 #include "common.cuh"
+#include "fixed.cuh"
 #include "modes.cuh"
 #include "nodal_o4_coeffs.cuh"
 
@@ -470,40 +471,58 @@ ADER_DEV void predict_nodal_src(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl&
 // Eqs. 64-65 for u_b and <u>; Eq. D.13 for the facial nodes; composing
 // Eq. D.14 with D.15, <F> = (11 F1 - 2 (F2 + F5 + F6 + F9) - 3 F14
 // + 3 (F15 + F16 + F17 + F18) + 9 F19 + 3 F24) / 24 over the nodes of Eq. D.11.
-template <int D, int NV, class R>
-ADER_DEV void face(const Vec<NV, R>* p, R gm1, Vec<NV, R>& ub, Vec<NV, R>& avg, Vec<NV, R>& Fa) {
-    const Vec<NV, R> c1 = p[1] + 0.5 * p[21] + 0.25 * p[22] + 0.125 * p[23] +
+template <int D, int NV, class R, class FR>
+ADER_DEV void face(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>& ub, Vec<NV, R>& avg,
+                   Vec<NV, R>& Fa) {
+    using V = Vec<NV, typename FR::S>;
+    const V c1 = p[1] + 0.5 * p[21] + 0.25 * p[22] + 0.125 * p[23] +
                     (4.0 * p[5] - 2.0 * p[6] - 2.0 * p[7] + 2.0 * p[30] - p[31] - p[32]) / 24.0;
-    const Vec<NV, R> c2 = 0.5 * p[2] + 0.05 * p[11] + 0.25 * p[24] + 0.125 * p[27] - (p[16] + p[18]) / 24.0;
-    ub = c1 + c2;
-    avg = ub + (2.0 * p[6] + 2.0 * p[7] + p[16] + p[18] + 2.0 * p[22] + 3.0 * p[23] + p[27] + p[31] + p[32]) / 24.0;
+    const V c2 = 0.5 * p[2] + 0.05 * p[11] + 0.25 * p[24] + 0.125 * p[27] - (p[16] + p[18]) / 24.0;
+    const V sb = c1 + c2;
+    ub = fr.leave(sb);
+    avg = fr.leave(sb + (2.0 * p[6] + 2.0 * p[7] + p[16] + p[18] + 2.0 * p[22] + 3.0 * p[23] + p[27] + p[31] + p[32]) / 24.0);
     // Eq. D.13 (caret terms of spatial modes read as w, G6)
-    const Vec<NV, R> t1 = p[1] + 0.5 * p[2] + 0.05 * p[11] + (4.0 * p[5] - 2.0 * p[6] - 2.0 * p[7] - p[16] - p[18]) / 24.0;
-    const Vec<NV, R> t2 = t1 + 0.5 * p[3] + 0.25 * (p[6] + p[8]) + 0.05 * p[12] + 0.125 * p[16] +
+    const V t1 = p[1] + 0.5 * p[2] + 0.05 * p[11] + (4.0 * p[5] - 2.0 * p[6] - 2.0 * p[7] - p[16] - p[18]) / 24.0;
+    const V t2 = t1 + 0.5 * p[3] + 0.25 * (p[6] + p[8]) + 0.05 * p[12] + 0.125 * p[16] +
                     (0.25 * p[14] - 0.125 * p[19]) / 3.0;
-    const Vec<NV, R> t3 = 0.5 * (t1 + t2) - 0.0625 * p[6] - 0.046875 * p[12] - 0.03125 * p[16];
-    const Vec<NV, R> t5 = 6.0 * t1 + 3.0 * t2 - 8.0 * t3 - 0.375 * p[12];
-    const Vec<NV, R> t6 = t1 + 0.5 * p[4] + 0.25 * (p[7] + p[10]) + 0.05 * p[13] + 0.125 * p[18] +
+    const V t3 = 0.5 * (t1 + t2) - 0.0625 * p[6] - 0.046875 * p[12] - 0.03125 * p[16];
+    const V t5 = 6.0 * t1 + 3.0 * t2 - 8.0 * t3 - 0.375 * p[12];
+    const V t6 = t1 + 0.5 * p[4] + 0.25 * (p[7] + p[10]) + 0.05 * p[13] + 0.125 * p[18] +
                     (0.25 * p[15] - 0.125 * p[17]) / 3.0;
-    const Vec<NV, R> t7 = 0.5 * (t1 + t6) - 0.0625 * p[7] - 0.046875 * p[13] - 0.03125 * p[18];
-    const Vec<NV, R> t9 = 6.0 * t1 + 3.0 * t6 - 8.0 * t7 - 0.375 * p[13];
-    const Vec<NV, R> t10 = t2 + t6 - t1 + 0.25 * p[9] + 0.125 * (p[17] + p[19] + p[20]);
-    const Vec<NV, R> t11 = t10 + t5 - t2 - 0.5 * p[9] - 0.25 * (p[19] + p[20]);
-    const Vec<NV, R> t12 = t10 + t9 - t6 - 0.5 * p[9] - 0.25 * (p[17] + p[20]);
-    const Vec<NV, R> t14 = t1 - (p[31] + p[32]) / 36.0 + (9.0 * p[21] + 3.0 * p[22] + p[23]) / 27.0 + p[24] / 6.0 +
+    const V t7 = 0.5 * (t1 + t6) - 0.0625 * p[7] - 0.046875 * p[13] - 0.03125 * p[18];
+    const V t9 = 6.0 * t1 + 3.0 * t6 - 8.0 * t7 - 0.375 * p[13];
+    const V t10 = t2 + t6 - t1 + 0.25 * p[9] + 0.125 * (p[17] + p[19] + p[20]);
+    const V t11 = t10 + t5 - t2 - 0.5 * p[9] - 0.25 * (p[19] + p[20]);
+    const V t12 = t10 + t9 - t6 - 0.5 * p[9] - 0.25 * (p[17] + p[20]);
+    const V t14 = t1 - (p[31] + p[32]) / 36.0 + (9.0 * p[21] + 3.0 * p[22] + p[23]) / 27.0 + p[24] / 6.0 +
                      (p[27] + p[30]) / 18.0;
-    const Vec<NV, R> t15 = t14 + t10 - t1 +
+    const V t15 = t14 + t10 - t1 +
                      (6.0 * p[25] + 6.0 * p[26] + 2.0 * p[28] + 2.0 * p[29] + 3.0 * p[31] + 3.0 * p[32] +
                       3.0 * p[33] + 3.0 * p[34] + 3.0 * p[35]) / 36.0;
-    const Vec<NV, R> t16 = t15 + t11 - t10 - (6.0 * p[25] + 2.0 * p[28] + 3.0 * p[33] + 3.0 * p[34]) / 18.0;
-    const Vec<NV, R> t17 = t15 + t12 - t10 - (6.0 * p[26] + 2.0 * p[29] + 3.0 * p[34] + 3.0 * p[35]) / 18.0;
-    const Vec<NV, R> t18 = t16 + t17 - t15 + p[9] + 0.5 * p[20] + p[34] / 3.0;
-    const Vec<NV, R> t19 = 2.0 * t14 - t1 + (2.0 * p[22] + 2.0 * p[23] + p[27]) / 9.0;
-    const Vec<NV, R> t24 = t1 - 3.0 * t14 + 3.0 * t19 + 2.0 * p[23] / 9.0;
-    Fa = (11.0 * flux<D>(t1, gm1) - 2.0 * (flux<D>(t2, gm1) + flux<D>(t5, gm1) + flux<D>(t6, gm1) + flux<D>(t9, gm1)) -
-          3.0 * flux<D>(t14, gm1) +
-          3.0 * (flux<D>(t15, gm1) + flux<D>(t16, gm1) + flux<D>(t17, gm1) + flux<D>(t18, gm1)) +
-          9.0 * flux<D>(t19, gm1) + 3.0 * flux<D>(t24, gm1)) / 24.0;
+    const V t16 = t15 + t11 - t10 - (6.0 * p[25] + 2.0 * p[28] + 3.0 * p[33] + 3.0 * p[34]) / 18.0;
+    const V t17 = t15 + t12 - t10 - (6.0 * p[26] + 2.0 * p[29] + 3.0 * p[34] + 3.0 * p[35]) / 18.0;
+    const V t18 = t16 + t17 - t15 + p[9] + 0.5 * p[20] + p[34] / 3.0;
+    const V t19 = 2.0 * t14 - t1 + (2.0 * p[22] + 2.0 * p[23] + p[27]) / 9.0;
+    const V t24 = t1 - 3.0 * t14 + 3.0 * t19 + 2.0 * p[23] / 9.0;
+    // nodes of equal weight in one sum each: 11, -2, 3 (node 14 with -3) and 9
+    FluxSum<D, R> s11, s2, s3, s9;
+    s11.add(fr.leave(t1));
+    s2.add(fr.leave(t2));
+    s2.add(fr.leave(t5));
+    s2.add(fr.leave(t6));
+    s2.add(fr.leave(t9));
+    s3.template add<-1>(fr.leave(t14));
+    s3.add(fr.leave(t15));
+    s3.add(fr.leave(t16));
+    s3.add(fr.leave(t17));
+    s3.add(fr.leave(t18));
+    s9.add(fr.leave(t19));
+    s3.add(fr.leave(t24));
+    s11.scale(R(11.0));
+    s11.merge(R(-2.0), s2);
+    s11.merge(R(3.0), s3);
+    s11.merge(R(9.0), s9);
+    Fa = s11.mean(avg, gm1, R(1.0 / 24.0));
 }
 
 // MHD face: all 24 facial nodes of Eq. D.11 (Eq. D.13); edge averages by
@@ -615,8 +634,8 @@ constexpr bool HAS_SOURCE_MODAL = true;
 
 // No paired-face form at this order: the faces are evaluated one at a time.
 constexpr bool HAS_FACE_PAIR = false;
-template <int D, int NV, class R>
-ADER_DEV void face_pair(const Vec<NV, R>*, R, Vec<NV, R>*, Vec<NV, R>*, Vec<NV, R>*) {}
+template <int D, int NV, class R, class FR>
+ADER_DEV void face_pair(const FR&, const Vec<NV, typename FR::S>*, R, Vec<NV, R>*, Vec<NV, R>*, Vec<NV, R>*) {}
 
 }  // namespace o4
 }  // namespace ader
