@@ -61,7 +61,7 @@ ADER_DEV bool batch_zone(const BatchGroupDev& g, long long gz, const BatchItem*&
 // One block-iteration's problem for kernels that read the full step arguments: every block covers
 // BATCH_ALIGN-aligned zones of one problem, so its item is copied once into shared memory, where the zone
 // code reads it (the zone's stores cannot alias it: nothing is reloaded from global memory or held in
-// registers across them).  Returns this thread's zone index in that problem (>= its n on padding).
+// registers across them).  Returns the zone index of `base` in that problem.
 // Called by every thread of the block.
 __device__ __forceinline__ long long batch_block_item(const BatchGroupDev& g, long long base, BatchItem& it) {
     static_assert(sizeof(BatchItem) % sizeof(int) == 0, "BatchItem is copied as ints");
@@ -70,7 +70,7 @@ __device__ __forceinline__ long long batch_block_item(const BatchGroupDev& g, lo
     for (int w = threadIdx.x; w < (int)(sizeof(BatchItem) / sizeof(int)); w += blockDim.x)
         reinterpret_cast<int*>(&it)[w] = reinterpret_cast<const int*>(g.items + p)[w];
     __syncthreads();
-    return base + threadIdx.x - g.zpad[p];
+    return base - g.zpad[p];
 }
 
 template <int ORDER, class R>
@@ -136,22 +136,32 @@ __global__ void __launch_bounds__(256) kb_cross2(BatchGroupDev g) {
     }
 }
 
-// at most 128 zones per block, three blocks per SM (two at order 4 and for MHD at order 3), as the
-// single-problem FP32 predictor
+// at most 128 zones per block, three blocks per SM (two at order 4), as the single-problem FP32 predictor
 constexpr int BATCH_PREDICT_MAX_THREADS = 128;
 
 // One zone per thread (never persistent): a grid-stride loop around the predictor's body keeps a few
 // more values live through it, and at 168 registers those spill (about 1 KB more local traffic per zone
 // at order 3); the launch covers the padded range (batch_phase_persistent).
 template <int ORDER, int FORM, int NV, class R>
-__global__ void __launch_bounds__(BATCH_PREDICT_MAX_THREADS, ORDER == 4 || (ORDER == 3 && NV == 8) ? 2 : 3)
-    kb_predict_faces(BatchGroupDev g) {
+__global__ void __launch_bounds__(BATCH_PREDICT_MAX_THREADS, ORDER == 4 ? 2 : 3) kb_predict_faces(BatchGroupDev g) {
     __shared__ BatchItem it;                            // the block's arguments (batch_block_item)
     const long long base = (long long)blockIdx.x * blockDim.x;
     if (base >= g.total) return;                        // the whole block
-    const long long z = batch_block_item(g, base, it);
+    const long long z = batch_block_item(g, base, it) + threadIdx.x;
     if (z >= it.a.grid.n) return;
     zone_predict_faces<ORDER, FORM, NV, R>(it.a, it.U, z);
+}
+
+// the same where a team computes a zone: 32 zones and NV warps per block (team.cuh)
+template <int ORDER, int FORM, int NV, class R>
+__global__ void __launch_bounds__(NV * 32, team_blocks<ORDER, NV, R>()) kb_team_predict_faces(BatchGroupDev g) {
+    extern __shared__ __align__(16) unsigned char team_raw[];
+    __shared__ BatchItem it;
+    const long long base = (long long)blockIdx.x * 32;
+    if (base >= g.total) return;                        // the whole block
+    const long long z0 = batch_block_item(g, base, it);
+    if (z0 >= it.a.grid.n) return;                      // 32 zones of padding: the whole block
+    team_zone<ORDER, FORM, NV, false, R>(it.a, it.U, z0 + (threadIdx.x & 31), (R*)team_raw);
 }
 
 // U += dt L(U) in place, dt from the problem's dt_dev: both faces of each direction solved per zone, the
@@ -160,7 +170,7 @@ template <int SOLVER, int NV, class R>
 __global__ void __launch_bounds__(256) kb_flux_update(BatchGroupDev g) {
     __shared__ BatchItem it;
     for (long long base = (long long)blockIdx.x * blockDim.x; base < g.total; base += batch_stride()) {
-        const long long z = batch_block_item(g, base, it);
+        const long long z = batch_block_item(g, base, it) + threadIdx.x;
         if (z >= it.a.grid.n) continue;
         double* U = it.U;
         if constexpr (sizeof(R) == 4)
@@ -174,7 +184,7 @@ template <class R>
 __global__ void __launch_bounds__(256) kb_emf(BatchGroupDev g) {
     __shared__ BatchItem it;
     for (long long base = (long long)blockIdx.x * blockDim.x; base < g.total; base += batch_stride()) {
-        const long long z = batch_block_item(g, base, it);
+        const long long z = batch_block_item(g, base, it) + threadIdx.x;
         if (z >= it.a.grid.n) continue;
         zone_emf<R>(it.a, z);
     }
@@ -184,7 +194,7 @@ template <class R>
 __global__ void __launch_bounds__(256) kb_ct(BatchGroupDev g) {
     __shared__ BatchItem it;
     for (long long base = (long long)blockIdx.x * blockDim.x; base < g.total; base += batch_stride()) {
-        const long long z = batch_block_item(g, base, it);
+        const long long z = batch_block_item(g, base, it) + threadIdx.x;
         if (z >= it.a.grid.n) continue;
         zone_ct<R>(it.a, it.Bf, 1.0, 1, z);
     }

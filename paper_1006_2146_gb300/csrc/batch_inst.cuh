@@ -11,6 +11,8 @@ int batch_phase(int ph, const BatchGroupDev& g, int form, int solver, int thread
                 bool launch, const void** fn) {
     using R = float;
     const void* k = nullptr;
+    size_t smem = 0;
+    bool team = false;
     switch (ph) {
         case PH_TO_F32: k = (const void*)kb_to_f32; break;
         case PH_FACE_B:
@@ -24,8 +26,26 @@ int batch_phase(int ph, const BatchGroupDev& g, int form, int solver, int thread
             if constexpr (ORDER == 4) k = (const void*)kb_cross2<NV, R>;
             break;
         case PH_PREDICT:
-            k = form == FORM_NODAL ? (const void*)kb_predict_faces<ORDER, FORM_NODAL, NV, R>
-                                   : (const void*)kb_predict_faces<ORDER, FORM_MODAL, NV, R>;
+            if (form == FORM_NODAL) {
+                if constexpr (uses_team<ORDER, FORM_NODAL, NV, R>()) {
+                    k = (const void*)kb_team_predict_faces<ORDER, FORM_NODAL, NV, R>;
+                    team = true;
+                } else {
+                    k = (const void*)kb_predict_faces<ORDER, FORM_NODAL, NV, R>;
+                }
+            } else if constexpr (uses_team<ORDER, FORM_MODAL, NV, R>()) {
+                k = (const void*)kb_team_predict_faces<ORDER, FORM_MODAL, NV, R>;
+                team = true;
+            } else {
+                k = (const void*)kb_predict_faces<ORDER, FORM_MODAL, NV, R>;
+            }
+            if (team) {                                 // 32 zones per block, whatever `threads` says
+                threads = NV * 32;
+                blocks = (int)((g.total + 31) / 32);
+                smem = team_smem<ORDER, NV, R>();
+                if (launch && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+                    return -1;
+            }
             break;
         case PH_UPDATE:
             k = solver == SOLVER_LINEARIZED ? (const void*)kb_flux_update<SOLVER_LINEARIZED, NV, R>
@@ -42,7 +62,7 @@ int batch_phase(int ph, const BatchGroupDev& g, int form, int solver, int thread
     if (fn) *fn = k;
     if (!k || !launch) return k ? 1 : 0;
     void* args[] = {(void*)&g};
-    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3((unsigned)threads), args, 0, st) == cudaSuccess ? 1 : -1;
+    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3((unsigned)threads), args, smem, st) == cudaSuccess ? 1 : -1;
 }
 
 template int batch_phase<ADER_BORDER, ADER_BNV>(int, const BatchGroupDev&, int, int, int, int, cudaStream_t, bool,

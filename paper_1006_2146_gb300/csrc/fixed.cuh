@@ -101,6 +101,8 @@ struct PlainFrame {
     ADER_DEV void include(const Vec<NV, R>&) {}
     ADER_DEV void close() {}
     ADER_DEV Vec<NV, S> enter(const Vec<NV, R>& m) const { return m; }
+    ADER_DEV PlainFrame extended(const Vec<NV, R>*, int) const { return *this; }
+    ADER_DEV Vec<NV, S> from(const PlainFrame&, const Vec<NV, S>& u) const { return u; }
     ADER_DEV Vec<NV, R> leave(const Vec<NV, S>& u) const { return u; }
 };
 
@@ -139,6 +141,28 @@ struct FixFrame {
             const unsigned long long q = (mant << LSH) >> (d < 63u ? d : 63u);
             const unsigned long long s = (unsigned long long)(b >> 63);
             r[v] = fix_wrap((q ^ s) - s);
+        }
+        return r;
+    }
+    // this frame, wide enough for the n modes m too; from() brings a state of the narrower frame into it
+    ADER_DEV FixFrame extended(const Vec<NV, double>* m, int n) const {
+        FixFrame r;
+#pragma unroll
+        for (int k = 0; k < n; ++k) r.include(m[k]);
+        r.close();
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            r.e[v] = r.e[v] > e[v] ? r.e[v] : e[v];
+            r.bad[v] |= bad[v];
+        }
+        return r;
+    }
+    ADER_DEV Vec<NV, Fix> from(const FixFrame& o, const Vec<NV, Fix>& u) const {
+        Vec<NV, Fix> r;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const unsigned d = e[v] - o.e[v];
+            r[v].q = u[v].q >> (d < 63u ? d : 63u);
         }
         return r;
     }
@@ -214,12 +238,10 @@ struct FluxSum {
     }
 };
 
-// The frame of an order: integers for FP64 at orders 2 and 3, with 5 of the 10 bits below the mantissa.  The
-// fourth order keeps FP64 states: its 35 modes and the wider node formulas do not fit the registers, and the integer
-// form only added to what they spill (30.2 -> 31.5 ms for the step of 96^3 zones).
-template <int ORDER, int NV, class R> struct FrameSelect { using T = PlainFrame<NV, R>; };
-template <int NV> struct FrameSelect<2, NV, double> { using T = FixFrame<NV, 5>; };
-template <int NV> struct FrameSelect<3, NV, double> { using T = FixFrame<NV, 5>; };
-template <int ORDER, int NV, class R> using FrameOf = typename FrameSelect<ORDER, NV, R>::T;
+// The frame of an order: integers for FP64, with LSH = 5 of the 10 bits below the mantissa at orders 2 and 3, and 3
+// at order 4, whose node formulas form larger sums (up to 106 times a mode).
+template <int LSH, int NV, class R> struct FrameAt { using T = PlainFrame<NV, R>; };
+template <int LSH, int NV> struct FrameAt<LSH, NV, double> { using T = FixFrame<NV, LSH>; };
+template <int ORDER, int NV, class R> using FrameOf = typename FrameAt<ORDER == 4 ? 3 : 5, NV, R>::T;
 
 }  // namespace ader

@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(TM * GROUPS, 1) k_guess_tc(StepArgs a, const d
             for (int k = 0; k < K1; ++k) x[k] = 0.f;
             if (z >= 0) {
                 Vec<NV, R> m[11];
-                load_modes<3>(a, U, z, m);
+                load_modes<3>(SerialTeam<NV, R>{}, a, U, z, m);
                 const float mag = guess_features_f32<NV, R>(m, cx, cy, cz, x, sv);
                 act = mag > (float)GUESS_MAG_MIN;
             }
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(256) k_guess_compact(StepArgs a, const double*
     bool act = false;
     if (z < a.grid.n) {
         Vec<NV, R> m[11];
-        load_modes<3>(a, U, z, m);
+        load_modes<3>(SerialTeam<NV, R>{}, a, U, z, m);
         act = guess_mag_f32<NV, R>(m) > (float)GUESS_MAG_MIN;
         a.Gact[z] = act ? 1 : 0;
         if (!act && Gzero) {

@@ -24,7 +24,9 @@ __global__ void __launch_bounds__(128) k_guess_samples(StepArgs a, const double*
     const long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (z >= a.grid.n) return;
     Vec<NV, double> m[16];
-    load_modes<3>(a, U, z, m);
+    SerialTeam<NV, double> team;
+    team_scales(team, a, a.dt);
+    load_modes<3>(team, a, U, z, m);
 #pragma unroll
     for (int k = 11; k <= 15; ++k) m[k] = vzero<NV, double>();
     const double dt = a.dt;
@@ -34,7 +36,7 @@ __global__ void __launch_bounds__(128) k_guess_samples(StepArgs a, const double*
     float* y = Y + z * mlp_out(NV);
     const double mag = g.ok ? guess_features<NV, double>(m, g, cx, cy, cz, x) : 0.0;
     PredCtl ctl{2, a.tol, a.max_iter, 0, false};
-    o3::predict_modal(m, a.gamma - 1.0, cx, cy, cz, ctl);
+    o3::predict_modal(team, m, ctl);
     const bool use = g.ok && mag > GUESS_MAG_MIN && !ctl.capped;
     if (use) guess_targets<NV, double>(m, g, mag, y);
     ok[z] = use ? 1 : 0;

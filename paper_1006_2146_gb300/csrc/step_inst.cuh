@@ -10,46 +10,30 @@
 
 namespace ader {
 
-#define ADER_ZONEOPS(O)                                                                                              \
-    template <> struct ZoneOps<O> {                                                                                  \
-        template <int NV, class R> static ADER_DEV void predict_modal(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& n) { \
-            o##O::predict_modal(m, gm1, cx, cy, cz, n);                                                              \
-        }                                                                                                            \
-        template <int NV, class R> static ADER_DEV void predict_nodal(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& n) { \
-            o##O::predict_nodal(m, gm1, cx, cy, cz, n);                                                              \
-        }                                                                                                            \
-        template <int D, int NV, class R, class FR>                                                                  \
-        static ADER_DEV void face(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>& ub,             \
-                                  Vec<NV, R>& avg, Vec<NV, R>& Fa) {                                                 \
-            o##O::face<D>(fr, p, gm1, ub, avg, Fa);                                                                   \
-        }                                                                                                            \
-        template <int D, class R>                                                                                    \
-        static ADER_DEV void face_mhd(const Vec<8, R>* p, R gm1, Vec<8, R>& ub, Vec<8, R>& avg, Vec<8, R>& Fa, R* eu, \
-                                      R* ef) {                                                                       \
-            o##O::face_mhd<D>(p, gm1, ub, avg, Fa, eu, ef);                                                           \
-        }                                                                                                            \
-        static constexpr bool HAS_SOURCE = o##O::HAS_SOURCE;                                                         \
-        static constexpr bool HAS_SOURCE_MODAL = o##O::HAS_SOURCE_MODAL;                                             \
-        template <int NV, class R>                                                                                   \
-        static ADER_DEV void predict_modal_src(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& n, const Src<R>& s,  \
-                                               Vec<NV, R>& sdt) {                                                    \
-            o##O::predict_modal_src(m, gm1, cx, cy, cz, n, s, sdt);                                                  \
-        }                                                                                                            \
-        template <int NV, class R>                                                                                   \
-        static ADER_DEV void predict_nodal_src(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& n, const Src<R>& s,  \
-                                               Vec<NV, R>& sdt) {                                                    \
-            o##O::predict_nodal_src(m, gm1, cx, cy, cz, n, s, sdt);                                                  \
-        }                                                                                                            \
-        static constexpr bool HAS_FACE_PAIR = o##O::HAS_FACE_PAIR;                                                   \
-        template <int D, int NV, class R, class FR>                                                                  \
-        static ADER_DEV void face_pair(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>* ub,        \
-                                       Vec<NV, R>* avg, Vec<NV, R>* Fa) {                                            \
-            o##O::face_pair<D>(fr, p, gm1, ub, avg, Fa);                                                              \
-        }                                                                                                            \
-        template <int D, class R>                                                                                    \
-        static ADER_DEV void edge_states(const Vec<8, R>* p, const Vec<8, R>& ub, const Vec<8, R>& avg, Vec<8, R>* e) { \
-            o##O::edge_states<D>(p, ub, avg, e);                                                                      \
-        }                                                                                                            \
+#define ADER_ZONEOPS(O)                                                                                             \
+    template <> struct ZoneOps<O> {                                                                                 \
+        template <bool SRC, class T>                                                                                \
+        static ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& n, const Src<typename T::R>* s,   \
+                                           typename T::V* sdt) {                                                    \
+            o##O::predict_modal<T, SRC>(t, m, n, s, sdt);                                                           \
+        }                                                                                                           \
+        template <bool SRC, class T>                                                                                \
+        static ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& n, const Src<typename T::R>* s,   \
+                                           typename T::V* sdt) {                                                    \
+            o##O::predict_nodal<T, SRC>(t, m, n, s, sdt);                                                           \
+        }                                                                                                           \
+        static constexpr int FACE_NODES = o##O::FACE_NODES, MEAN_NODES = o##O::MEAN_NODES;                          \
+        static ADER_DEV constexpr int mean_node(int k) { return o##O::mean_node(k); }                               \
+        template <bool ALL, class V> static ADER_DEV void face_states(const V* p, V& ub, V& avg, V* t) {            \
+            o##O::face_states<ALL>(p, ub, avg, t);                                                                  \
+        }                                                                                                           \
+        template <class V> static ADER_DEV V face_mean(const V* F) { return o##O::face_mean(F); }                   \
+        template <class V> static ADER_DEV void edge_fluxes(const V* f, int s, V& plus, V& minus) {                 \
+            o##O::edge_fluxes(f, s, plus, minus);                                                                   \
+        }                                                                                                           \
+        template <class V> static ADER_DEV void edge_states(const V* p, const V& ub, const V& avg, V* e) {          \
+            o##O::edge_states(p, ub, avg, e);                                                                       \
+        }                                                                                                           \
     };
 
 #ifndef ADER_ZONEOPS_DEFINED
@@ -57,6 +41,26 @@ namespace ader {
 ADER_ZONEOPS(2)
 ADER_ZONEOPS(3)
 ADER_ZONEOPS(4)
+#endif
+
+#ifndef ADER_BOTH_FACES_DEFINED
+#define ADER_BOTH_FACES_DEFINED
+template <int D, class R>
+ADER_DEV void both_faces_o2(const FrameOf<2, 5, R>& fr, const Vec<5, typename FrameOf<2, 5, R>::S>* s, R gm1,
+                            Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
+    Vec<5, typename FrameOf<2, 5, R>::S> p[6];
+    to_face_frame<2, D, +1>(s, p);
+    o2::face<D>(fr, p, gm1, ub[0], avg[0], Fa[0]);
+    to_face_frame<2, D, -1>(s, p);
+    o2::face<D>(fr, p, gm1, ub[1], avg[1], Fa[1]);
+}
+template <int D, class R>
+ADER_DEV void both_faces_o3(const FrameOf<3, 5, R>& fr, const Vec<5, typename FrameOf<3, 5, R>::S>* s, R gm1,
+                            Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
+    Vec<5, typename FrameOf<3, 5, R>::S> p[16];
+    to_face_frame<3, D, +1>(s, p);
+    o3::face_pair<D>(fr, p, gm1, ub, avg, Fa);
+}
 #endif
 
 #ifdef ADER_ORDER

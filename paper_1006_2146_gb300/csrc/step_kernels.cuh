@@ -16,90 +16,140 @@
 #include "modes.cuh"
 #include "riemann.cuh"
 #include "mlp.cuh"
+#include "team.cuh"
 
 namespace ader {
 
 template <int ORDER> struct ZoneOps;
 
-template <int ORDER, int NV, class R>
-ADER_DEV void load_modes(const StepArgs& a, const double* __restrict__ U, long long z, Vec<NV, R>* m) {
+// the spatial modes of the team's variables (every variable for a thread of its own, one for a warp of a team)
+template <int ORDER, class T>
+ADER_DEV void load_modes(const T& t, const StepArgs& a, const double* __restrict__ U, long long z, typename T::V* m) {
+    using R = typename T::R;
+    constexpr int NV = T::NV;
     const long long N = a.grid.n;
     const R* S1 = (const R*)a.S1;
     const R* S2 = (const R*)a.S2;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
+    for (int i = 0; i < T::NL; ++i) {
+        const int v = t.var(i);
         if constexpr (sizeof(R) == 4)       // FP32 bulk: the zone means from the FP32 copy of the state
-            m[1][v] = v < 5 ? (a.Uf ? a.Uf[v * N + z] : R(U[v * N + z])) : ((const R*)a.ZB)[(v - 5) * N + z];
+            m[1][i] = v < 5 ? (a.Uf ? a.Uf[v * N + z] : R(U[v * N + z])) : ((const R*)a.ZB)[(v - 5) * N + z];
         else
-            m[1][v] = v < 5 ? R(U[v * N + z]) : ((const R*)a.ZB)[(v - 5) * N + z];
+            m[1][i] = v < 5 ? R(U[v * N + z]) : ((const R*)a.ZB)[(v - 5) * N + z];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) m[2 + d][v] = S1[((0 * 3 + d) * NV + v) * N + z];          // w2 w3 w4
+        for (int d = 0; d < 3; ++d) m[2 + d][i] = S1[((0 * 3 + d) * NV + v) * N + z];          // w2 w3 w4
         if (ORDER >= 3) {
 #pragma unroll
-            for (int d = 0; d < 3; ++d) m[5 + d][v] = S1[((1 * 3 + d) * NV + v) * N + z];      // w5 w6 w7
+            for (int d = 0; d < 3; ++d) m[5 + d][i] = S1[((1 * 3 + d) * NV + v) * N + z];      // w5 w6 w7
 #pragma unroll
-            for (int c = 0; c < 3; ++c) m[8 + c][v] = S2[(c * NV + v) * N + z];                 // w8 w9 w10
+            for (int c = 0; c < 3; ++c) m[8 + c][i] = S2[(c * NV + v) * N + z];                 // w8 w9 w10
         }
         if (ORDER == 4) {
 #pragma unroll
-            for (int d = 0; d < 3; ++d) m[11 + d][v] = S1[((2 * 3 + d) * NV + v) * N + z];     // w11 w12 w13
+            for (int d = 0; d < 3; ++d) m[11 + d][i] = S1[((2 * 3 + d) * NV + v) * N + z];     // w11 w12 w13
 #pragma unroll
-            for (int c = 0; c < 7; ++c) m[14 + c][v] = S2[((3 + c) * NV + v) * N + z];          // w14..w20
+            for (int c = 0; c < 7; ++c) m[14 + c][i] = S2[((3 + c) * NV + v) * N + z];          // w14..w20
         }
     }
 }
 
-// the Euler part of one face side: the barycentre state (replaced by the zone
-// average for the wave speeds when it is not physical), <u> and <F>
-template <int D, int S, int NV, class R>
-ADER_DEV void write_side(const StepArgs& a, long long z, const Vec<NV, R>& mean, Vec<NV, R> ub, const Vec<NV, R>& avg,
-                         const Vec<NV, R>& Fa, R gm1) {
-    constexpr int NQ = side_values(NV);
-    const Prim<NV, R> q = primitives(ub, gm1);
-    if (!(ub[0] > R(0)) || !(q.p > R(0))) ub = mean;
-    constexpr int side = 2 * D + (S < 0 ? 1 : 0);
+// ------------------------------------------------------------------ faces in a team
+// NS faces of direction D (S0 = 0 the upper first, 1 the lower) from the zone's modes s in the frame fr: face_states
+// per side, every facial flux and the check of the barycentre states in one exchange, then each variable's share of
+// the face data to S3.  `store` is false for the lanes past the grid's end, which only take part in the exchanges.
+template <int ORDER, int D, int S0, int NS, class T>
+ADER_DEV void store_sides(const T& t, const StepArgs& a, long long z, bool store, const typename T::V& mean,
+                               const FrameOf<ORDER, T::NL, typename T::R>& fr,
+                               const Vec<T::NL, typename FrameOf<ORDER, T::NL, typename T::R>::S>* s) {
+    using R = typename T::R;
+    using V = typename T::V;
+    using Z = ZoneOps<ORDER>;
+    constexpr int NV = T::NV, NL = T::NL, L = ModeCount<ORDER>::L, NQ = side_values(NV);
+    constexpr int NN = NV == 8 ? Z::FACE_NODES : Z::MEAN_NODES;
+    constexpr int T1 = D == 0 ? 1 : 0, T2 = D == 2 ? 1 : 2;
+    using VS = Vec<NL, typename FrameOf<ORDER, NL, R>::S>;
+    V ub[NS], avg[NS], u[NS * NN], es[NV == 8 ? 4 * NS : 1];
+#pragma unroll
+    for (int side = 0; side < NS; ++side) {
+        VS p[L + 1], b, av, n[Z::FACE_NODES + 1];
+        if (S0 + side == 0) to_face_frame<ORDER, D, +1>(s, p);
+        else to_face_frame<ORDER, D, -1>(s, p);
+        Z::template face_states<NV == 8>(p, b, av, n);
+        ub[side] = fr.leave(b);
+        avg[side] = fr.leave(av);
+#pragma unroll
+        for (int k = 0; k < NN; ++k) u[side * NN + k] = fr.leave(n[NV == 8 ? k + 1 : Z::mean_node(k)]);
+        if constexpr (NV == 8) {
+            VS e[4];
+            Z::edge_states(p, b, av, e);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) es[side * 4 + k] = fr.leave(e[k]);
+        }
+    }
+    V f[NS * NN];
+    bool ok[NS];
+    t.template face_fluxes<D, NS * NN, NS>(u, ub, f, ok);
     R* S3 = (R*)a.S3;
     const long long N = a.grid.n;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        S3[(side * NQ + v) * N + z] = ub[v];
-        S3[(side * NQ + NV + v) * N + z] = avg[v];
-        S3[(side * NQ + 2 * NV + v) * N + z] = Fa[v];
+    for (int side = 0; side < NS; ++side) {
+        // the sums over the nodes in the state scalar too (up to 110 times a flux: 8 bits of headroom)
+        using FF = typename FrameAt<2, NL, R>::T;
+        FF ff;
+        Vec<NL, typename FF::S> F[Z::FACE_NODES + 1];
+#pragma unroll
+        for (int k = 0; k < NN; ++k) ff.include(f[side * NN + k]);
+        ff.close();
+#pragma unroll
+        for (int k = 0; k < NN; ++k) F[NV == 8 ? k + 1 : Z::mean_node(k)] = ff.enter(f[side * NN + k]);
+        const V Fa = ff.leave(Z::face_mean(F));
+        R* out = S3 + (long long)((2 * D + S0 + side) * NQ) * N + z;
+#pragma unroll
+        for (int i = 0; i < NL; ++i) {
+            const int v = t.var(i);
+            if (store) {
+                // the zone average replaces a barycentre state that is not physical, for the wave speeds
+                out[v * N] = ok[side] ? ub[side][i] : mean[i];
+                out[(NV + v) * N] = avg[side][i];
+                out[(2 * NV + v) * N] = Fa[i];
+            }
+            if constexpr (NV == 8) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (v != 5 + (e == 0 ? T1 : T2)) continue;
+                    Vec<NL, typename FF::S> plus, minus;
+                    Z::edge_fluxes(F, e, plus, minus);
+                    if (store) {
+                        out[(3 * NV + 4 * e) * N] = es[side * 4 + 2 * e][i];
+                        out[(3 * NV + 4 * e + 1) * N] = ff.leave(plus)[i];
+                        out[(3 * NV + 4 * e + 2) * N] = es[side * 4 + 2 * e + 1][i];
+                        out[(3 * NV + 4 * e + 3) * N] = ff.leave(minus)[i];
+                    }
+                }
+                if (store && a.solver == SOLVER_LINEARIZED) {   // the linearized edge fluxes need every component
+                    R* X = S3 + (long long)6 * NQ * N + (long long)((2 * D + S0 + side) * EDGE_STATE_VALUES) * N + z;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) X[(e * 8 + v) * N] = es[side * 4 + e][i];
+                }
+            }
+        }
     }
 }
 
-template <int ORDER, int D, int S, int NV, class R>
-ADER_DEV void store_face(const StepArgs& a, long long z, const Vec<NV, R>* m, R gm1) {
-    constexpr int L = ModeCount<ORDER>::L;
-    constexpr int NQ = side_values(NV);
-    Vec<NV, R> p[L + 1];
-    to_face_frame<ORDER, D, S>(m, p);
-    Vec<NV, R> ub, avg, Fa;
-    R eu[4], ef[4];
-    ZoneOps<ORDER>::template face_mhd<D>(p, gm1, ub, avg, Fa, eu, ef);
-    write_side<D, S>(a, z, m[1], ub, avg, Fa, gm1);
-    if constexpr (NV == 8) {
-        constexpr int side = 2 * D + (S < 0 ? 1 : 0);
-        R* S3 = (R*)a.S3;
-        const long long N = a.grid.n;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            S3[(side * NQ + 3 * NV + 2 * e) * N + z] = eu[e];
-            S3[(side * NQ + 3 * NV + 2 * e + 1) * N + z] = ef[e];
-        }
-        if (a.solver == SOLVER_LINEARIZED) {      // the linearized edge fluxes need every component
-            Vec<8, R> es[4];
-            ZoneOps<ORDER>::template edge_states<D>(p, ub, avg, es);
-            R* X = S3 + (long long)6 * NQ * N;
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-#pragma unroll
-                for (int v = 0; v < 8; ++v) X[(side * EDGE_STATE_VALUES + e * 8 + v) * N + z] = es[e][v];
-        }
+// both faces: in one exchange of a team, one after the other in a thread of its own (fewer live values)
+template <int ORDER, int D, class T>
+ADER_DEV void store_faces_team(const T& t, const StepArgs& a, long long z, bool store, const typename T::V& mean,
+                               const FrameOf<ORDER, T::NL, typename T::R>& fr,
+                               const Vec<T::NL, typename FrameOf<ORDER, T::NL, typename T::R>::S>* s) {
+    if constexpr (T::NL == 1) {
+        store_sides<ORDER, D, 0, 2>(t, a, z, store, mean, fr, s);
+    } else {
+        store_sides<ORDER, D, 0, 1>(t, a, z, store, mean, fr, s);
+        store_sides<ORDER, D, 1, 1>(t, a, z, store, mean, fr, s);
     }
 }
 
-// ------------------------------------------------------------------ Euler faces from zone-framed states
 // the zone's modes in the state scalar of its frame (fixed.cuh)
 template <int ORDER, int NV, class R>
 ADER_DEV void enter_frame(const Vec<NV, R>* m, FrameOf<ORDER, NV, R>& fr,
@@ -112,20 +162,38 @@ ADER_DEV void enter_frame(const Vec<NV, R>* m, FrameOf<ORDER, NV, R>& fr,
     for (int k = 1; k <= L; ++k) s[k] = fr.enter(m[k]);
 }
 
-// the two faces of direction D (index 0 upper, 1 lower): the paired form where the order has one
+// ------------------------------------------------------------------ Euler faces of orders 2 and 3, one thread per zone
+// one face side: the barycentre state (replaced by the zone average for the wave speeds when it is not physical),
+// <u> and <F>
+template <int D, int S, int NV, class R>
+ADER_DEV void write_side(const StepArgs& a, long long z, const Vec<NV, R>& mean, Vec<NV, R> ub, const Vec<NV, R>& avg,
+                         const Vec<NV, R>& Fa, R gm1) {
+    constexpr int NQ = side_values(NV);
+    if (!physical_state(ub, gm1)) ub = mean;
+    constexpr int side = 2 * D + (S < 0 ? 1 : 0);
+    R* S3 = (R*)a.S3;
+    const long long N = a.grid.n;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        S3[(side * NQ + v) * N + z] = ub[v];
+        S3[(side * NQ + NV + v) * N + z] = avg[v];
+        S3[(side * NQ + 2 * NV + v) * N + z] = Fa[v];
+    }
+}
+
+template <int D, class R>
+ADER_DEV void both_faces_o2(const FrameOf<2, 5, R>& fr, const Vec<5, typename FrameOf<2, 5, R>::S>* s, R gm1,
+                            Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa);
+template <int D, class R>
+ADER_DEV void both_faces_o3(const FrameOf<3, 5, R>& fr, const Vec<5, typename FrameOf<3, 5, R>::S>* s, R gm1,
+                            Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa);
+
+// the two faces of direction D (index 0 upper, 1 lower)
 template <int ORDER, int D, class R>
 ADER_DEV void both_faces(const FrameOf<ORDER, 5, R>& fr, const Vec<5, typename FrameOf<ORDER, 5, R>::S>* s, R gm1,
                          Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
-    constexpr int L = ModeCount<ORDER>::L;
-    Vec<5, typename FrameOf<ORDER, 5, R>::S> p[L + 1];
-    to_face_frame<ORDER, D, +1>(s, p);
-    if constexpr (ZoneOps<ORDER>::HAS_FACE_PAIR) {
-        ZoneOps<ORDER>::template face_pair<D>(fr, p, gm1, ub, avg, Fa);
-    } else {
-        ZoneOps<ORDER>::template face<D>(fr, p, gm1, ub[0], avg[0], Fa[0]);
-        to_face_frame<ORDER, D, -1>(s, p);
-        ZoneOps<ORDER>::template face<D>(fr, p, gm1, ub[1], avg[1], Fa[1]);
-    }
+    if constexpr (ORDER == 2) both_faces_o2<D, R>(fr, s, gm1, ub, avg, Fa);
+    else both_faces_o3<D, R>(fr, s, gm1, ub, avg, Fa);
 }
 
 template <int ORDER, int D, class R>
@@ -160,88 +228,134 @@ ADER_DEV void record_iterations(unsigned long long* stats, const PredCtl& ctl) {
 // The ADER-CG predictor of zone z (Sec. II.2): the spatial modes, the learned or zero initial guess of
 // the evolutionary modes, the iteration, and what the step keeps besides the face data (dt S-bar with a
 // source, the whole space-time polynomial for dense output).  m[1..L] holds the space-time modes after.
-// SRC: the context carries a non-stiff source (orders with ZoneOps::HAS_SOURCE); the predictor then also
-// writes dt S-bar of Eq. 6 for the update (a.Sb).
-// dt_in: the step size (the caller reads a.dt_dev, once per thread where it can)
-template <int ORDER, int FORM, int NV, class R, bool SRC = false>
-ADER_DEV void zone_predict(const StepArgs& a, const double* __restrict__ U, long long z, Vec<NV, R>* m, R dt) {
-    constexpr int LS = ModeCount<ORDER>::LS, L = ModeCount<ORDER>::L;
-    load_modes<ORDER>(a, U, z, m);
+// SRC: the context carries a non-stiff source; the predictor then also writes dt S-bar of Eq. 6 for the update
+// (a.Sb).  `store` is false for a team's lanes past the grid's end.
+template <int ORDER, int FORM, bool SRC, class T>
+ADER_DEV void zone_predict(const T& t, const StepArgs& a, const double* __restrict__ U, long long z, bool store,
+                           typename T::V* m, typename T::R dt) {
+    using R = typename T::R;
+    using V = typename T::V;
+    constexpr int LS = ModeCount<ORDER>::LS, L = ModeCount<ORDER>::L, NV = T::NV, NL = T::NL;
+    load_modes<ORDER>(t, a, U, z, m);
 #pragma unroll
-    for (int k = LS + 1; k <= L; ++k) m[k] = vzero<NV, R>();
-    const R gm1 = arg_gm1<R>(a);
-    const R cx = dt * arg_idx<R>(a, 0), cy = dt * arg_idx<R>(a, 1), cz = dt * arg_idx<R>(a, 2);
+    for (int k = LS + 1; k <= L; ++k) m[k] = vzero<NL, R>();
     if (a.n_iter > 0) {      // n_iter = 0: spatial polynomial only (SSP-RK face rule)
         if constexpr (ORDER == 3) {
             if (a.G && (!a.Gact || a.Gact[z])) {          // learned initial guess of the evolutionary modes
 #pragma unroll
                 for (int j = 0; j < 5; ++j)
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) m[11 + j][v] = R(a.G[(long long)(j * NV + v) * a.grid.n + z]);
+                    for (int i = 0; i < NL; ++i) m[11 + j][i] = R(a.G[(long long)(j * NV + t.var(i)) * a.grid.n + z]);
             }
         }
         PredCtl ctl{a.n_iter, a.tol, a.max_iter, 0, false};
+        Src<R> src;
+        V sdt;
         if constexpr (SRC) {
-            Src<R> src;
             src.kind = a.src_kind;
 #pragma unroll
             for (int i = 0; i < 3; ++i) src.a[i] = dt * bulk_arg<R>(a.src_par[i]);
-            Vec<NV, R> sdt;
-            if (FORM == FORM_MODAL)
-                ZoneOps<ORDER>::predict_modal_src(m, gm1, cx, cy, cz, ctl, src, sdt);
-            else
-                ZoneOps<ORDER>::predict_nodal_src(m, gm1, cx, cy, cz, ctl, src, sdt);
+        }
+        if constexpr (FORM == FORM_MODAL) ZoneOps<ORDER>::template predict_modal<SRC>(t, m, ctl, &src, &sdt);
+        else ZoneOps<ORDER>::template predict_nodal<SRC>(t, m, ctl, &src, &sdt);
+        if constexpr (SRC) {
             R* Sb = (R*)a.Sb;
 #pragma unroll
-            for (int v = 0; v < 5; ++v) Sb[v * a.grid.n + z] = sdt[v];
-        } else if (FORM == FORM_MODAL) {
-            ZoneOps<ORDER>::predict_modal(m, gm1, cx, cy, cz, ctl);
-        } else {
-            ZoneOps<ORDER>::predict_nodal(m, gm1, cx, cy, cz, ctl);
+            for (int i = 0; i < NL; ++i)
+                if (store && t.var(i) < 5) Sb[t.var(i) * a.grid.n + z] = sdt[i];
         }
-        if (a.stats && positive_arg(a.tol)) record_iterations(a.stats, ctl);
-        if (ctl.capped) raise_flag(a.flag, FLAG_NOT_CONVERGED);
+        if (store && t.lead()) {
+            if (a.stats && positive_arg(a.tol)) record_iterations(a.stats, ctl);
+            if (ctl.capped) raise_flag(a.flag, FLAG_NOT_CONVERGED);
+        }
     }
-    if (a.modes_out) {      // dense output (Sec. VII): keep the whole space-time polynomial of the step
+    if (a.modes_out && store) {      // dense output (Sec. VII): keep the whole space-time polynomial of the step
         R* o = (R*)a.modes_out;
 #pragma unroll
         for (int k = 1; k <= L; ++k)
 #pragma unroll
-            for (int v = 0; v < NV; ++v) o[(long long)((k - 1) * NV + v) * a.grid.n + z] = m[k][v];
+            for (int i = 0; i < NL; ++i) o[(long long)((k - 1) * NV + t.var(i)) * a.grid.n + z] = m[k][i];
     }
 }
 
+template <class T>
+ADER_DEV void team_scales(T& t, const StepArgs& a, typename T::R dt) {
+    using R = typename T::R;
+    t.gm1 = arg_gm1<R>(a);
+    t.cx = dt * arg_idx<R>(a, 0);
+    t.cy = dt * arg_idx<R>(a, 1);
+    t.cz = dt * arg_idx<R>(a, 2);
+}
+
+// predictor and face data of one zone by one team
+template <int ORDER, int FORM, bool SRC, class T>
+ADER_DEV void team_predict_faces(T& t, const StepArgs& a, const double* __restrict__ U, long long z, bool store) {
+    using R = typename T::R;
+    constexpr int L = ModeCount<ORDER>::L;
+    const R dt = bulk_arg<R>(a.dt_dev ? *a.dt_dev : a.dt);
+    team_scales(t, a, dt);
+    typename T::V m[L + 1];
+    zone_predict<ORDER, FORM, SRC>(t, a, U, z, store, m, dt);
+    FrameOf<ORDER, T::NL, R> fr;
+    Vec<T::NL, typename FrameOf<ORDER, T::NL, R>::S> s[L + 1];
+    enter_frame<ORDER>(m, fr, s);
+    if constexpr (T::NL == 5 && ORDER <= 3) {
+        store_faces<ORDER, 0, R>(a, z, m[1], fr, s, t.gm1);
+        store_faces<ORDER, 1, R>(a, z, m[1], fr, s, t.gm1);
+        store_faces<ORDER, 2, R>(a, z, m[1], fr, s, t.gm1);
+    } else {
+        store_faces_team<ORDER, 0>(t, a, z, store, m[1], fr, s);
+        store_faces_team<ORDER, 1>(t, a, z, store, m[1], fr, s);
+        store_faces_team<ORDER, 2>(t, a, z, store, m[1], fr, s);
+    }
+}
+
+// one thread per zone
 template <int ORDER, int FORM, int NV, class R, bool SRC = false>
 ADER_DEV void zone_predict_faces(const StepArgs& a, const double* __restrict__ U, long long z) {
-    Vec<NV, R> m[ModeCount<ORDER>::L + 1];
-    zone_predict<ORDER, FORM, NV, R, SRC>(a, U, z, m, bulk_arg<R>(a.dt_dev ? *a.dt_dev : a.dt));
-    const R gm1 = arg_gm1<R>(a);
-    if constexpr (NV == 5) {
-        FrameOf<ORDER, 5, R> fr;
-        Vec<5, typename FrameOf<ORDER, 5, R>::S> s[ModeCount<ORDER>::L + 1];
-        enter_frame<ORDER>(m, fr, s);
-        store_faces<ORDER, 0>(a, z, m[1], fr, s, gm1);
-        store_faces<ORDER, 1>(a, z, m[1], fr, s, gm1);
-        store_faces<ORDER, 2>(a, z, m[1], fr, s, gm1);
-    } else {
-        store_face<ORDER, 0, +1>(a, z, m, gm1);
-        store_face<ORDER, 0, -1>(a, z, m, gm1);
-        store_face<ORDER, 1, +1>(a, z, m, gm1);
-        store_face<ORDER, 1, -1>(a, z, m, gm1);
-        store_face<ORDER, 2, +1>(a, z, m, gm1);
-        store_face<ORDER, 2, -1>(a, z, m, gm1);
-    }
+    SerialTeam<NV, R> t;
+    team_predict_faces<ORDER, FORM, SRC>(t, a, U, z, true);
 }
 
-// FP32 bulk asks for three 128-thread blocks per SM at orders 2-3 (at most 168 registers, a few hundred
-// bytes of spills to L1): the extra warps hide more latency than the spills cost (about 12% per 256^3
-// step).  At order 4, and for MHD at order 3, the predictor spills kilobytes per zone at 168 registers;
-// there it takes two blocks per SM and 255 registers (a 128^3 MHD step at order 3: 3.5 -> 2.4 ms).
+// Where a team of warps computes a zone: order 4 and MHD (see team.cuh), except
+//   * FP32 MHD at order 2, whose forty modes fit one thread (56^3 zones: 176 us a step against the team's 199);
+//   * the FP32 nodal form of order 4 (Euler): behind strong jumps its predicted density comes near zero at a node,
+//     which amplifies the rounding of the fluxes by up to 10^4, and the team sums them with other roundings.
+template <int ORDER, int FORM, int NV, class R>
+constexpr bool uses_team() {
+    if (sizeof(R) == 4 && ((ORDER == 2 && NV == 8) || (ORDER == 4 && NV == 5 && FORM == FORM_NODAL))) return false;
+    return ORDER == 4 || NV == 8;
+}
+
+// FP32 bulk asks for three 128-thread blocks per SM (at most 168 registers): the extra warps hide more latency than
+// what spills costs (about 12% per 256^3 step at orders 2-3); order 4 spills kilobytes per zone there and takes two
+// blocks and 255 registers.
 template <int ORDER, int FORM, int NV, class R, bool SRC = false>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? (ORDER == 4 || (ORDER == 3 && NV == 8) ? 2 : 3) : 1)
-    k_predict_faces(StepArgs a, const double* __restrict__ U) {
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? (ORDER == 4 ? 2 : 3) : 1) k_predict_faces(StepArgs a, const double* __restrict__ U) {
     const long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (z < a.grid.n) zone_predict_faces<ORDER, FORM, NV, R, SRC>(a, U, z);
+}
+
+// The team kernel: a block of NV warps takes 32 zones, a warp one variable of each.
+template <int ORDER, int NV, class R>
+constexpr int team_smem() { return team_values<ORDER, NV>() * 32 * (int)sizeof(R); }
+template <int ORDER, int NV, class R>
+constexpr int team_blocks() { return sizeof(R) == 4 ? (NV == 8 ? 2 : 3) : (NV == 8 && ORDER == 4 ? 1 : 2); }
+
+template <int ORDER, int FORM, int NV, bool SRC, class R>
+__device__ __forceinline__ void team_zone(const StepArgs& a, const double* __restrict__ U, long long z, R* sh) {
+    WarpTeam<NV, R> t;
+    t.sh = sh + (threadIdx.x & 31);
+    t.v = threadIdx.x >> 5;
+    const bool store = z < a.grid.n;
+    team_predict_faces<ORDER, FORM, SRC>(t, a, U, store ? z : a.grid.n - 1, store);
+}
+
+template <int ORDER, int FORM, int NV, class R, bool SRC>
+__global__ void __launch_bounds__(NV * 32, team_blocks<ORDER, NV, R>())
+    k_team_predict_faces(StepArgs a, const double* __restrict__ U) {
+    extern __shared__ __align__(16) unsigned char team_raw[];
+    team_zone<ORDER, FORM, NV, SRC, R>(a, U, (long long)blockIdx.x * 32 + (threadIdx.x & 31), (R*)team_raw);
 }
 
 template <int NV, class R>
@@ -528,8 +642,7 @@ ADER_DEV R* pt_slot(R* sh, int slot, int tid) { return sh + slot * PT_NQ * PT_TH
 // write_side does), <u>, <F>
 template <class R>
 ADER_DEV void pt_side(R* dst, const Vec<5, R>& mean, Vec<5, R> ub, const Vec<5, R>& avg, const Vec<5, R>& Fa, R gm1) {
-    const Prim<5, R> q = primitives(ub, gm1);
-    if (!(ub[0] > R(0)) || !(q.p > R(0))) ub = mean;
+    if (!physical_state(ub, gm1)) ub = mean;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
         dst[v * PT_THREADS] = ub[v];
@@ -640,7 +753,9 @@ __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 3 : 1)
         const int zp_slot = (k & 1) ? 6 : 4;          // this plane's z+ sides; the previous plane's in the other
         if (valid) {
             Vec<5, R> m[ModeCount<ORDER>::L + 1];
-            zone_predict<ORDER, FORM, 5, R, SRC>(a, U, z, m, dt);
+            SerialTeam<5, R> team;
+            team_scales(team, a, dt);
+            zone_predict<ORDER, FORM, SRC>(team, a, U, z, true, m, dt);
             FrameOf<ORDER, 5, R> fr;
             Vec<5, typename FrameOf<ORDER, 5, R>::S> s[ModeCount<ORDER>::L + 1];
             enter_frame<ORDER>(m, fr, s);
@@ -952,24 +1067,25 @@ void launch_pf_variant(const StepArgs& a, const double* U, cudaStream_t st) {
             return;
         }
     }
-    const int T = 128;
-    const unsigned blocks = (unsigned)((a.grid.n + T - 1) / T);
-    k_predict_faces<ORDER, FORM, NV, R, SRC><<<blocks, T, 0, st>>>(a, U);
+    if constexpr (uses_team<ORDER, FORM, NV, R>()) {
+        auto kern = k_team_predict_faces<ORDER, FORM, NV, R, SRC>;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, team_smem<ORDER, NV, R>());
+        kern<<<(unsigned)((a.grid.n + 31) / 32), NV * 32, team_smem<ORDER, NV, R>(), st>>>(a, U);
+    } else {
+        const int T = 128;
+        const unsigned blocks = (unsigned)((a.grid.n + T - 1) / T);
+        k_predict_faces<ORDER, FORM, NV, R, SRC><<<blocks, T, 0, st>>>(a, U);
+    }
 }
 
 template <int ORDER, int NV, class R>
 int launch_predict_faces_nv(const StepArgs& a, const double* U, cudaStream_t st) {
-    if constexpr (ZoneOps<ORDER>::HAS_SOURCE) {
-        if (a.src_kind != SOURCE_NONE && a.Sb && a.n_iter > 0) {
-            if (a.form == FORM_NODAL) {
-                launch_pf_variant<ORDER, FORM_NODAL, NV, R, true>(a, U, st);
-                return (NV == 5 && ORDER <= 3 && a.tiled) ? 2 : 1;
-            }
-            if constexpr (ZoneOps<ORDER>::HAS_SOURCE_MODAL) {
-                launch_pf_variant<ORDER, FORM_MODAL, NV, R, true>(a, U, st);
-                return (NV == 5 && ORDER <= 3 && a.tiled) ? 2 : 1;
-            }
-        }
+    if (a.src_kind != SOURCE_NONE && a.Sb && a.n_iter > 0) {
+        if (a.form == FORM_NODAL)
+            launch_pf_variant<ORDER, FORM_NODAL, NV, R, true>(a, U, st);
+        else
+            launch_pf_variant<ORDER, FORM_MODAL, NV, R, true>(a, U, st);
+        return (NV == 5 && ORDER <= 3 && a.tiled) ? 2 : 1;
     }
     if (a.form == FORM_MODAL)
         launch_pf_variant<ORDER, FORM_MODAL, NV, R, false>(a, U, st);

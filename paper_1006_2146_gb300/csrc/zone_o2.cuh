@@ -4,119 +4,120 @@
 #include "common.cuh"
 #include "fixed.cuh"
 #include "modes.cuh"
+#include "team.cuh"
 
 namespace ader {
 namespace o2 {
 
-template <int NV, class R>
-ADER_DEV void finish_o2(Vec<NV, R>* m, const Vec<NV, R>& n5, PredCtl& ctl) {
-    const bool conv = positive_arg(ctl.tol);
-    const int cap = conv ? ctl.max_iter : ctl.n_iter;
-    const R ref = max_abs(m[1]) + R(sizeof(R) == 8 ? 1e-300 : 1e-30);   // never zero in R
-    ctl.iters = 0;
-    ctl.capped = conv;
-    for (int it = 0; it < cap; ++it) {
-        const R change = max_abs_diff(n5, m[5]);
-        m[5] = n5;
-        ++ctl.iters;
-        if (conv && change < R(ctl.tol) * ref) {
-            ctl.capped = false;
-            break;
-        }
-    }
-}
-
-
-// Eqs. 31-33 and 30 (one iteration, no sources)
-// The update uses only tau = 0 fluxes, so one step reaches the fixed point
+// The update without sources uses only tau = 0 fluxes, so one step reaches the fixed point n5
 // (in converged mode a second step confirms it).
-template <int NV, class R>
-ADER_DEV void predict_modal(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& ctl) {
-    const Vec<NV, R> u1 = m[1] + 0.5 * m[2], u2 = m[1] - 0.5 * m[2];
-    const Vec<NV, R> u3 = m[1] + 0.5 * m[3], u4 = m[1] - 0.5 * m[3];
-    const Vec<NV, R> u5 = m[1] + 0.5 * m[4], u6 = m[1] - 0.5 * m[4];
-    const Vec<NV, R> F2 = scale(cx, flux<0>(u1, gm1) - flux<0>(u2, gm1));
-    const Vec<NV, R> G3 = scale(cy, flux<1>(u3, gm1) - flux<1>(u4, gm1));
-    const Vec<NV, R> H4 = scale(cz, flux<2>(u5, gm1) - flux<2>(u6, gm1));
-    const Vec<NV, R> n5 = -(F2 + G3 + H4);
-    finish_o2(m, n5, ctl);
-}
-
-// Eqs. A.5, A.4 (h term at node 4, the zeta node of Eq. A.1) and A.6
-template <int NV, class R>
-ADER_DEV void predict_nodal(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& ctl) {
-    const Vec<NV, R> u1 = m[1];
-    const Vec<NV, R> u2 = m[1] + 0.5 * m[2], u3 = m[1] + 0.5 * m[3], u4 = m[1] + 0.5 * m[4];
-    const Prim<NV, R> p1 = primitives(u1, gm1);
-    const Vec<NV, R> u5 = u1 - 2.0 * (scale(cx, flux<0>(u2, gm1) - flux_from<0>(u1, p1)) +
-                                scale(cy, flux<1>(u3, gm1) - flux_from<1>(u1, p1)) +
-                                scale(cz, flux<2>(u4, gm1) - flux_from<2>(u1, p1)));
-    finish_o2(m, u5 - u1, ctl);
-}
-
-// ---- with a non-stiff source (s = dt S at the nodes of the current iterate)
-// The update of u5 now depends on u5 through the source at the tau = 1 node,
-// so each iteration recomputes it; sdt receives dt S-bar from the final
-// iterate.  `next(m5)` gives the new u5 for the current one.
-template <int NV, class R, class Next>
-ADER_DEV void iterate_o2(Vec<NV, R>* m, PredCtl& ctl, Next next) {
+template <class T>
+ADER_DEV void finish_o2(const T& t, typename T::V* m, const typename T::V& n5, PredCtl& ctl) {
     const bool conv = positive_arg(ctl.tol);
-    const int cap = conv ? ctl.max_iter : ctl.n_iter;
-    const R ref = max_abs(m[1]) + R(sizeof(R) == 8 ? 1e-300 : 1e-30);   // never zero in R
     ctl.iters = 0;
     ctl.capped = conv;
+    if (!conv) {
+        if (ctl.n_iter > 0) m[5] = n5;
+        ctl.iters = ctl.n_iter;
+        return;
+    }
+    using R = typename T::R;
+    const R ref = t.zone_max(max_abs(m[1])) + R(sizeof(R) == 8 ? 1e-300 : 1e-30);   // never zero in R
+    const R change = t.zone_max(max_abs_diff(n5, m[5]));
+    if (ctl.max_iter > 0) m[5] = n5;
+    if (change < R(ctl.tol) * ref || R(0) < R(ctl.tol) * ref) {
+        ctl.iters = change < R(ctl.tol) * ref ? 1 : 2;          // the second step changes nothing
+        ctl.capped = ctl.iters > ctl.max_iter;
+    }
+    if (ctl.capped) ctl.iters = ctl.max_iter;
+}
+
+// With a source the update of u5 depends on u5 through the source at the tau = 1 node, so each iteration recomputes
+// it: `next(m5)` gives the new u5 for the current one.
+template <class T, class Next>
+ADER_DEV void iterate_o2(const T& t, typename T::V* m, PredCtl& ctl, Next next) {
+    using R = typename T::R;
+    using V = typename T::V;
+    const bool conv = positive_arg(ctl.tol);
+    const int cap = conv ? ctl.max_iter : ctl.n_iter;
+    R ref = R(1);
+    if (conv) ref = t.zone_max(max_abs(m[1])) + R(sizeof(R) == 8 ? 1e-300 : 1e-30);   // never zero in R
+    ctl.iters = 0;
+    bool done = false;                  // this zone has converged (others of the team may go on)
     for (int it = 0; it < cap; ++it) {
-        const Vec<NV, R> n5 = next(m[5]);
-        const R change = max_abs_diff(n5, m[5]);
-        m[5] = n5;
-        ++ctl.iters;
-        if (conv && change < R(ctl.tol) * ref) {
-            ctl.capped = false;
-            break;
+        const V n5 = next(m[5]);
+        R change = R(0);
+        if (!t.waits(done)) {
+            change = max_abs_diff(n5, m[5]);
+            m[5] = n5;
+            ++ctl.iters;
         }
+        if (conv) {
+            change = t.zone_max(change);
+            done = done || change < R(ctl.tol) * ref;
+            if (!t.any(!done)) break;
+        }
+    }
+    ctl.capped = conv && !done;
+}
+
+// Eqs. 31-33 and 30; with a source Eqs. 34-35: s at the seven nodes of Eq. 31 (node 7 = u1 + u5 at tau = 1), sdt
+// receives dt S-bar from the final iterate
+template <class T, bool SRC = false>
+ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Src<typename T::R>* src = nullptr,
+                            typename T::V* sdt = nullptr) {
+    using V = typename T::V;
+    // x+, x-, y+, y-, z+, z-, the order of T::fluxes
+    const V u[6] = {m[1] + 0.5 * m[2], m[1] - 0.5 * m[2], m[1] + 0.5 * m[3],
+                    m[1] - 0.5 * m[3], m[1] + 0.5 * m[4], m[1] - 0.5 * m[4]};
+    V f[2], g[2], h[2];
+    t.template fluxes<0, 2, false>(u, f, g, h);
+    const V div = scale(t.cx, f[0] - f[1]) + scale(t.cy, g[0] - g[1]) + scale(t.cz, h[0] - h[1]);
+    if constexpr (SRC) {
+        V s[6], s7;
+        t.template sources<6>(u, *src, s);
+        const V s1 = (s[0] + s[1] + s[2] + s[3] + s[4] + s[5]) / 6.0;                  // Eq. 34
+        const V base = s1 - div;
+        iterate_o2(t, m, ctl, [&](const V& m5) {
+            const V u7 = m[1] + m5;
+            V s5;
+            t.template sources<1>(&u7, *src, &s5);
+            return base + (2.0 / 3.0) * (s5 - s1);                                     // Eqs. 34 and 30
+        });
+        const V u7 = m[1] + m[5];
+        t.template sources<1>(&u7, *src, &s7);
+        *sdt = s1 + 0.5 * (s7 - s1);                                                   // Eq. 35 (times dt)
+    } else {
+        finish_o2(t, m, -div, ctl);
     }
 }
 
-// Eqs. 31-34, 30 and 35: s at the seven nodes of Eq. 31 (node 7 = u1 + u5 at tau = 1)
-constexpr bool HAS_SOURCE = true;
-constexpr bool HAS_SOURCE_MODAL = true;
-
-template <int NV, class R>
-ADER_DEV void predict_modal_src(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& ctl, const Src<R>& src,
-                                Vec<NV, R>& sdt) {
-    const Vec<NV, R> u1 = m[1] + 0.5 * m[2], u2 = m[1] - 0.5 * m[2];
-    const Vec<NV, R> u3 = m[1] + 0.5 * m[3], u4 = m[1] - 0.5 * m[3];
-    const Vec<NV, R> u5 = m[1] + 0.5 * m[4], u6 = m[1] - 0.5 * m[4];
-    const Vec<NV, R> F2 = scale(cx, flux<0>(u1, gm1) - flux<0>(u2, gm1));
-    const Vec<NV, R> G3 = scale(cy, flux<1>(u3, gm1) - flux<1>(u4, gm1));
-    const Vec<NV, R> H4 = scale(cz, flux<2>(u5, gm1) - flux<2>(u6, gm1));
-    const Vec<NV, R> s1 = (source_at(u1, src) + source_at(u2, src) + source_at(u3, src) + source_at(u4, src) +
-                           source_at(u5, src) + source_at(u6, src)) / 6.0;          // Eq. 34
-    const Vec<NV, R> base = s1 - (F2 + G3 + H4);
-    iterate_o2(m, ctl, [&](const Vec<NV, R>& m5) {
-        const Vec<NV, R> s5 = source_at(m[1] + m5, src) - s1;                      // Eq. 34
-        return base + (2.0 / 3.0) * s5;                                             // Eq. 30
-    });
-    sdt = s1 + 0.5 * (source_at(m[1] + m[5], src) - s1);                            // Eq. 35 (times dt)
-}
-
-// Eqs. A.5, A.4 and A.6-A.7: s at node 1 (tau = 0) and node 5 (tau = 1)
-template <int NV, class R>
-ADER_DEV void predict_nodal_src(Vec<NV, R>* m, R gm1, R cx, R cy, R cz, PredCtl& ctl, const Src<R>& src,
-                                Vec<NV, R>& sdt) {
-    const Vec<NV, R> u1 = m[1];
-    const Vec<NV, R> u2 = m[1] + 0.5 * m[2], u3 = m[1] + 0.5 * m[3], u4 = m[1] + 0.5 * m[4];
-    const Prim<NV, R> p1 = primitives(u1, gm1);
-    const Vec<NV, R> s1 = source_at(u1, src);
-    const Vec<NV, R> base = u1 - 2.0 * (scale(cx, flux<0>(u2, gm1) - flux_from<0>(u1, p1)) +
-                                        scale(cy, flux<1>(u3, gm1) - flux_from<1>(u1, p1)) +
-                                        scale(cz, flux<2>(u4, gm1) - flux_from<2>(u1, p1))) +
-                            s1 / 3.0;
-    iterate_o2(m, ctl, [&](const Vec<NV, R>& m5) {
-        const Vec<NV, R> u5 = base + (2.0 / 3.0) * source_at(u1 + m5, src);         // Eq. A.4
-        return u5 - u1;                                                              // Eq. A.6
-    });
-    sdt = 0.5 * (s1 + source_at(u1 + m[5], src));                                   // Eq. A.7 (times dt)
+// Eqs. A.5, A.4 (h term at node 4, the zeta node of Eq. A.1) and A.6; with a source A.7: s at node 1 (tau = 0) and
+// node 5 (tau = 1)
+template <class T, bool SRC = false>
+ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Src<typename T::R>* src = nullptr,
+                            typename T::V* sdt = nullptr) {
+    using V = typename T::V;
+    using R = typename T::R;
+    const V u1 = m[1];
+    const V u[4] = {u1, m[1] + 0.5 * m[2], m[1] + 0.5 * m[3], m[1] + 0.5 * m[4]};
+    const V d = t.axis_differences(u, R(2));                // 2 sum_d c_d (F_d(u1) - F_d(u_{1+d}))
+    if constexpr (SRC) {
+        V s1, s5;
+        t.template sources<1>(&u1, *src, &s1);
+        const V base = d + s1 / 3.0;
+        iterate_o2(t, m, ctl, [&](const V& m5) {
+            const V u5 = u1 + m5;
+            V s;
+            t.template sources<1>(&u5, *src, &s);
+            return base + (2.0 / 3.0) * s;                                             // Eqs. A.4 and A.6
+        });
+        const V u5 = u1 + m[5];
+        t.template sources<1>(&u5, *src, &s5);
+        *sdt = 0.5 * (s1 + s5);                                                        // Eq. A.7 (times dt)
+    } else {
+        finish_o2(t, m, d, ctl);
+    }
 }
 
 // Eqs. 58-59 and D.3-D.5: composing D.4 with D.5, <F> is the mean of the flux
@@ -136,50 +137,45 @@ ADER_DEV void face(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV
     Fa = sum.mean(avg, gm1, R(0.25));
 }
 
-// MHD face: also the edge averages (Eq. 60 for <u>, Eqs. D.4-D.5 for <F>) of
-// the field component each edge's EMF needs.  eu/ef slots: t1+, t1-, t2+, t2-
-// (t1 < t2 the transverse axes); component 5 + t1 on the t1 edges, 5 + t2 on
-// the t2 edges.
-template <int D, class R>
-ADER_DEV void face_mhd(const Vec<8, R>* p, R gm1, Vec<8, R>& ub, Vec<8, R>& avg, Vec<8, R>& Fa, R* eu, R* ef) {
-    constexpr int T1 = D == 0 ? 1 : 0, T2 = D == 2 ? 1 : 2;
+// MHD: the states of a face and its five nodes (Eqs. 58-59, D.3), and the mean of the flux at the first four.
+template <bool ALL, class V>
+ADER_DEV void face_states(const V* p, V& ub, V& avg, V* t) {
     ub = p[1] + 0.5 * (p[2] + p[5]);
     avg = ub;
-    const Vec<8, R> t[6] = {ub, ub + 0.5 * p[3], ub - 0.5 * p[3], ub + 0.5 * p[4], ub - 0.5 * p[4], ub + 0.5 * p[5]};
-    Vec<8, R> F[6];
-#pragma unroll
-    for (int n = 1; n <= 5; ++n) F[n] = flux<D>(t[n], gm1);
-    Fa = 0.25 * (F[1] + F[2] + F[3] + F[4]);
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        const int c = 5 + (s == 0 ? T1 : T2);
-        const R m2 = F[1][c] - F[2][c], m3 = F[3][c] - F[4][c];
-        const R m4 = R(2) * F[5][c] - R(0.5) * (F[1][c] + F[2][c] + F[3][c] + F[4][c]);
-        const R af = F[5][c] - m4 + R(0.5) * m4;
-        const R half = R(0.5) * (s == 0 ? m2 : m3);
-        ef[2 * s] = af + half;
-        ef[2 * s + 1] = af - half;
-        const R hu = R(0.5) * p[s == 0 ? 3 : 4][c];
-        eu[2 * s] = ub[c] + hu;
-        eu[2 * s + 1] = ub[c] - hu;
-    }
+    t[1] = ub + 0.5 * p[3];
+    t[2] = ub - 0.5 * p[3];
+    t[3] = ub + 0.5 * p[4];
+    t[4] = ub - 0.5 * p[4];
+    if (ALL) t[5] = ub + 0.5 * p[5];
+}
+constexpr int FACE_NODES = 5, MEAN_NODES = 4;
+ADER_DEV constexpr int mean_node(int k) { return k + 1; }
+template <class V>
+ADER_DEV V face_mean(const V* F) {
+    return 0.25 * (F[1] + F[2] + F[3] + F[4]);
 }
 
-// Full edge-averaged states (all eight components; Eq. 60) for the
-// linearized edge fluxes.  Slots as in face_mhd.
-template <int D, class R>
-ADER_DEV void edge_states(const Vec<8, R>* p, const Vec<8, R>& ub, const Vec<8, R>& avg, Vec<8, R>* e) {
+// the edge averages (Eqs. D.4-D.5) of the facial flux f[n] on the edges of the transverse direction
+// s (0: t1, 1: t2), upper and lower
+template <class V>
+ADER_DEV void edge_fluxes(const V* f, int s, V& plus, V& minus) {
+    const V m2 = f[1] - f[2], m3 = f[3] - f[4];
+    const V m4 = 2.0 * f[5] - 0.5 * (f[1] + f[2] + f[3] + f[4]);
+    const V af = f[5] - m4 + 0.5 * m4;
+    const V half = 0.5 * (s == 0 ? m2 : m3);
+    plus = af + half;
+    minus = af - half;
+}
+
+// Edge-averaged states (Eq. 60) on the edges t1+, t1-, t2+, t2-.
+template <class V>
+ADER_DEV void edge_states(const V* p, const V& ub, const V& avg, V* e) {
     (void)avg;
     e[0] = ub + 0.5 * p[3];
     e[1] = ub - 0.5 * p[3];
     e[2] = ub + 0.5 * p[4];
     e[3] = ub - 0.5 * p[4];
 }
-
-// No paired-face form at this order: the faces are evaluated one at a time.
-constexpr bool HAS_FACE_PAIR = false;
-template <int D, int NV, class R, class FR>
-ADER_DEV void face_pair(const FR&, const Vec<NV, typename FR::S>*, R, Vec<NV, R>*, Vec<NV, R>*, Vec<NV, R>*) {}
 
 }  // namespace o2
 }  // namespace ader
