@@ -27,6 +27,9 @@
 namespace ader {
 
 // ---------------------------------------------------------------- kernels (one thread per zone)
+// FP64: blockIdx.y takes the variables apart (one thread per zone and variable), which shortens the chain of FP64
+// operations a thread carries and fills the chip on small grids (16^3 zones: 32 blocks of 128 zones); FP32 holds all
+// variables of a zone in one thread.
 template <int ORDER, class R>
 __global__ void __launch_bounds__(128) k_face_b(Grid g, const double* __restrict__ Bf, R* __restrict__ ZB,
                                                 R* __restrict__ S1) {
@@ -38,7 +41,7 @@ template <int ORDER, int NV, class R, class T>
 __global__ void __launch_bounds__(128) k_weno1d(Grid g, const T* __restrict__ U, const R* __restrict__ ZB,
                                                 R* __restrict__ S1) {
     const long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (z < g.n) zone_weno1d<ORDER, NV>(g, U, ZB, S1, z);
+    if (z < g.n) zone_weno1d<ORDER, NV>(g, U, ZB, S1, z, (int)blockIdx.y, (int)gridDim.y);
 }
 
 // FP32 copy of the state: every value is rounded once per step here instead of
@@ -74,7 +77,7 @@ int launch_to_f32(float* out, const double* U, long long count, cudaStream_t st)
 template <int ORDER, int NV, class R>
 __global__ void __launch_bounds__(128) k_cross1(Grid g, const R* __restrict__ S1, R* __restrict__ S2) {
     const long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (z < g.n) zone_cross1<ORDER, NV>(g, S1, S2, z);
+    if (z < g.n) zone_cross1<ORDER, NV>(g, S1, S2, z, (int)blockIdx.y, (int)gridDim.y);
 }
 
 // Third-order cross moments in FP32 from shared-memory tiles (2.5-D
@@ -182,10 +185,12 @@ static bool launch_cross1_tiled(const Grid& g, const float* S1, float* S2, cudaS
 // of the y slopes (w2, w4: rows j0-1 .. j0+9 and j0-1 .. j0+8); each thread keeps the z terms of its
 // column (w2, w3) in registers and slides them up one plane at a time.  A zone's slope then takes four
 // d and three E from there: about 27 FP64 operations instead of 39.  Same bits as zone_cross1.
-// Requires nx % CT_X == 0 and ny % CT_Y == 0 (other grids use k_cross1).
+// Any grid (tiles64 says which take it).  The next plane's values are loaded a plane ahead: the loads' latency stood
+// between two barriers of every plane.  Bound by the FP64 unit at 81% of its measured rate; three blocks per SM
+// instead of two, in 80 registers, and the loads ahead: 256^3 step 80.5 -> 77.3 ms with k_weno1d_tiled64's.
 template <int NV>
-__global__ void __launch_bounds__(CT_X * CT_Y) k_cross1_tiled64(Grid g, const double* __restrict__ S1,
-                                                                double* __restrict__ S2) {
+__global__ void __launch_bounds__(CT_X * CT_Y, 3) k_cross1_tiled64(Grid g, const double* __restrict__ S1,
+                                                                double* __restrict__ S2, int cz) {
     __shared__ double s2[CT_Y + 4][CT_X];          // w2 with two rows of y halo on each side
     __shared__ double s3[CT_Y][CT_X + 4];          // w3 with two columns of x halo
     __shared__ double s4[CT_Y + 4][CT_X + 4];      // w4 with both
@@ -194,14 +199,19 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_cross1_tiled64(Grid g, const do
     __shared__ double dy2[CT_Y + 3][CT_X], dy4[CT_Y + 3][CT_X];    // d along y at j0 - 1 + r
     __shared__ double ey2[CT_Y + 2][CT_X], ey4[CT_Y + 2][CT_X];    // E along y at j0 - 1 + r
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int tiles_x = g.nx / CT_X;
+    const int tiles_x = (g.nx + CT_X - 1) / CT_X;
     const int i = (int)(blockIdx.x % tiles_x) * CT_X + tx, j = (int)(blockIdx.x / tiles_x) * CT_Y + ty;
-    const int k0 = (int)blockIdx.y * CT_Z, k1 = min(k0 + CT_Z, g.nz);
+    const int k0 = (int)blockIdx.y * cz, k1 = min(k0 + cz, g.nz);
+    const bool inside = i < g.nx && j < g.ny;        // columns past the grid's end only serve as halos
     const long long N = g.n;
     const long long nxy = (long long)g.nx * g.ny;
-    const long long xy = (long long)j * g.nx + i;
-    const long long xy_jm = (long long)wrap(j - 2, g.ny) * g.nx + i, xy_jp = (long long)wrap(j + 2, g.ny) * g.nx + i;
-    const long long xy_im = (long long)j * g.nx + wrap(i - 2, g.nx), xy_ip = (long long)j * g.nx + wrap(i + 2, g.nx);
+    const int iw = wrap(i, g.nx), jw = wrap(j, g.ny);
+    const long long xy = (long long)jw * g.nx + iw;
+    // the halo columns this thread brings: two rows below and above, two columns left and right
+    const bool halo_y = ty < 2 || ty >= CT_Y - 2, halo_x = tx < 2 || tx >= CT_X - 2;
+    const int ry = ty < 2 ? ty : ty + 4, rx = tx < 2 ? tx : tx + 4;
+    const long long xy_y = (long long)wrap(ty < 2 ? j - 2 : j + 2, g.ny) * g.nx + iw;
+    const long long xy_x = (long long)jw * g.nx + wrap(tx < 2 ? i - 2 : i + 2, g.nx);
     auto plane = [&](int kk) -> long long { return (long long)wrap(kk, g.nz) * nxy; };
     // the halo entries of the term arrays: along x, threads tx = 0, 1, 2 of each row add the positions -1,
     // 32, 33 (d) and tx = 0, 1 the positions -1, 32 (E); along y, rows ty = 0, 1, 2 and ty = 0, 1 likewise
@@ -231,6 +241,20 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_cross1_tiled64(Grid g, const do
             ez2[s] = w3_curv(rn_sub(dz2[s + 1], dz2[s]));
             ez3[s] = w3_curv(rn_sub(dz3[s + 1], dz3[s]));
         }
+        // the next plane's values are loaded a plane ahead, behind the first barrier
+        double up2 = 0.0, up3 = 0.0, own4 = w4[k0 * nxy + xy];
+        double hy2 = 0.0, hy4 = 0.0, hx3 = 0.0, hx4 = 0.0;
+        auto halos = [&](long long p) {
+            if (halo_y) {
+                hy2 = w2[p + xy_y];
+                hy4 = w4[p + xy_y];
+            }
+            if (halo_x) {
+                hx3 = w3[p + xy_x];
+                hx4 = w4[p + xy_x];
+            }
+        };
+        halos(k0 * nxy);
         for (int k = k0; k < k1; ++k) {
             if (k > k0) {              // slide the column up one plane
 #pragma unroll
@@ -238,9 +262,8 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_cross1_tiled64(Grid g, const do
                     c2[q] = c2[q + 1];
                     c3[q] = c3[q + 1];
                 }
-                const long long p2 = plane(k + 2) + xy;
-                c2[4] = w2[p2];
-                c3[4] = w3[p2];
+                c2[4] = up2;
+                c3[4] = up3;
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
                     dz2[q] = dz2[q + 1];
@@ -260,24 +283,23 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_cross1_tiled64(Grid g, const do
             const long long pk = (long long)k * nxy;
             s2[ty + 2][tx] = c2[2];
             s3[ty][tx + 2] = c3[2];
-            s4[ty + 2][tx + 2] = w4[pk + xy];
-            if (ty < 2) {
-                s2[ty][tx] = w2[pk + xy_jm];
-                s4[ty][tx + 2] = w4[pk + xy_jm];
+            s4[ty + 2][tx + 2] = own4;
+            if (halo_y) {
+                s2[ry][tx] = hy2;
+                s4[ry][tx + 2] = hy4;
             }
-            if (ty >= CT_Y - 2) {
-                s2[ty + 4][tx] = w2[pk + xy_jp];
-                s4[ty + 4][tx + 2] = w4[pk + xy_jp];
-            }
-            if (tx < 2) {
-                s3[ty][tx] = w3[pk + xy_im];
-                s4[ty + 2][tx] = w4[pk + xy_im];
-            }
-            if (tx >= CT_X - 2) {
-                s3[ty][tx + 4] = w3[pk + xy_ip];
-                s4[ty + 2][tx + 4] = w4[pk + xy_ip];
+            if (halo_x) {
+                s3[ty][rx] = hx3;
+                s4[ty + 2][rx] = hx4;
             }
             __syncthreads();
+            if (k + 1 < k1) {
+                const long long p3 = plane(k + 3) + xy;
+                up2 = w2[p3];
+                up3 = w3[p3];
+                own4 = w4[pk + nxy + xy];
+                halos(pk + nxy);
+            }
             // d: own position (index + 1), then the halo positions; d at index c is w(c) - w(c - 1) in
             // the shifted columns (x: s[.][c + 1] - s[.][c]; y: s[r + 1][.] - s[r][.])
             dx3[ty][tx + 1] = rn_sub(s3[ty][tx + 2], s3[ty][tx + 1]);
@@ -332,9 +354,11 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_cross1_tiled64(Grid g, const do
             for (int q = 0; q < 3; ++q) E[q] = ex4[ty][tx + q];
             weno3_terms<false, double>(d, E, nullptr, sx4, unused);
             const long long z = pk + xy;
-            S2[(0 * NV + v) * N + z] = rn_mul(0.5, rn_add(sy2, sx3));
-            S2[(1 * NV + v) * N + z] = rn_mul(0.5, rn_add(sz3, sy4));
-            S2[(2 * NV + v) * N + z] = rn_mul(0.5, rn_add(sz2, sx4));
+            if (inside) {
+                S2[(0 * NV + v) * N + z] = rn_mul(0.5, rn_add(sy2, sx3));
+                S2[(1 * NV + v) * N + z] = rn_mul(0.5, rn_add(sz3, sy4));
+                S2[(2 * NV + v) * N + z] = rn_mul(0.5, rn_add(sz2, sx4));
+            }
         }
         __syncthreads();           // the next variable's first plane overwrites the tiles
     }
@@ -345,24 +369,29 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_cross1_tiled64(Grid g, const do
 // along x and y, the z terms in registers per column; each zone then blends from four d, three D2 and
 // three E per direction (weno3_terms).  MHD field components (v >= 5) come from the face-B WENO's zone
 // means, and their own direction is left to it, as in zone_weno1d.  Same bits as zone_weno1d.
-// Requires nx % CT_X == 0 and ny % CT_Y == 0 (other grids use k_weno1d).
+// Any grid (tiles64 says which take it).
 template <int ORDER, int NV>
-__global__ void __launch_bounds__(CT_X * CT_Y) k_weno1d_tiled64(Grid g, const double* __restrict__ U,
+__global__ void __launch_bounds__(CT_X * CT_Y, 3) k_weno1d_tiled64(Grid g, const double* __restrict__ U,
                                                                 const double* __restrict__ ZB,
-                                                                double* __restrict__ S1) {
+                                                                double* __restrict__ S1, int cz) {
     constexpr bool WANT_C = ORDER == 3;
     __shared__ double su[CT_Y + 4][CT_X + 4];                         // the plane, x and y halos of two
     __shared__ double dx[CT_Y][CT_X + 3], cx[CT_Y][CT_X + 2], ex[CT_Y][CT_X + 2];   // at i0 - 1 + c
     __shared__ double dy[CT_Y + 3][CT_X], cy[CT_Y + 2][CT_X], ey[CT_Y + 2][CT_X];   // at j0 - 1 + r
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int tiles_x = g.nx / CT_X;
+    const int tiles_x = (g.nx + CT_X - 1) / CT_X;
     const int i = (int)(blockIdx.x % tiles_x) * CT_X + tx, j = (int)(blockIdx.x / tiles_x) * CT_Y + ty;
-    const int k0 = (int)blockIdx.y * CT_Z, k1 = min(k0 + CT_Z, g.nz);
+    const int k0 = (int)blockIdx.y * cz, k1 = min(k0 + cz, g.nz);
+    const bool inside = i < g.nx && j < g.ny;        // columns past the grid's end only serve as halos
     const long long N = g.n;
     const long long nxy = (long long)g.nx * g.ny;
-    const long long xy = (long long)j * g.nx + i;
-    const long long xy_jm = (long long)wrap(j - 2, g.ny) * g.nx + i, xy_jp = (long long)wrap(j + 2, g.ny) * g.nx + i;
-    const long long xy_im = (long long)j * g.nx + wrap(i - 2, g.nx), xy_ip = (long long)j * g.nx + wrap(i + 2, g.nx);
+    const int iw = wrap(i, g.nx), jw = wrap(j, g.ny);
+    const long long xy = (long long)jw * g.nx + iw;
+    // the halo columns this thread brings: two rows below and above, two columns left and right
+    const bool halo_y = ty < 2 || ty >= CT_Y - 2, halo_x = tx < 2 || tx >= CT_X - 2;
+    const int ry = ty < 2 ? ty : ty + 4, rx = tx < 2 ? tx : tx + 4;
+    const long long xy_y = (long long)wrap(ty < 2 ? j - 2 : j + 2, g.ny) * g.nx + iw;
+    const long long xy_x = (long long)jw * g.nx + wrap(tx < 2 ? i - 2 : i + 2, g.nx);
     auto plane = [&](int kk) -> long long { return (long long)wrap(kk, g.nz) * nxy; };
     const int hx_d = tx == 0 ? 0 : CT_X + tx;          // halo entries, as in k_cross1_tiled64
     const int hx_e = tx == 0 ? 0 : CT_X + 1;
@@ -381,11 +410,13 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_weno1d_tiled64(Grid g, const do
             cz[q] = rn_sub(dz[q + 1], dz[q]);
             ez[q] = w3_curv(cz[q]);
         }
+        // the next plane's values are loaded a plane ahead, behind the first barrier
+        double hy = halo_y ? u[k0 * nxy + xy_y] : 0.0, hx = halo_x ? u[k0 * nxy + xy_x] : 0.0, up = 0.0;
         for (int k = k0; k < k1; ++k) {
             if (k > k0) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) c[q] = c[q + 1];
-                c[4] = u[plane(k + 2) + xy];
+                c[4] = up;
 #pragma unroll
                 for (int q = 0; q < 3; ++q) dz[q] = dz[q + 1];
                 dz[3] = rn_sub(c[4], c[3]);
@@ -399,11 +430,14 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_weno1d_tiled64(Grid g, const do
             }
             const long long pk = (long long)k * nxy;
             su[ty + 2][tx + 2] = c[2];
-            if (ty < 2) su[ty][tx + 2] = u[pk + xy_jm];
-            if (ty >= CT_Y - 2) su[ty + 4][tx + 2] = u[pk + xy_jp];
-            if (tx < 2) su[ty + 2][tx] = u[pk + xy_im];
-            if (tx >= CT_X - 2) su[ty + 2][tx + 4] = u[pk + xy_ip];
+            if (halo_y) su[ry][tx + 2] = hy;
+            if (halo_x) su[ty + 2][rx] = hx;
             __syncthreads();
+            if (k + 1 < k1) {
+                up = u[plane(k + 3) + xy];
+                if (halo_y) hy = u[pk + nxy + xy_y];
+                if (halo_x) hx = u[pk + nxy + xy_x];
+            }
             dx[ty][tx + 1] = rn_sub(su[ty + 2][tx + 2], su[ty + 2][tx + 1]);
             dy[ty + 1][tx] = rn_sub(su[ty + 2][tx + 2], su[ty + 1][tx + 2]);
             if (tx < 3) dx[ty][hx_d] = rn_sub(su[ty + 2][hx_d + 1], su[ty + 2][hx_d]);
@@ -433,8 +467,8 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_weno1d_tiled64(Grid g, const do
                     E[q] = ex[ty][tx + q];
                 }
                 weno3_terms<WANT_C, double>(d, E, D2, b, cc);
-                S1[((0 * 3 + 0) * NV + v) * N + z] = b;
-                if (WANT_C) S1[((1 * 3 + 0) * NV + v) * N + z] = cc;
+                if (inside) S1[((0 * 3 + 0) * NV + v) * N + z] = b;
+                if (WANT_C && inside) S1[((1 * 3 + 0) * NV + v) * N + z] = cc;
             }
             if (own != 1) {
 #pragma unroll
@@ -445,45 +479,65 @@ __global__ void __launch_bounds__(CT_X * CT_Y) k_weno1d_tiled64(Grid g, const do
                     E[q] = ey[ty + q][tx];
                 }
                 weno3_terms<WANT_C, double>(d, E, D2, b, cc);
-                S1[((0 * 3 + 1) * NV + v) * N + z] = b;
-                if (WANT_C) S1[((1 * 3 + 1) * NV + v) * N + z] = cc;
+                if (inside) S1[((0 * 3 + 1) * NV + v) * N + z] = b;
+                if (WANT_C && inside) S1[((1 * 3 + 1) * NV + v) * N + z] = cc;
             }
             if (own != 2) {
                 weno3_terms<WANT_C, double>(dz, ez, cz, b, cc);
-                S1[((0 * 3 + 2) * NV + v) * N + z] = b;
-                if (WANT_C) S1[((1 * 3 + 2) * NV + v) * N + z] = cc;
+                if (inside) S1[((0 * 3 + 2) * NV + v) * N + z] = b;
+                if (WANT_C && inside) S1[((1 * 3 + 2) * NV + v) * N + z] = cc;
             }
         }
         __syncthreads();
     }
 }
 
+// The FP64 tiles take any grid; a column past its end only serves as a halo.  They share a position's terms among the
+// zones that use them, so they pay where at least half of their columns are zones (93 x 75 x 110 zones, second order,
+// 73% of the columns: 0.81 ms by zones in FP64, 0.49 ms in tiles with the integer blends); below that, and where there
+// are too few tiles for the chip, the per-zone kernels run.  A block marches through up to CT_Z planes, fewer where that leaves the chip idle.
+static bool tiles64(const Grid& g, dim3& grid, int& cz) {
+    const long long tx = (g.nx + CT_X - 1) / CT_X, ty = (g.ny + CT_Y - 1) / CT_Y;
+    if ((long long)g.nx * g.ny * 2 < tx * ty * CT_X * CT_Y) return false;
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long planes = tx * ty * g.nz / (2 * sms);      // planes a block for two blocks per SM
+    if (planes < 1) return false;
+    cz = (int)(planes < CT_Z ? planes : CT_Z);
+    grid = dim3((unsigned)(tx * ty), (unsigned)((g.nz + cz - 1) / cz));
+    return grid.y <= 65535u;
+}
+
 template <int ORDER, int NV>
 static bool launch_weno1d_tiled64(const Grid& g, const double* U, const double* ZB, double* S1, cudaStream_t st) {
-    if (g.nx % CT_X != 0 || g.ny % CT_Y != 0) return false;
-    const dim3 grid((unsigned)((g.nx / CT_X) * (g.ny / CT_Y)), (unsigned)((g.nz + CT_Z - 1) / CT_Z));
-    k_weno1d_tiled64<ORDER, NV><<<grid, dim3(CT_X, CT_Y), 0, st>>>(g, U, ZB, S1);
+    dim3 grid;
+    int cz;
+    if (!tiles64(g, grid, cz)) return false;
+    k_weno1d_tiled64<ORDER, NV><<<grid, dim3(CT_X, CT_Y), 0, st>>>(g, U, ZB, S1, cz);
     return true;
 }
 
 template <int NV>
 static bool launch_cross1_tiled64(const Grid& g, const double* S1, double* S2, cudaStream_t st) {
-    if (g.nx % CT_X != 0 || g.ny % CT_Y != 0) return false;
-    const dim3 grid((unsigned)((g.nx / CT_X) * (g.ny / CT_Y)), (unsigned)((g.nz + CT_Z - 1) / CT_Z));
-    k_cross1_tiled64<NV><<<grid, dim3(CT_X, CT_Y), 0, st>>>(g, S1, S2);
+    dim3 grid;
+    int cz;
+    if (!tiles64(g, grid, cz)) return false;
+    k_cross1_tiled64<NV><<<grid, dim3(CT_X, CT_Y), 0, st>>>(g, S1, S2, cz);
     return true;
 }
 
 template <int NV, class R>
 __global__ void __launch_bounds__(128) k_cross2(Grid g, R* __restrict__ S2) {
     const long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (z < g.n) zone_cross2<NV>(g, S2, z);
+    if (z < g.n) zone_cross2<NV>(g, S2, z, (int)blockIdx.y, (int)gridDim.y);
 }
 
 template <int NV, class R>
 static int launch_recon_nv(const StepArgs& a, const double* U, cudaStream_t st) {
     const int T = 128;
     const unsigned blocks = (unsigned)((a.grid.n + T - 1) / T);
+    const dim3 split(blocks, sizeof(R) == 8 ? NV : 1);
     R* S1 = (R*)a.S1;
     R* S2 = (R*)a.S2;
     R* ZB = (R*)a.ZB;
@@ -513,25 +567,25 @@ static int launch_recon_nv(const StepArgs& a, const double* U, cudaStream_t st) 
     }
     switch (a.order) {
         case 2:
-            if (!tiled1d) k_weno1d<2, NV, R, In><<<blocks, T, 0, st>>>(a.grid, Ui, ZB, S1);
+            if (!tiled1d) k_weno1d<2, NV, R, In><<<split, T, 0, st>>>(a.grid, Ui, ZB, S1);
             n += 1;
             break;
         case 3:
-            if (!tiled1d) k_weno1d<3, NV, R, In><<<blocks, T, 0, st>>>(a.grid, Ui, ZB, S1);
+            if (!tiled1d) k_weno1d<3, NV, R, In><<<split, T, 0, st>>>(a.grid, Ui, ZB, S1);
             // shared-memory tiles where the grid allows them (and the context has not turned tiles off)
             if constexpr (sizeof(R) == 4) {
                 if (!(a.tiled && launch_cross1_tiled<NV>(a.grid, S1, S2, st)))
-                    k_cross1<3, NV, R><<<blocks, T, 0, st>>>(a.grid, S1, S2);
+                    k_cross1<3, NV, R><<<split, T, 0, st>>>(a.grid, S1, S2);
             } else {
                 if (!(a.tiled && launch_cross1_tiled64<NV>(a.grid, S1, S2, st)))
-                    k_cross1<3, NV, R><<<blocks, T, 0, st>>>(a.grid, S1, S2);
+                    k_cross1<3, NV, R><<<split, T, 0, st>>>(a.grid, S1, S2);
             }
             n += 2;
             break;
         default:
-            k_weno1d<4, NV, R, In><<<blocks, T, 0, st>>>(a.grid, Ui, ZB, S1);
-            k_cross1<4, NV, R><<<blocks, T, 0, st>>>(a.grid, S1, S2);
-            k_cross2<NV, R><<<blocks, T, 0, st>>>(a.grid, S2);
+            k_weno1d<4, NV, R, In><<<split, T, 0, st>>>(a.grid, Ui, ZB, S1);
+            k_cross1<4, NV, R><<<split, T, 0, st>>>(a.grid, S1, S2);
+            k_cross2<NV, R><<<split, T, 0, st>>>(a.grid, S2);
             n += 3;
     }
     return n;

@@ -109,7 +109,9 @@ int launch_max_dt(const Grid& g, const double* U, const double* Bf, double gamma
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    long long want = (g.n + 1023) / 1024;                 // four zones per thread and pass
+    // four zones per thread and pass; one while that leaves SMs idle (16^3 zones: 16 blocks instead of 4)
+    long long want = (g.n + 1023) / 1024;
+    if (want < sms) want = (g.n + 255) / 256 < sms ? (g.n + 255) / 256 : sms;
     const long long cap = (long long)sms * 8;
     const unsigned blocks = (unsigned)(want < cap ? (want > 0 ? want : 1) : cap);
     if (fp32)

@@ -92,26 +92,26 @@ ADER_DEV Vec<8, R> mhd_abs_jacobian_apply(R rho, const R* v, R p, const R* B, R 
     const R k = R(0.28209479177387814);        // 1 / sqrt(4 pi)
     const R bx = B[D] * k, by = B[T1] * k, bz = B[T2] * k;
     const R u = v[D], vt1 = v[T1], vt2 = v[T2];
-    const R irho = rcp(rho), sr = sqrt(rho), isr = rcp(sr);
-    const R a2 = gamma * p * irho, a = sqrt(a2);
+    const R irho = rcp(rho), sr = speed_root(rho), isr = rcp(sr);
+    const R a2 = gamma * p * irho, a = speed_root(a2);
     const R ca2 = bx * bx * irho, bt2 = (by * by + bz * bz) * irho;
     const R sum = a2 + ca2 + bt2;
-    const R disc = sqrt(fmax(sum * sum - R(4) * a2 * ca2, R(0)));
+    const R disc = speed_root(fmax(sum * sum - R(4) * a2 * ca2, R(0)));
     const R cf2 = R(0.5) * (sum + disc), cs2 = fmax(R(0.5) * (sum - disc), R(0));
-    const R cf = sqrt(cf2), cs = sqrt(cs2), ca = sqrt(ca2);
+    const R cf = speed_root(cf2), cs = speed_root(cs2), ca = speed_root(ca2);
     const R tiny = sizeof(R) == 8 ? R(1e-12) : R(1e-6);
     const R dc = cf2 - cs2;
     R af = R(1), as = R(0);
     if (dc > tiny * cf2) {
-        af = sqrt(fmax(a2 - cs2, R(0)));
-        as = sqrt(fmax(cf2 - a2, R(0)));
-        const R n = rcp(sqrt(af * af + as * as));       // af^2 + as^2 = 1 up to round-off
+        af = speed_root(fmax(a2 - cs2, R(0)));
+        as = speed_root(fmax(cf2 - a2, R(0)));
+        const R n = rcp(speed_root(af * af + as * as));       // af^2 + as^2 = 1 up to round-off
         af *= n;
         as *= n;
     }
-    const R bt = sqrt(by * by + bz * bz);
+    const R bt = speed_root(by * by + bz * bz);
     R ey = R(0.70710678118654752), ez = R(0.70710678118654752);
-    if (bt > tiny * sqrt(rho * sum)) {
+    if (bt > tiny * speed_root(rho * sum)) {
         ey = by / bt;
         ez = bz / bt;
     }

@@ -1,6 +1,9 @@
 // WENO building blocks of the zone-centred reconstruction (see recon.cu for the reading).
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
+#include "fixed.cuh"
 
 namespace ader {
 
@@ -111,8 +114,132 @@ template <> ADER_DEV double rn_mul<double>(double x, double y) {
 template <class R>
 ADER_DEV R w3_curv(R D2) { return fma(rn_mul(R(13.0 / 3.0), D2), D2, R(4.0 * WENO_EPS)); }
 
+// ---------------------------------------------------------------- FP64: the blend on the integer units
+// A blend sum_s g_s x_s / t_s^2 / sum_s g_s / t_s^2 of S candidates, t = EPS + IS > 0, is the FP64 kernels' costliest
+// part: squares and products of the t (the cleared denominators), a reciprocal and the weighted sum, 17 FP64
+// instructions for S = 3 and one output.  Here the products run as 64 x 64-bit integer products of normalised
+// mantissas (upper halves; 7.4 a clock and SM against 1.7 FP64 multiplications) with their exponents apart, and the
+// two sums are integers aligned to their largest term with 57 bits or more (56 for S = 4).  What stays FP64 is the quotient of the
+// sums: one reciprocal for all outputs and one product each.  Errors against 80-bit arithmetic are smaller than the
+// FP64 form's, and no intermediate value overflows.
+ADER_DEV unsigned long long u64_mulhi(unsigned long long a, unsigned long long b) {
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (unsigned long long)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+ADER_DEV int u32_clz(unsigned x) {          // x > 0
+#ifdef __CUDA_ARCH__
+    return __clz((int)x);
+#else
+    return __builtin_clz(x);
+#endif
+}
+
+// m 2^e, the leading bit of m set
+struct Scaled {
+    unsigned long long m;
+    int e;
+};
+// x > 0; e counts from the exponent field (the same offset for every value, which the quotient cancels)
+ADER_DEV Scaled scaled_of(double x) {
+    const unsigned long long b = (unsigned long long)bits_of(x);
+    return {(b << 11) | 0x8000000000000000ull, (int)((unsigned)(b >> 52) & 0x7ffu)};
+}
+ADER_DEV Scaled operator*(Scaled a, Scaled b) {
+    const unsigned long long m = u64_mulhi(a.m, b.m);
+    const int up = (int)(~m >> 63);                          // the product of two in [1, 2) halves: one place at most
+    return {m << up, a.e + b.e - up};
+}
+
+// an integer 2^32 <= w < 2^63 as the FP64 number w 2^-63, to nearest (ties up)
+ADER_DEV double unit_of(unsigned long long w) {
+    const int lz = u32_clz((unsigned)(w >> 32));
+    const unsigned long long n = ((w << (lz - 1)) + 0x200ull) >> 10;
+    return of_bits((long long)(n + ((unsigned long long)(1023 - lz - 1) << 52)));      // the leading one adds one
+}
+
+// the candidates' weights g_s prod_{r != s} t_r^2 without the gains g (1, 10, 1 or 1, 10, 10, 1), their largest exponent
+// and 2^63 / sum g_s w_s 2^-(GUARD + em)
+template <int S>
+struct IntWeights {
+    Scaled w[S];
+    int em;
+    double inv;
+
+    ADER_DEV explicit IntWeights(const double* t) {
+        Scaled q[S];
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            const Scaled x = scaled_of(t[s]);
+            q[s] = x * x;
+        }
+        if constexpr (S == 3) {
+            w[0] = q[1] * q[2];
+            w[1] = q[0] * q[2];
+            w[2] = q[0] * q[1];
+        } else {
+            const Scaled q01 = q[0] * q[1], q23 = q[2] * q[3];
+            w[0] = q[1] * q23;
+            w[1] = q[0] * q23;
+            w[2] = q01 * q[3];
+            w[3] = q01 * q[2];
+        }
+        em = w[0].e;
+#pragma unroll
+        for (int s = 1; s < S; ++s) em = w[s].e > em ? w[s].e : em;
+        unsigned long long sum = 0;
+#pragma unroll
+        for (int s = 0; s < S; ++s) sum += gain(s, down(w[s].m, em - w[s].e));
+        inv = rcp(unit_of(sum));
+    }
+    // m 2^-(GUARD + d): places for the sum of gains (12 or 22 times the largest term, and a sign)
+    static constexpr int GUARD = S == 3 ? 5 : 6;
+    static ADER_DEV unsigned long long down(unsigned long long m, int d) { return m >> (d < 63 - GUARD ? d + GUARD : 63); }
+    static ADER_DEV unsigned long long gain(int s, unsigned long long x) { return s == 0 || s == S - 1 ? x : 10ull * x; }
+
+    // half the blend of the candidates' values x (the candidates are carried doubled)
+    ADER_DEV double half_blend(const double* x) const {
+        unsigned long long m[S];
+        int e[S], tm = -4096, ex = 0;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            const Scaled v = scaled_of(x[s]);
+            m[s] = u64_mulhi(w[s].m, v.m);
+            e[s] = w[s].e + v.e;
+            tm = e[s] > tm ? e[s] : tm;
+            ex = v.e > ex ? v.e : ex;
+        }
+        unsigned long long n = 0;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            const unsigned long long g = gain(s, down(m[s], tm - e[s]));
+            const unsigned long long sg = (unsigned long long)(bits_of(x[s]) >> 63);
+            n += (g ^ sg) - sg;
+        }
+        // n 2^(tm - em - 1086) times inv is the result
+        const unsigned long long sg = (unsigned long long)((long long)n >> 63), a = (n ^ sg) - sg;
+        const unsigned hi = (unsigned)(a >> 32), top = hi ? hi : (unsigned)a;
+        const int lz = u32_clz(top | 1u) + (hi ? 0 : 32);
+        const int be = tm - em - lz;                         // the exponent field
+        unsigned long long r = (((a << (lz - 1 & 63)) + 0x200ull) >> 10) + ((unsigned long long)(unsigned)(be - 1) << 52);
+        r = a && be > 0 && ex > 0 ? r : 0ull;                // zero where all candidates are zero or subnormal
+        r |= (sg & 0x8000000000000000ull) | (ex == 0x7ff ? 0x7ff8000000000000ull : 0ull);
+        return rn_mul(of_bits((long long)r), inv);
+    }
+};
+
 template <bool WANT_C, class R>
 ADER_DEV void weno3_terms(const R* d, const R* E, const R* D2, R& b, R& c) {
+    if constexpr (std::is_same<R, double>::value) {
+        const double B[3] = {fma(3.0, d[1], -d[0]), rn_add(d[1], d[2]), fma(3.0, d[2], -d[3])};
+        const double t[3] = {fma(B[0], B[0], E[0]), fma(B[1], B[1], E[1]), fma(B[2], B[2], E[2])};
+        const IntWeights<3> w(t);
+        b = w.half_blend(B);
+        if (WANT_C) c = w.half_blend(D2);
+        return;
+    }
     const R B0 = fma(R(3.0), d[1], -d[0]), B1 = rn_add(d[1], d[2]), B2 = fma(R(3.0), d[2], -d[3]);
     const R t0 = fma(B0, B0, E[0]), t1 = fma(B1, B1, E[1]), t2 = fma(B2, B2, E[2]);
     const R q0 = rn_mul(t0, t0), q1 = rn_mul(t1, t1), q2 = rn_mul(t2, t2);
@@ -152,6 +279,42 @@ ADER_DEV void weno3(const R* a, R& b, R& c) {
 // order-4 1-D WENO on the seven values a[-3..3] (a[3] = centre); returns b, c, d
 template <class R>
 ADER_DEV void weno4(const R* a, R& b, R& c, R& d) {
+    if constexpr (std::is_same<R, double>::value) {
+        // The candidates from the six neighbour differences e, as integers of a common exponent: 60 b, 2 c and 6 d
+        // of each stencil (sums of up to 200 e), and 3600 (EPS + IS) = T^2 + 3900 (2 c)^2 + 3905 (6 d)^2 + 3600 EPS
+        // with T = 60 b + 6 d.  34 FP64 instructions; all in FP64 it took 135.
+        FixFrame<1, 2> fr;
+        Vec<1, double> e[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            e[j][0] = a[j + 1] - a[j];
+            fr.include(e[j]);
+        }
+        fr.close();
+        Fix x[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) x[j] = fr.enter(e[j])[0];
+        const Fix cb[4] = {109.0 * x[2] - 68.0 * x[1] + 19.0 * x[0], 19.0 * x[3] + 52.0 * x[2] - 11.0 * x[1],
+                           52.0 * x[3] + 19.0 * x[2] - 11.0 * x[4], 109.0 * x[3] - 68.0 * x[4] + 19.0 * x[5]};
+        const Fix cc[3] = {2.0 * x[2] - 3.0 * x[1] + x[0], x[3] - x[2], 3.0 * x[4] - 2.0 * x[3] - x[5]};
+        double B[4], C[4], D[4], t[4];
+        C[0] = fr.leave_one(0, cc[0]);
+        C[1] = C[2] = fr.leave_one(0, cc[1]);
+        C[3] = fr.leave_one(0, cc[2]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const Fix cd = x[q + 2] - 2.0 * x[q + 1] + x[q];
+            B[q] = fr.leave_one(0, cb[q]);
+            D[q] = fr.leave_one(0, cd);
+            const double T = fr.leave_one(0, cb[q] + cd);
+            t[q] = fma(T, T, fma(3900.0 * C[q], C[q], fma(3905.0 * D[q], D[q], 3600.0 * WENO_EPS)));
+        }
+        const IntWeights<4> w(t);
+        b = w.half_blend(B) * (1.0 / 30.0);
+        c = w.half_blend(C);
+        d = w.half_blend(D) * (1.0 / 3.0);
+        return;
+    }
     const R um3 = a[0], um2 = a[1], um1 = a[2], u0 = a[3], up1 = a[4], up2 = a[5], up3 = a[6];
     R cb[4], cc[4], cd[4];
     // stencil {i-3..i}
@@ -258,9 +421,10 @@ ADER_DEV R slope_of(const Grid& g, const R* __restrict__ F, int i, int j, int k,
 // whose moments along e come from the face-B WENO (zone_face_b), so only the
 // two transverse directions are reconstructed here.
 // T: the type U is read in (double, or the FP32 copy of FP32-bulk steps).
+// The variables v0, v0 + vstep, ... (FP32 Euler at orders 2-3: all of them, paired).
 template <int ORDER, int NV, class R, class T>
 ADER_DEV void zone_weno1d(const Grid& g, const T* __restrict__ U, const R* __restrict__ ZB,
-                          R* __restrict__ S1, long long z) {
+                          R* __restrict__ S1, long long z, int v0 = 0, int vstep = 1) {
     int i, j, k;
     zone_ijk(g, z, i, j, k);
 #ifdef __CUDA_ARCH__
@@ -313,7 +477,7 @@ ADER_DEV void zone_weno1d(const Grid& g, const T* __restrict__ U, const R* __res
             for (int o = -RAD; o <= RAD; ++o) off[d][o + RAD] = o == 0 ? 0 : nbr_along(g, z, i, j, k, d, o) - z;
         // per variable the three directions' moments before any store (a store could alias the next
         // loads for all the compiler knows, and would hold them back)
-        for (int v = 0; v < NV; ++v) {
+        for (int v = v0; v < NV; v += vstep) {
             const T* Uv = v < 5 ? U + (long long)v * g.n + z : nullptr;
             const R* Bv = v >= 5 ? ZB + (long long)(v - 5) * g.n + z : nullptr;
             const R centre = v < 5 ? R(Uv[0]) : Bv[0];
@@ -347,9 +511,10 @@ ADER_DEV void zone_weno1d(const Grid& g, const T* __restrict__ U, const R* __res
     }
 }
 
-// first-level cross moments w8 w9 w10 (w14..w19 at order 4) of zone z
+// first-level cross moments w8 w9 w10 (w14..w19 at order 4) of zone z, variables v0, v0 + vstep, ... (FP32: all)
 template <int ORDER, int NV, class R>
-ADER_DEV void zone_cross1(const Grid& g, const R* __restrict__ S1, R* __restrict__ S2, long long z) {
+ADER_DEV void zone_cross1(const Grid& g, const R* __restrict__ S1, R* __restrict__ S2, long long z, int v0 = 0,
+                          int vstep = 1) {
     int i, j, k;
     zone_ijk(g, z, i, j, k);
 #ifdef __CUDA_ARCH__
@@ -402,7 +567,7 @@ ADER_DEV void zone_cross1(const Grid& g, const R* __restrict__ S1, R* __restrict
         }
     } else
 #endif
-    for (int v = 0; v < NV; ++v) {
+    for (int v = v0; v < NV; v += vstep) {
         const R* w2 = S1 + ((0 * 3 + 0) * NV + v) * g.n;
         const R* w3 = S1 + ((0 * 3 + 1) * NV + v) * g.n;
         const R* w4 = S1 + ((0 * 3 + 2) * NV + v) * g.n;
@@ -423,12 +588,12 @@ ADER_DEV void zone_cross1(const Grid& g, const R* __restrict__ S1, R* __restrict
     }
 }
 
-// w20 of zone z from the first-level cross moments of its neighbours
+// w20 of zone z from the first-level cross moments of its neighbours, variables v0, v0 + vstep, ...
 template <int NV, class R>
-ADER_DEV void zone_cross2(const Grid& g, R* __restrict__ S2, long long z) {
+ADER_DEV void zone_cross2(const Grid& g, R* __restrict__ S2, long long z, int v0 = 0, int vstep = 1) {
     int i, j, k;
     zone_ijk(g, z, i, j, k);
-    for (int v = 0; v < NV; ++v) {
+    for (int v = v0; v < NV; v += vstep) {
         const R* w8 = S2 + (0 * NV + v) * g.n;
         const R* w9 = S2 + (1 * NV + v) * g.n;
         const R* w10 = S2 + (2 * NV + v) * g.n;
