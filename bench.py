@@ -183,7 +183,7 @@ UPDATE_FLOPS = 3 * 5 * 3 + 5 * 2      # Eq. 6 from stored fluxes: per direction 
 def flops_per_zone(order, form, solver, fp32, tiled=True):
     """Exact FLOPs per zone of each kernel (op-counting instantiation of the kernels' per-zone code).
 
-    Tiled layout (Euler, orders 2-3): the predictor kernel also solves each face once, so it carries the
+    Tiled layout (FP32 Euler, orders 2-3): the predictor kernel also solves each face once, so it carries the
     face solves and the update kernel only Eq. 6 from the stored fluxes."""
     path = os.path.join(ROOT, "paper_1006_2146_gb300", "flops.json")
     if not os.path.exists(path):
@@ -955,7 +955,8 @@ def gpu_arm(args):
 
     # dominant kernel roofline: FLOPs per zone x zones / mean launch time.  The plain kernels are bound by
     # the FP64 (or FP32) ALUs; the learned-guess kernel is a dense contraction on the tensor cores.
-    fpz = flops_per_zone(args.order, args.form, args.solver, args.fp32)
+    # (FP64 predicts by teams of warps and solves the faces in the update phase; the FP32 tiles solve them themselves)
+    fpz = flops_per_zone(args.order, args.form, args.solver, args.fp32, tiled=args.fp32)
     fpz["learned_guess"] = 2.0 * (52 * 128 + 128 * 128 + 128 * 25)       # the MLP's multiply-adds per zone
     kname, (kl, kms) = max(((k, v) for k, v in prof.items()), key=lambda kv: kv[1][1])
     k_avg = kms / kl / 1e3

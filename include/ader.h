@@ -180,14 +180,16 @@ int ader_set_predictor(ader_ctx* ctx, double tol, int max_iter);
  * writes its face data to the context's scratch and a second pass solves the
  * faces.  Both give the same numbers bit for bit in FP64 (in FP32 bulk to
  * FP32 rounding: the compiler may contract the predictor's multiply-adds
- * differently in the two kernels); MHD contexts and order 4
- * always take the second layout (the edge fields need the face data of four
- * zones; the fourth-order predictor's cost dwarfs the face data's traffic).
- * on = 1 also computes the third-order cross moments of the reconstruction
- * (Euler and MHD) in shared-memory tiles of 32 x 8 columns where nx is a
- * multiple of 32 and ny of 8, each WENO term of a position once for all the
- * zones that use it; on = 0 takes the per-zone kernel, with the same bits in
- * FP64 (FP32 to FP32 rounding).
+ * differently in the two kernels).  Only FP32 bulk (Euler, orders 2-3) has
+ * the predictor tiles; FP64, MHD and order 4 always write the face data (the
+ * FP64 predictor runs by teams of warps, MHD's edge fields need the face data
+ * of four zones).
+ * on = 1 also computes the moments of the reconstruction in shared-memory
+ * tiles of 32 x 8 columns, each WENO term of a position once for all the
+ * zones that use it: FP64 1-D and cross moments of orders 2-3 (Euler and MHD)
+ * on every grid that fills at least half of its tiles' columns, FP32 cross
+ * moments of order 3 where nx is a multiple of 32 and ny of 8; on = 0 takes
+ * the per-zone kernels, with the same bits in FP64 (FP32 to FP32 rounding).
  * ADER_ERR_ARG for a NULL context. */
 int ader_set_tiled(ader_ctx* ctx, int on);
 

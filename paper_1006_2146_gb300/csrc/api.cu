@@ -36,7 +36,7 @@ struct ader_ctx {
     double* rkB[6] = {};                      // MHD: SSP-RK stage face fields and the stored operator
     double tol = 0.0;                         // converged predictor tolerance (0: fixed M-1 iterations)
     int max_iter = 50;
-    bool tiled = true;                        // Euler: per-tile predictor and face solves (ader_set_tiled)
+    bool tiled = true;                        // WENO tiles and FP32 predictor tiles (ader_set_tiled)
     bool wait_test = false;                   // the next learned-guess launch tests its bounded waits
     int bc[6] = {0, 0, 0, 0, 0, 0};           // box faces (ader_set_boundary); all periodic by default
     int ghosts[3] = {0, 0, 0};                // ghost zones per side of each non-periodic axis
@@ -149,7 +149,7 @@ static StepArgs make_args(const ader_ctx* c, double dt, const double* dt_dev, in
     a.modes_out = nullptr;
     a.emf_transonic = (c->flags & ADER_EMF_TRANSONIC) ? 1 : 0;
     a.defer_nonfinite = 0;
-    a.tiled = c->tiled ? 1 : 0;               // the predictor tiles check the physics and order themselves
+    a.tiled = c->tiled ? 1 : 0;               // the tiles check physics, precision and order themselves
     a.wait_test = c->wait_test ? 1 : 0;
     return a;
 }

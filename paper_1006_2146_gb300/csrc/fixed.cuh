@@ -16,7 +16,7 @@
 //
 // Range.  HEADROOM = 10 - LSH bits are left above the largest mode for sums; intermediate sums may wrap (the
 // arithmetic is modulo 2^64) as long as no wrapped value is shifted or scaled by a fraction.  Modes of magnitude
-// below 2^-959 count as zero; a variable with a mode that is not finite, or within 2^16 of the largest FP64
+// below 2^-767 count as zero; a variable with a mode that is not finite, or within 2^16 of the largest FP64
 // number, leaves as NaN at every node.
 #pragma once
 #include "common.cuh"
@@ -102,6 +102,7 @@ struct PlainFrame {
     ADER_DEV void close() {}
     ADER_DEV Vec<NV, S> enter(const Vec<NV, R>& m) const { return m; }
     ADER_DEV PlainFrame extended(const Vec<NV, R>*, int) const { return *this; }
+    ADER_DEV void join(const PlainFrame&) {}
     ADER_DEV Vec<NV, S> from(const PlainFrame&, const Vec<NV, S>& u) const { return u; }
     ADER_DEV Vec<NV, R> leave(const Vec<NV, S>& u) const { return u; }
 };
@@ -128,7 +129,7 @@ struct FixFrame {
         for (int v = 0; v < NV; ++v) {
             e[v] >>= 20;
             bad[v] = e[v] > 2046u - 16u ? 0x7ff80000u : 0u;
-            e[v] = e[v] < 64u ? 64u : e[v];
+            e[v] = e[v] < 256u ? 256u : e[v];
         }
     }
     ADER_DEV Vec<NV, Fix> enter(const Vec<NV, double>& m) const {
@@ -150,12 +151,16 @@ struct FixFrame {
 #pragma unroll
         for (int k = 0; k < n; ++k) r.include(m[k]);
         r.close();
+        r.join(*this);
+        return r;
+    }
+    // after close(): wide enough for the values of o too
+    ADER_DEV void join(const FixFrame& o) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-            r.e[v] = r.e[v] > e[v] ? r.e[v] : e[v];
-            r.bad[v] |= bad[v];
+            e[v] = e[v] > o.e[v] ? e[v] : o.e[v];
+            bad[v] |= o.bad[v];
         }
-        return r;
     }
     ADER_DEV Vec<NV, Fix> from(const FixFrame& o, const Vec<NV, Fix>& u) const {
         Vec<NV, Fix> r;
@@ -188,6 +193,56 @@ struct FixFrame {
         Vec<NV, double> r;
 #pragma unroll
         for (int v = 0; v < NV; ++v) r[v] = leave_one(v, u[v]);
+        return r;
+    }
+};
+
+// Multiplication of flux modes by c_d = dt / dx_d inside a frame.  For integers c_d is a 63-bit integer with the
+// exponent of the largest of the three, the product the upper half of 128 bits; out() is the frame of the products.
+template <class FR> struct AxisScale;
+template <int NV, class R>
+struct AxisScale<PlainFrame<NV, R>> {
+    R c[3];
+    ADER_DEV AxisScale(R cx, R cy, R cz) : c{cx, cy, cz} {}
+    template <int D> ADER_DEV Vec<NV, R> times(const Vec<NV, R>& f) const { return ader::scale(c[D], f); }
+    ADER_DEV PlainFrame<NV, R> out(const PlainFrame<NV, R>& f) const { return f; }
+};
+template <int NV, int LSH>
+struct AxisScale<FixFrame<NV, LSH>> {
+    long long c[3];
+    int k;
+    ADER_DEV AxisScale(double cx, double cy, double cz) {
+        const long long b[3] = {bits_of(cx), bits_of(cy), bits_of(cz)};
+        int e[3];
+        k = 0;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            e[d] = (int)((unsigned)((unsigned long long)b[d] >> 52) & 0x7ffu);
+            k = e[d] > k ? e[d] : k;
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const unsigned long long m = (((unsigned long long)b[d] & 0xfffffffffffffull) | 0x10000000000000ull) << 10;
+            const int sh = k - e[d];
+            const unsigned long long q = e[d] == 0 ? 0ull : m >> (sh < 63 ? sh : 63);
+            const unsigned long long s = (unsigned long long)(b[d] >> 63);
+            c[d] = (long long)((q ^ s) - s);             // c_d = c[d] 2^(k - 1023 - 62)
+        }
+    }
+    template <int D> ADER_DEV Vec<NV, Fix> times(const Vec<NV, Fix>& f) const {
+        Vec<NV, Fix> r;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) r[v].q = fix_mulhi(f[v].q, c[D]);
+        return r;
+    }
+    ADER_DEV FixFrame<NV, LSH> out(const FixFrame<NV, LSH>& f) const {
+        FixFrame<NV, LSH> r = f;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int e = (int)f.e[v] + 2 + k - 1023;
+            r.e[v] = (unsigned)(e < 64 ? 64 : e);
+            if (e > 2046 - 16 || k == 0x7ff) r.bad[v] = 0x7ff80000u;
+        }
         return r;
     }
 };

@@ -257,12 +257,11 @@ int launch_flux_update(const StepArgs& a, double* out, const double* base, doubl
     const int T = 128;
     const unsigned blocks = (unsigned)((a.grid.n + T - 1) / T);
     const int dd = use_dt_dev ? 1 : 0;
-    if (!a.mhd && a.order <= 3 && a.tiled) {   // the tile kernel stored every face flux once
-        if constexpr (sizeof(R) == 4)
+    if constexpr (sizeof(R) == 4) {
+        if (!a.mhd && a.order <= 3 && a.tiled) {   // the tile kernel stored every face flux once
             k_flux_update_stored_pair<R><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
-        else
-            k_flux_update_stored<R><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
-        return 1;
+            return 1;
+        }
     }
     if constexpr (sizeof(R) == 4) {           // fused, both faces of each direction per zone, FP32 pairs
         if (a.mhd && a.solver == SOLVER_HLL)

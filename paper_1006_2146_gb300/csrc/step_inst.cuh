@@ -27,7 +27,7 @@ namespace ader {
         template <bool ALL, class V> static ADER_DEV void face_states(const V* p, V& ub, V& avg, V* t) {            \
             o##O::face_states<ALL>(p, ub, avg, t);                                                                  \
         }                                                                                                           \
-        template <class V> static ADER_DEV V face_mean(const V* F) { return o##O::face_mean(F); }                   \
+        template <class F> static ADER_DEV auto face_mean(const F& f) { return o##O::face_mean(f); }                \
         template <class V> static ADER_DEV void edge_fluxes(const V* f, int s, V& plus, V& minus) {                 \
             o##O::edge_fluxes(f, s, plus, minus);                                                                   \
         }                                                                                                           \
@@ -46,20 +46,18 @@ ADER_ZONEOPS(4)
 #ifndef ADER_BOTH_FACES_DEFINED
 #define ADER_BOTH_FACES_DEFINED
 template <int D, class R>
-ADER_DEV void both_faces_o2(const FrameOf<2, 5, R>& fr, const Vec<5, typename FrameOf<2, 5, R>::S>* s, R gm1,
-                            Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
-    Vec<5, typename FrameOf<2, 5, R>::S> p[6];
-    to_face_frame<2, D, +1>(s, p);
-    o2::face<D>(fr, p, gm1, ub[0], avg[0], Fa[0]);
-    to_face_frame<2, D, -1>(s, p);
-    o2::face<D>(fr, p, gm1, ub[1], avg[1], Fa[1]);
+ADER_DEV void both_faces_o2(const Vec<5, R>* m, R gm1, Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
+    Vec<5, R> p[6];
+    to_face_frame<2, D, +1>(m, p);
+    o2::face<D>(p, gm1, ub[0], avg[0], Fa[0]);
+    to_face_frame<2, D, -1>(m, p);
+    o2::face<D>(p, gm1, ub[1], avg[1], Fa[1]);
 }
 template <int D, class R>
-ADER_DEV void both_faces_o3(const FrameOf<3, 5, R>& fr, const Vec<5, typename FrameOf<3, 5, R>::S>* s, R gm1,
-                            Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
-    Vec<5, typename FrameOf<3, 5, R>::S> p[16];
-    to_face_frame<3, D, +1>(s, p);
-    o3::face_pair<D>(fr, p, gm1, ub, avg, Fa);
+ADER_DEV void both_faces_o3(const Vec<5, R>* m, R gm1, Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
+    Vec<5, R> p[16];
+    to_face_frame<3, D, +1>(m, p);
+    o3::face_pair<D>(p, gm1, ub, avg, Fa);
 }
 #endif
 

@@ -162,7 +162,7 @@ ADER_DEV void enter_frame(const Vec<NV, R>* m, FrameOf<ORDER, NV, R>& fr,
     for (int k = 1; k <= L; ++k) s[k] = fr.enter(m[k]);
 }
 
-// ------------------------------------------------------------------ Euler faces of orders 2 and 3, one thread per zone
+// ------------------------------------------------------------------ FP32 Euler faces, one thread per zone
 // one face side: the barycentre state (replaced by the zone average for the wave speeds when it is not physical),
 // <u> and <F>
 template <int D, int S, int NV, class R>
@@ -182,27 +182,45 @@ ADER_DEV void write_side(const StepArgs& a, long long z, const Vec<NV, R>& mean,
 }
 
 template <int D, class R>
-ADER_DEV void both_faces_o2(const FrameOf<2, 5, R>& fr, const Vec<5, typename FrameOf<2, 5, R>::S>* s, R gm1,
-                            Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa);
+ADER_DEV void both_faces_o2(const Vec<5, R>* m, R gm1, Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa);
 template <int D, class R>
-ADER_DEV void both_faces_o3(const FrameOf<3, 5, R>& fr, const Vec<5, typename FrameOf<3, 5, R>::S>* s, R gm1,
-                            Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa);
+ADER_DEV void both_faces_o3(const Vec<5, R>* m, R gm1, Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa);
 
 // the two faces of direction D (index 0 upper, 1 lower)
 template <int ORDER, int D, class R>
-ADER_DEV void both_faces(const FrameOf<ORDER, 5, R>& fr, const Vec<5, typename FrameOf<ORDER, 5, R>::S>* s, R gm1,
-                         Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
-    if constexpr (ORDER == 2) both_faces_o2<D, R>(fr, s, gm1, ub, avg, Fa);
-    else both_faces_o3<D, R>(fr, s, gm1, ub, avg, Fa);
+ADER_DEV void both_faces(const Vec<5, R>* m, R gm1, Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
+    if constexpr (ORDER == 2) both_faces_o2<D, R>(m, gm1, ub, avg, Fa);
+    else both_faces_o3<D, R>(m, gm1, ub, avg, Fa);
+}
+
+// the flux of direction D at node k of u, evaluated where a sum takes it
+template <int D, class R>
+struct FluxAt {
+    const Vec<5, R>* u;
+    R gm1;
+    ADER_DEV Vec<5, R> operator[](int k) const { return flux<D>(u[k], gm1); }
+};
+
+template <int ORDER, int D, int S, class R>
+ADER_DEV void store_face(const StepArgs& a, long long z, const Vec<5, R>* m, R gm1) {
+    using Z = ZoneOps<ORDER>;
+    Vec<5, R> p[ModeCount<ORDER>::L + 1], n[Z::FACE_NODES + 1], ub, avg;
+    to_face_frame<ORDER, D, S>(m, p);
+    Z::template face_states<false>(p, ub, avg, n);
+    write_side<D, S>(a, z, m[1], ub, avg, Z::face_mean(FluxAt<D, R>{n, gm1}), gm1);
 }
 
 template <int ORDER, int D, class R>
-ADER_DEV void store_faces(const StepArgs& a, long long z, const Vec<5, R>& mean, const FrameOf<ORDER, 5, R>& fr,
-                          const Vec<5, typename FrameOf<ORDER, 5, R>::S>* s, R gm1) {
-    Vec<5, R> ub[2], avg[2], Fa[2];
-    both_faces<ORDER, D, R>(fr, s, gm1, ub, avg, Fa);
-    write_side<D, +1>(a, z, mean, ub[0], avg[0], Fa[0], gm1);
-    write_side<D, -1>(a, z, mean, ub[1], avg[1], Fa[1], gm1);
+ADER_DEV void store_faces(const StepArgs& a, long long z, const Vec<5, R>* m, R gm1) {
+    if constexpr (ORDER == 4) {            // one at a time: fewer live values
+        store_face<ORDER, D, +1>(a, z, m, gm1);
+        store_face<ORDER, D, -1>(a, z, m, gm1);
+    } else {
+        Vec<5, R> ub[2], avg[2], Fa[2];
+        both_faces<ORDER, D, R>(m, gm1, ub, avg, Fa);
+        write_side<D, +1>(a, z, m[1], ub[0], avg[0], Fa[0], gm1);
+        write_side<D, -1>(a, z, m[1], ub[1], avg[1], Fa[1], gm1);
+    }
 }
 
 // Iteration statistics of the converged predictor: sum, maximum and capped zones.
@@ -296,14 +314,14 @@ ADER_DEV void team_predict_faces(T& t, const StepArgs& a, const double* __restri
     team_scales(t, a, dt);
     typename T::V m[L + 1];
     zone_predict<ORDER, FORM, SRC>(t, a, U, z, store, m, dt);
-    FrameOf<ORDER, T::NL, R> fr;
-    Vec<T::NL, typename FrameOf<ORDER, T::NL, R>::S> s[L + 1];
-    enter_frame<ORDER>(m, fr, s);
-    if constexpr (T::NL == 5 && ORDER <= 3) {
-        store_faces<ORDER, 0, R>(a, z, m[1], fr, s, t.gm1);
-        store_faces<ORDER, 1, R>(a, z, m[1], fr, s, t.gm1);
-        store_faces<ORDER, 2, R>(a, z, m[1], fr, s, t.gm1);
+    if constexpr (T::NL == 5 && sizeof(R) == 4) {
+        store_faces<ORDER, 0, R>(a, z, m, t.gm1);
+        store_faces<ORDER, 1, R>(a, z, m, t.gm1);
+        store_faces<ORDER, 2, R>(a, z, m, t.gm1);
     } else {
+        FrameOf<ORDER, T::NL, R> fr;
+        Vec<T::NL, typename FrameOf<ORDER, T::NL, R>::S> s[L + 1];
+        enter_frame<ORDER>(m, fr, s);
         store_faces_team<ORDER, 0>(t, a, z, store, m[1], fr, s);
         store_faces_team<ORDER, 1>(t, a, z, store, m[1], fr, s);
         store_faces_team<ORDER, 2>(t, a, z, store, m[1], fr, s);
@@ -317,13 +335,15 @@ ADER_DEV void zone_predict_faces(const StepArgs& a, const double* __restrict__ U
     team_predict_faces<ORDER, FORM, SRC>(t, a, U, z, true);
 }
 
-// Where a team of warps computes a zone: order 4 and MHD (see team.cuh), except
+// Where a team of warps computes a zone (team.cuh): FP64, order 4 and MHD, except
 //   * FP32 MHD at order 2, whose forty modes fit one thread (56^3 zones: 176 us a step against the team's 199);
 //   * the FP32 nodal form of order 4 (Euler): behind strong jumps its predicted density comes near zero at a node,
 //     which amplifies the rounding of the fluxes by up to 10^4, and the team sums them with other roundings.
+// FP32 Euler at orders 2-3 has the tiles below (third order, 128^3 zones: 0.33 ms against the team's 0.64).
 template <int ORDER, int FORM, int NV, class R>
 constexpr bool uses_team() {
-    if (sizeof(R) == 4 && ((ORDER == 2 && NV == 8) || (ORDER == 4 && NV == 5 && FORM == FORM_NODAL))) return false;
+    if (sizeof(R) == 8) return true;
+    if ((ORDER == 2 && NV == 8) || (ORDER == 4 && NV == 5 && FORM == FORM_NODAL)) return false;
     return ORDER == 4 || NV == 8;
 }
 
@@ -339,8 +359,14 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? (ORDER == 4 ? 2 : 3) : 1
 // The team kernel: a block of NV warps takes 32 zones, a warp one variable of each.
 template <int ORDER, int NV, class R>
 constexpr int team_smem() { return team_values<ORDER, NV>() * 32 * (int)sizeof(R); }
+// Blocks an SM holds: as many as registers and shared memory allow without a kilobyte of spills (FP64 Euler: five at
+// second order instead of three, 1.3% of a 96^3 step; four at third order instead of two, 3%; FP64 MHD at second order
+// four, 3%; FP32 Euler at order 4 four instead of three, 3%).
 template <int ORDER, int NV, class R>
-constexpr int team_blocks() { return sizeof(R) == 4 ? (NV == 8 ? 2 : 3) : (NV == 8 && ORDER == 4 ? 1 : 2); }
+constexpr int team_blocks() {
+    if (NV == 5) return sizeof(R) == 4 ? 4 : ORDER == 2 ? 5 : ORDER == 3 ? 4 : 2;
+    return sizeof(R) == 4 ? 2 : ORDER == 2 ? 4 : ORDER == 3 ? 2 : 1;
+}
 
 template <int ORDER, int FORM, int NV, bool SRC, class R>
 __device__ __forceinline__ void team_zone(const StepArgs& a, const double* __restrict__ U, long long z, R* sh) {
@@ -432,13 +458,6 @@ ADER_DEV void zone_flux_update(const StepArgs& a, double* out, const double* bas
     flux_difference<SOLVER, 1, NV, R>(a, z, i, j, k, gamma, gm1, acc);
     flux_difference<SOLVER, 2, NV, R>(a, z, i, j, k, gamma, gm1, acc);
     store_update<R>(a, out, base, c_host, use_dt_dev, acc, z);
-}
-
-template <int SOLVER, int NV, class R>
-__global__ void __launch_bounds__(128) k_flux_update(StepArgs a, double* out, const double* base, double c_host,
-                                                     int use_dt_dev) {
-    const long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (z < a.grid.n) zone_flux_update<SOLVER, NV, R>(a, out, base, c_host, use_dt_dev, z);
 }
 
 // ------------------------------------------------------------------ FP32 bulk: Eq. 6 without FP64 arithmetic per face
@@ -652,12 +671,11 @@ ADER_DEV void pt_side(R* dst, const Vec<5, R>& mean, Vec<5, R> ub, const Vec<5, 
 }
 
 template <int ORDER, int D, class R>
-ADER_DEV void pt_sides(R* sh, int tid, int slot_plus, int slot_minus, const Vec<5, R>& mean,
-                       const FrameOf<ORDER, 5, R>& fr, const Vec<5, typename FrameOf<ORDER, 5, R>::S>* s, R gm1) {
+ADER_DEV void pt_sides(R* sh, int tid, int slot_plus, int slot_minus, const Vec<5, R>* m, R gm1) {
     Vec<5, R> ub[2], avg[2], Fa[2];
-    both_faces<ORDER, D, R>(fr, s, gm1, ub, avg, Fa);
-    pt_side(pt_slot(sh, slot_plus, tid), mean, ub[0], avg[0], Fa[0], gm1);
-    pt_side(pt_slot(sh, slot_minus, tid), mean, ub[1], avg[1], Fa[1], gm1);
+    both_faces<ORDER, D, R>(m, gm1, ub, avg, Fa);
+    pt_side(pt_slot(sh, slot_plus, tid), m[1], ub[0], avg[0], Fa[0], gm1);
+    pt_side(pt_slot(sh, slot_minus, tid), m[1], ub[1], avg[1], Fa[1], gm1);
 }
 
 template <class R>
@@ -727,7 +745,7 @@ ADER_DEV void pt_store_flux(const StepArgs& a, long long zl, const Vec<5, R>& f)
 
 // grid: (tiles_x * tiles_y, ceil(nz / cz)); dynamic shared memory PT_SLOTS * PT_NQ * PT_THREADS values of R
 template <int ORDER, int FORM, int SOLVER, class R, bool SRC>
-__global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 3 : 1)
+__global__ void __launch_bounds__(PT_THREADS, 3)
     k_pf_tile(StepArgs a, const double* __restrict__ U, int cz) {
 
     extern __shared__ __align__(16) unsigned char pt_raw[];
@@ -756,12 +774,9 @@ __global__ void __launch_bounds__(PT_THREADS, sizeof(R) == 4 ? 3 : 1)
             SerialTeam<5, R> team;
             team_scales(team, a, dt);
             zone_predict<ORDER, FORM, SRC>(team, a, U, z, true, m, dt);
-            FrameOf<ORDER, 5, R> fr;
-            Vec<5, typename FrameOf<ORDER, 5, R>::S> s[ModeCount<ORDER>::L + 1];
-            enter_frame<ORDER>(m, fr, s);
-            pt_sides<ORDER, 0>(sh, tid, 0, 1, m[1], fr, s, gm1);
-            pt_sides<ORDER, 1>(sh, tid, 2, 3, m[1], fr, s, gm1);
-            pt_sides<ORDER, 2>(sh, tid, zp_slot, 5, m[1], fr, s, gm1);
+            pt_sides<ORDER, 0>(sh, tid, 0, 1, m, gm1);
+            pt_sides<ORDER, 1>(sh, tid, 2, 3, m, gm1);
+            pt_sides<ORDER, 2>(sh, tid, zp_slot, 5, m, gm1);
         }
         __syncthreads();
         if (valid) {
@@ -1056,12 +1071,16 @@ __global__ void __launch_bounds__(128) k_ct(StepArgs a, double* Bf, double c_hos
     if (z < a.grid.n) zone_ct<R>(a, Bf, c_host, use_dt_dev, z);
 }
 
+// where a context with tiles on takes the tile kernel
+template <int ORDER, int NV, class R>
+constexpr bool uses_tiles() { return NV == 5 && ORDER <= 3 && sizeof(R) == 4; }
+
 // One variant of the predictor + face kernel, launched over the grid.  Each variant can be compiled in a
 // translation unit of its own (the fourth-order ones are, see step_inst.cuh), which keeps the parallel
 // build's longest compile short.
 template <int ORDER, int FORM, int NV, class R, bool SRC>
 void launch_pf_variant(const StepArgs& a, const double* U, cudaStream_t st) {
-    if constexpr (NV == 5 && ORDER <= 3) {
+    if constexpr (uses_tiles<ORDER, NV, R>()) {
         if (a.tiled) {
             launch_pf_tile<ORDER, FORM, R, SRC>(a, U, st);
             return;
@@ -1085,13 +1104,13 @@ int launch_predict_faces_nv(const StepArgs& a, const double* U, cudaStream_t st)
             launch_pf_variant<ORDER, FORM_NODAL, NV, R, true>(a, U, st);
         else
             launch_pf_variant<ORDER, FORM_MODAL, NV, R, true>(a, U, st);
-        return (NV == 5 && ORDER <= 3 && a.tiled) ? 2 : 1;
+        return uses_tiles<ORDER, NV, R>() && a.tiled ? 2 : 1;
     }
     if (a.form == FORM_MODAL)
         launch_pf_variant<ORDER, FORM_MODAL, NV, R, false>(a, U, st);
     else
         launch_pf_variant<ORDER, FORM_NODAL, NV, R, false>(a, U, st);
-    return (NV == 5 && ORDER <= 3 && a.tiled) ? 2 : 1;
+    return uses_tiles<ORDER, NV, R>() && a.tiled ? 2 : 1;
 }
 
 }  // namespace ader

@@ -9,31 +9,9 @@
 namespace ader {
 namespace o2 {
 
-// The update without sources uses only tau = 0 fluxes, so one step reaches the fixed point n5
-// (in converged mode a second step confirms it).
-template <class T>
-ADER_DEV void finish_o2(const T& t, typename T::V* m, const typename T::V& n5, PredCtl& ctl) {
-    const bool conv = positive_arg(ctl.tol);
-    ctl.iters = 0;
-    ctl.capped = conv;
-    if (!conv) {
-        if (ctl.n_iter > 0) m[5] = n5;
-        ctl.iters = ctl.n_iter;
-        return;
-    }
-    using R = typename T::R;
-    const R ref = t.zone_max(max_abs(m[1])) + R(sizeof(R) == 8 ? 1e-300 : 1e-30);   // never zero in R
-    const R change = t.zone_max(max_abs_diff(n5, m[5]));
-    if (ctl.max_iter > 0) m[5] = n5;
-    if (change < R(ctl.tol) * ref || R(0) < R(ctl.tol) * ref) {
-        ctl.iters = change < R(ctl.tol) * ref ? 1 : 2;          // the second step changes nothing
-        ctl.capped = ctl.iters > ctl.max_iter;
-    }
-    if (ctl.capped) ctl.iters = ctl.max_iter;
-}
-
-// With a source the update of u5 depends on u5 through the source at the tau = 1 node, so each iteration recomputes
-// it: `next(m5)` gives the new u5 for the current one.
+// The update without sources uses only tau = 0 fluxes, so one step reaches the fixed point (in converged mode a second
+// step confirms it).  With a source the update of u5 depends on u5 through the source at the tau = 1 node, so each
+// iteration recomputes it: `next(m5)` gives the new u5 for the current one.
 template <class T, class Next>
 ADER_DEV void iterate_o2(const T& t, typename T::V* m, PredCtl& ctl, Next next) {
     using R = typename T::R;
@@ -88,7 +66,7 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         t.template sources<1>(&u7, *src, &s7);
         *sdt = s1 + 0.5 * (s7 - s1);                                                   // Eq. 35 (times dt)
     } else {
-        finish_o2(t, m, -div, ctl);
+        iterate_o2(t, m, ctl, [&](const V&) { return -div; });
     }
 }
 
@@ -116,28 +94,25 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         t.template sources<1>(&u5, *src, &s5);
         *sdt = 0.5 * (s1 + s5);                                                        // Eq. A.7 (times dt)
     } else {
-        finish_o2(t, m, d, ctl);
+        iterate_o2(t, m, ctl, [&](const V&) { return d; });
     }
 }
 
 // Eqs. 58-59 and D.3-D.5: composing D.4 with D.5, <F> is the mean of the flux
 // at the four tau = 1/2 facial nodes (node 5 enters only through the time mode).
-template <int D, int NV, class R, class FR>
-ADER_DEV void face(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>& ub, Vec<NV, R>& avg,
-                   Vec<NV, R>& Fa) {
-    using V = Vec<NV, typename FR::S>;
-    const V q1 = p[1] + 0.5 * (p[2] + p[5]), h3 = 0.5 * p[3], h4 = 0.5 * p[4];
-    ub = fr.leave(q1);
+template <int D, class R>
+ADER_DEV void face(const Vec<5, R>* p, R gm1, Vec<5, R>& ub, Vec<5, R>& avg, Vec<5, R>& Fa) {
+    ub = p[1] + 0.5 * (p[2] + p[5]);
     avg = ub;
     FluxSum<D, R> sum;
-    sum.add(fr.leave(q1 + h3));
-    sum.add(fr.leave(q1 - h3));
-    sum.add(fr.leave(q1 + h4));
-    sum.add(fr.leave(q1 - h4));
+    sum.add(ub + 0.5 * p[3]);
+    sum.add(ub - 0.5 * p[3]);
+    sum.add(ub + 0.5 * p[4]);
+    sum.add(ub - 0.5 * p[4]);
     Fa = sum.mean(avg, gm1, R(0.25));
 }
 
-// MHD: the states of a face and its five nodes (Eqs. 58-59, D.3), and the mean of the flux at the first four.
+// The states of a face and its five nodes (Eqs. 58-59, D.3), and the mean of the flux at the first four.
 template <bool ALL, class V>
 ADER_DEV void face_states(const V* p, V& ub, V& avg, V* t) {
     ub = p[1] + 0.5 * (p[2] + p[5]);
@@ -150,8 +125,8 @@ ADER_DEV void face_states(const V* p, V& ub, V& avg, V* t) {
 }
 constexpr int FACE_NODES = 5, MEAN_NODES = 4;
 ADER_DEV constexpr int mean_node(int k) { return k + 1; }
-template <class V>
-ADER_DEV V face_mean(const V* F) {
+template <class F_>
+ADER_DEV auto face_mean(const F_& F) {
     return 0.25 * (F[1] + F[2] + F[3] + F[4]);
 }
 

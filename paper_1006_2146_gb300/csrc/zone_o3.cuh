@@ -64,30 +64,51 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
 #pragma unroll
         for (int k = 1; k <= 13; ++k) u[k] = fr.leave(s[k]);
     }
-    // fluxes at the tau = 0 nodes, built once (Sec. IV.2)
-    V f[14], g[14], h[14];
-    t.template fluxes<13, 0, false>(u + 1, f + 1, g + 1, h + 1);
-    // Eqs. 40-42, tau = 0 modes
-    const V q1 = f[2] + f[3] + f[4] + f[5], q2 = f[6] + f[7] + f[8] + f[9], q3 = f[10] + f[11] + f[12] + f[13];
-    const V F2 = scale(cx, 0.25 * (q1 - q2));
-    const V F5 = scale(cx, 0.5 * (q1 + q2 - q3) - 2.0 * f[1]);
-    const V F8 = scale(cx, f[2] - f[3] - f[6] + f[7]);
-    const V F10 = scale(cx, f[4] - f[5] - f[8] + f[9]);
-    const V q4 = g[2] + g[6] + g[10] + g[12], q5 = g[3] + g[7] + g[11] + g[13], q6 = g[4] + g[5] + g[8] + g[9];
-    const V G3 = scale(cy, 0.25 * (q4 - q5));
-    const V G6 = scale(cy, 0.5 * (q4 + q5 - q6) - 2.0 * g[1]);
-    const V G8 = scale(cy, g[2] - g[3] - g[6] + g[7]);
-    const V G9 = scale(cy, g[10] - g[11] - g[12] + g[13]);
-    const V q7 = h[4] + h[8] + h[10] + h[11], q8 = h[5] + h[9] + h[12] + h[13], q9 = h[2] + h[3] + h[6] + h[7];
-    const V H4 = scale(cz, 0.25 * (q7 - q8));
-    const V H7 = scale(cz, 0.5 * (q7 + q8 - q9) - 2.0 * h[1]);
-    const V H9 = scale(cz, h[10] - h[11] - h[12] + h[13]);
-    const V H10 = scale(cz, h[4] - h[5] - h[8] + h[9]);
-    // Eq. 36 without sources: the modes fed by tau = 0 fluxes alone
-    const V e11 = -(F2 + G3 + H4);
-    const V e13 = -(2.0 * F5 + G8 + H10);
-    const V e14 = -(F8 + 2.0 * G6 + H9);
-    const V e15 = -(F10 + G9 + 2.0 * H7);
+    // fluxes at the tau = 0 nodes, built once (Sec. IV.2); the sums of Eqs. 40-42 and 36 in the state scalar (up to
+    // 32 times a flux)
+    V e11, e13, e14, e15;       // Eq. 36 without sources: the modes fed by tau = 0 fluxes alone
+    {
+        using FF = typename FrameAt<2, NL, R>::T;
+        using VF = Vec<NL, typename FF::S>;
+        V fn[14], gn[14], hn[14];
+        t.template fluxes<13, 0, false>(u + 1, fn + 1, gn + 1, hn + 1);
+        FF ff;
+        VF f[14], g[14], h[14];
+#pragma unroll
+        for (int n = 1; n <= 13; ++n) {
+            ff.include(fn[n]);
+            ff.include(gn[n]);
+            ff.include(hn[n]);
+        }
+        ff.close();
+#pragma unroll
+        for (int n = 1; n <= 13; ++n) {
+            f[n] = ff.enter(fn[n]);
+            g[n] = ff.enter(gn[n]);
+            h[n] = ff.enter(hn[n]);
+        }
+        const AxisScale<FF> c(cx, cy, cz);
+        const FF fo = c.out(ff);
+        const VF q1 = f[2] + f[3] + f[4] + f[5], q2 = f[6] + f[7] + f[8] + f[9], q3 = f[10] + f[11] + f[12] + f[13];
+        const VF F2 = c.template times<0>(0.25 * (q1 - q2));
+        const VF F5 = c.template times<0>(0.5 * (q1 + q2 - q3) - 2.0 * f[1]);
+        const VF F8 = c.template times<0>(f[2] - f[3] - f[6] + f[7]);
+        const VF F10 = c.template times<0>(f[4] - f[5] - f[8] + f[9]);
+        const VF q4 = g[2] + g[6] + g[10] + g[12], q5 = g[3] + g[7] + g[11] + g[13], q6 = g[4] + g[5] + g[8] + g[9];
+        const VF G3 = c.template times<1>(0.25 * (q4 - q5));
+        const VF G6 = c.template times<1>(0.5 * (q4 + q5 - q6) - 2.0 * g[1]);
+        const VF G8 = c.template times<1>(g[2] - g[3] - g[6] + g[7]);
+        const VF G9 = c.template times<1>(g[10] - g[11] - g[12] + g[13]);
+        const VF q7 = h[4] + h[8] + h[10] + h[11], q8 = h[5] + h[9] + h[12] + h[13], q9 = h[2] + h[3] + h[6] + h[7];
+        const VF H4 = c.template times<2>(0.25 * (q7 - q8));
+        const VF H7 = c.template times<2>(0.5 * (q7 + q8 - q9) - 2.0 * h[1]);
+        const VF H9 = c.template times<2>(h[10] - h[11] - h[12] + h[13]);
+        const VF H10 = c.template times<2>(h[4] - h[5] - h[8] + h[9]);
+        e11 = fo.leave(-(F2 + G3 + H4));
+        e13 = fo.leave(-(2.0 * F5 + G8 + H10));
+        e14 = fo.leave(-(F8 + 2.0 * G6 + H9));
+        e15 = fo.leave(-(F10 + G9 + 2.0 * H7));
+    }
     // source modes from the tau = 0 nodes (Eqs. 40-43 with f, g, h -> s), built once
     V S1, S2, S3, S4, s1;
     if constexpr (SRC) {
@@ -217,26 +238,42 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
     // (1.5 f1 - f2 - f3 / 2 = -A and f2 + f3 - 2 f1 = A + X / 2), for y and z the same with the axes exchanged.
     V q11, q12, q13, q14, q15;
     {
-        const R hx = R(0.5) * cx, hy = R(0.5) * cy, hz = R(0.5) * cz;
-        // all directions at nodes 1, 2, 4, 6, 8, 9, 10; x alone at 3, y at 5, z at 7
+        // all directions at nodes 1, 2, 4, 6, 8, 9, 10; x alone at 3, y at 5, z at 7; the sums in the state scalar
+        using FF = typename FrameAt<2, NL, R>::T;
+        using VF = Vec<NL, typename FF::S>;
         const V un[10] = {u[1], u[2], u[4], u[6], u[8], u[9], u[10], u[3], u[5], u[7]};
-        V f[8], g[8], h[8];
-        t.template fluxes<7, 1, false>(un, f, g, h);
-        const V X = f[7] - f[0], Y = g[7] - g[0], Z = h[7] - h[0];
-        V ax = f[1] - f[0], ay = g[2] - g[0], az = h[3] - h[0];
-        const V half = scale(hx, X) + scale(hy, Y) + scale(hz, Z);
-        q11 = u[1] + half;
+        V fn[8], gn[8], hn[8];
+        t.template fluxes<7, 1, false>(un, fn, gn, hn);
+        FF ff;
+        VF f[8], g[8], h[8];
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            if (n != 4) ff.include(fn[n]);
+            if (n != 5) ff.include(gn[n]);
+            if (n != 6) ff.include(hn[n]);
+        }
+        ff.close();
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            if (n != 4) f[n] = ff.enter(fn[n]);
+            if (n != 5) g[n] = ff.enter(gn[n]);
+            if (n != 6) h[n] = ff.enter(hn[n]);
+        }
+        const AxisScale<FF> c(cx, cy, cz);
+        const FF fo = c.out(ff);
+        const VF X = c.template times<0>(f[7] - f[0]), Y = c.template times<1>(g[7] - g[0]);
+        const VF Z = c.template times<2>(h[7] - h[0]), half = 0.5 * (X + Y + Z);
+        const VF ax = c.template times<0>(f[1] - f[0]) + 0.5 * X, ay = c.template times<1>(g[2] - g[0]) + 0.5 * Y;
+        const VF az = c.template times<2>(h[3] - h[0]) + 0.5 * Z;
         // the mixed differences of q12, q13, q14
-        const V d12 = scale(cy, g[1] - g[6]) + scale(cz, h[1] - h[5]);
-        const V d13 = scale(cx, f[2] - f[6]) + scale(cz, h[2] - h[4]);
-        const V d14 = scale(cx, f[3] - f[5]) + scale(cy, g[3] - g[4]);
-        ax = scale(cx, ax + 0.5 * X);
-        ay = scale(cy, ay + 0.5 * Y);
-        az = scale(cz, az + 0.5 * Z);
-        q12 = u[2] + (d12 + (ay + az - ax));
-        q13 = u[4] + (d13 + (ax + az - ay));
-        q14 = u[6] + (d14 + (ax + ay - az));
-        q15 = u[1] + (half + (ax + ay + az));   // u1 + sum_d c_d (A + X / 2)
+        const VF d12 = c.template times<1>(g[1] - g[6]) + c.template times<2>(h[1] - h[5]);
+        const VF d13 = c.template times<0>(f[2] - f[6]) + c.template times<2>(h[2] - h[4]);
+        const VF d14 = c.template times<0>(f[3] - f[5]) + c.template times<1>(g[3] - g[4]);
+        q11 = u[1] + fo.leave(half);
+        q12 = u[2] + fo.leave(d12 + (ay + az - ax));
+        q13 = u[4] + fo.leave(d13 + (ax + az - ay));
+        q14 = u[6] + fo.leave(d14 + (ax + ay - az));
+        q15 = u[1] + fo.leave(half + (ax + ay + az));   // u1 + sum_d c_d (A + X / 2)
     }
     V s0sum, s1;         // with a source: s2 + ... + s7 and s1 (nodes 1-7, built once)
     if constexpr (SRC) {          // Eq. B.2, source terms
@@ -311,11 +348,20 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
     ctl.capped = conv && !done;
     if (!conv) {
         // Eq. B.5: nodal -> modal
-        m[12] = 2.0 * (u15 - 2.0 * u11 + u[1]);
-        m[11] = 2.0 * (u11 - u[1] - 0.25 * m[12]);
-        m[13] = 4.0 * (u12 - u11 - u[2] + u[1]);
-        m[14] = 4.0 * (u13 - u11 - u[4] + u[1]);
-        m[15] = 4.0 * (u14 - u11 - u[6] + u[1]);
+        FR fm;
+        const V in[9] = {u[1], u[2], u[4], u[6], u11, u12, u13, u14, u15};
+        VS s[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) fm.include(in[k]);
+        fm.close();
+#pragma unroll
+        for (int k = 0; k < 9; ++k) s[k] = fm.enter(in[k]);
+        const VS n12 = 2.0 * (s[8] - 2.0 * s[4] + s[0]);
+        m[12] = fm.leave(n12);
+        m[11] = fm.leave(2.0 * (s[4] - s[0] - 0.25 * n12));
+        m[13] = fm.leave(4.0 * (s[5] - s[4] - s[1] + s[0]));
+        m[14] = fm.leave(4.0 * (s[6] - s[4] - s[2] + s[0]));
+        m[15] = fm.leave(4.0 * (s[7] - s[4] - s[3] + s[0]));
     }
     if constexpr (SRC)            // Eq. B.6 from the source at the final iterate (times dt)
     {
@@ -326,72 +372,66 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
     }
 }
 
-
 // ------------------------------------------------------------------ x+ face, Sec. V.2 and App. D
-// p = the zone's modes in the face's x-frame (modes.cuh), in the state scalar of the frame fr (fixed.cuh).
-// Outputs the
-// barycentre state (Eq. 61), the face average of u (Eq. 62) and the face
-// average of the physical normal flux: composing Eq. D.9 with D.10 gives
-// <F> = (F1 + F6 + F7 + F8 + F9 + F10) / 6 over the facial nodes of Eq. D.6
-// (the four corner nodes enter only the edge averages).
-// Both x-faces of one direction at once (Euler).  p is the zone's modes in
-// the frame of the upper face; the lower face's frame differs only in the
-// sign of the modes odd in the normal coordinate (2, 8, 10, 13), so each of
-// the node states of Eq. D.8 is E + O on the upper face and E - O on the lower one,
-// with E its part from the even modes and O from the odd ones, each computed once; the
-// nodes are taken in an order that keeps few of them alive at a time.
+// p = the zone's modes in the face's x-frame (modes.cuh).  The barycentre state (Eq. 61), the face average of u
+// (Eq. 62) and the face average of the physical normal flux: composing Eq. D.9 with D.10 gives
+// <F> = (F1 + F6 + F7 + F8 + F9 + F10) / 6 over the facial nodes of Eq. D.6 (the four corner nodes enter only the
+// edge averages).
+// Both x-faces of one direction at once (FP32 Euler).  p is in the frame of the upper face; the lower face's frame
+// differs only in the sign of the modes odd in the normal coordinate (2, 8, 10, 13), so each of the node states of
+// Eq. D.8 is E + O on the upper face and E - O on the lower one, with E its part from the even modes and O from the
+// odd ones, each computed once; the nodes are taken in an order that keeps few of them alive at a time.
 // Index 0 of ub, avg, Fa is the upper face (S = +1), index 1 the lower.
-template <int D, int NV, class R, class FR>
-ADER_DEV void face_pair(const FR& fr, const Vec<NV, typename FR::S>* p, R gm1, Vec<NV, R>* ub, Vec<NV, R>* avg,
-                        Vec<NV, R>* Fa) {
-    using V = Vec<NV, typename FR::S>;
+template <int D, class R>
+ADER_DEV void face_pair(const Vec<5, R>* p, R gm1, Vec<5, R>* ub, Vec<5, R>* avg, Vec<5, R>* Fa) {
+    using V = Vec<5, R>;
     const V t1e = p[1] + (2.0 * p[5] - p[6] - p[7]) / 12.0, t1o = 0.5 * p[2];
     const V q1e = 0.5 * p[11] + 0.25 * p[12], q1o = 0.25 * p[13];
     {
         const V ube = t1e + q1e, ubo = t1o + q1o;
         const V avge = ube + (p[6] + p[7] + p[12]) / 12.0;
-        ub[0] = fr.leave(ube + ubo);
-        ub[1] = fr.leave(ube - ubo);
-        avg[0] = fr.leave(avge + ubo);
-        avg[1] = fr.leave(avge - ubo);
+        ub[0] = ube + ubo;
+        ub[1] = ube - ubo;
+        avg[0] = avge + ubo;
+        avg[1] = avge - ubo;
     }
     FluxSum<D, R> up, lo;
-    up.add(fr.leave(t1e + t1o));                                                        // node 1
-    lo.add(fr.leave(t1e - t1o));
+    up.add(t1e + t1o);                                                        // node 1
+    lo.add(t1e - t1o);
     {
         const V e = t1e + p[11] + p[12], o = t1o + 0.5 * p[13];                   // node 10
-        up.add(fr.leave(e + o));
-        lo.add(fr.leave(e - o));
+        up.add(e + o);
+        lo.add(e - o);
     }
     const V t2e = t1e + 0.5 * (p[3] + p[4]) + 0.25 * (p[6] + p[7] + p[9]), t2o = t1o + 0.25 * (p[8] + p[10]);
     const V t3e = t2e - p[3] - 0.5 * p[9], t3o = t2o - 0.5 * p[8];
     const V t4e = t2e - p[4] - 0.5 * p[9], t4o = t2o - 0.5 * p[10];
     {
         const V e = 0.5 * (t2e + t4e) + q1e + 0.25 * (p[14] - p[7]), o = 0.5 * (t2o + t4o) + q1o;   // 6
-        up.add(fr.leave(e + o));
-        lo.add(fr.leave(e - o));
+        up.add(e + o);
+        lo.add(e - o);
     }
     {
         const V e = 0.5 * (t2e + t3e) + q1e + 0.25 * (p[15] - p[6]), o = 0.5 * (t2o + t3o) + q1o;   // 8
-        up.add(fr.leave(e + o));
-        lo.add(fr.leave(e - o));
+        up.add(e + o);
+        lo.add(e - o);
     }
     const V t5e = t4e - p[3] + 0.5 * p[9], t5o = t4o - 0.5 * p[8];
     {
         const V e = 0.5 * (t4e + t5e) + q1e - 0.25 * (p[6] + p[15]), o = 0.5 * (t4o + t5o) + q1o;   // 9
-        up.add(fr.leave(e + o));
-        lo.add(fr.leave(e - o));
+        up.add(e + o);
+        lo.add(e - o);
     }
     {
         const V e = 0.5 * (t3e + t5e) + q1e - 0.25 * (p[7] + p[14]), o = 0.5 * (t3o + t5o) + q1o;   // 7
-        up.add(fr.leave(e + o));
-        lo.add(fr.leave(e - o));
+        up.add(e + o);
+        lo.add(e - o);
     }
     Fa[0] = up.mean(avg[0], gm1, R(1.0 / 6.0));
     Fa[1] = lo.mean(avg[1], gm1, R(1.0 / 6.0));
 }
 
-// One face at a time (MHD): the barycentre state, the face average and all ten facial nodes of Eq. D.6 (Eq. D.8).
+// One face at a time: the barycentre state, the face average and all ten facial nodes of Eq. D.6 (Eq. D.8).
 template <bool ALL, class V>
 ADER_DEV void face_states(const V* p, V& ub, V& avg, V* t) {
     ub = p[1] + 0.5 * (p[2] + p[11]) + 0.25 * (p[12] + p[13]) + (2.0 * p[5] - p[6] - p[7]) / 12.0;
@@ -413,8 +453,8 @@ ADER_DEV void face_states(const V* p, V& ub, V& avg, V* t) {
 // the edge averages)
 constexpr int FACE_NODES = 10, MEAN_NODES = 6;
 ADER_DEV constexpr int mean_node(int k) { return k == 0 ? 1 : k + 5; }
-template <class V>
-ADER_DEV V face_mean(const V* F) {
+template <class F_>
+ADER_DEV auto face_mean(const F_& F) {
     return (F[1] + F[6] + F[7] + F[8] + F[9] + F[10]) / 6.0;
 }
 

@@ -57,19 +57,37 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         s[21] = s[19] + s[20] - s[18] + w[9] - 0.5 * w[20];
     }
 
-    // tau = 0 parts of Eqs. 49-51 (built once)
-    V F2, F5, F8, F10, F11, F20, PF14, PF15, PF16, QF12;
-    V G3, G6, G8, G9, G12, G20, PG14, PG15, PG16, QG34;
-    V H4, H7, H9, H10, H13, H20, PH14, PH15, PH16, QH56;
+    // tau = 0 parts of Eqs. 49-51 (built once), in the state scalar: sums of up to 110 fluxes
+    using FF = typename FrameAt<2, NL, R>::T;
+    using VF = Vec<NL, typename FF::S>;
+    const AxisScale<FF> c(cx, cy, cz);
+    FF ff;
+    VF F2, F5, F8, F10, F11, F20, PF14, PF15, PF16, QF12;
+    VF G3, G6, G8, G9, G12, G20, PG14, PG15, PG16, QG34;
+    VF H4, H7, H9, H10, H13, H20, PH14, PH15, PH16, QH56;
     {
-        V u[22], f[22], g[22], h[22];
+        V u[22], fn[22], gn[22], hn[22];
+        VF f[22], g[22], h[22];
 #pragma unroll
         for (int k = 1; k <= 21; ++k) u[k] = fr.leave(s[k]);
-        t.template fluxes<21, 0, false>(u + 1, f + 1, g + 1, h + 1);
+        t.template fluxes<21, 0, false>(u + 1, fn + 1, gn + 1, hn + 1);
+#pragma unroll
+        for (int k = 1; k <= 21; ++k) {
+            ff.include(fn[k]);
+            ff.include(gn[k]);
+            ff.include(hn[k]);
+        }
+        ff.close();
+#pragma unroll
+        for (int k = 1; k <= 21; ++k) {
+            f[k] = ff.enter(fn[k]);
+            g[k] = ff.enter(gn[k]);
+            h[k] = ff.enter(hn[k]);
+        }
         // q1..q6 of Eqs. 49-51 (corner sums), per flux
-        const V fq1 = f[14] + f[15] + f[16] + f[17], fq2 = f[18] + f[19] + f[20] + f[21];
-        const V fq3 = f[14] + f[16] + f[18] + f[20], fq4 = f[15] + f[17] + f[19] + f[21];
-        const V fq5 = f[14] + f[15] + f[18] + f[19], fq6 = f[16] + f[17] + f[20] + f[21];
+        const VF fq1 = f[14] + f[15] + f[16] + f[17], fq2 = f[18] + f[19] + f[20] + f[21];
+        const VF fq3 = f[14] + f[16] + f[18] + f[20], fq4 = f[15] + f[17] + f[19] + f[21];
+        const VF fq5 = f[14] + f[15] + f[18] + f[19], fq6 = f[16] + f[17] + f[20] + f[21];
         F5 = 2.0 * (f[2] - 2.0 * f[1] + f[5]);
         F8 = 0.5 * (f[14] - f[15] + f[16] - f[17] - f[18] + f[19] - f[20] + f[21]);
         F10 = 0.5 * (f[14] + f[15] - f[16] - f[17] - f[18] - f[19] + f[20] + f[21]);
@@ -80,9 +98,9 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         PF15 = 0.5 * (fq5 - fq6) - 2.0 * (f[10] - f[13]);
         PF16 = 0.5 * (fq1 - fq2) - 2.0 * (f[2] - f[5]);
         QF12 = fq1 - fq2;
-        const V gq1 = g[14] + g[15] + g[16] + g[17], gq2 = g[18] + g[19] + g[20] + g[21];
-        const V gq3 = g[14] + g[16] + g[18] + g[20], gq4 = g[15] + g[17] + g[19] + g[21];
-        const V gq5 = g[14] + g[15] + g[18] + g[19], gq6 = g[16] + g[17] + g[20] + g[21];
+        const VF gq1 = g[14] + g[15] + g[16] + g[17], gq2 = g[18] + g[19] + g[20] + g[21];
+        const VF gq3 = g[14] + g[16] + g[18] + g[20], gq4 = g[15] + g[17] + g[19] + g[21];
+        const VF gq5 = g[14] + g[15] + g[18] + g[19], gq6 = g[16] + g[17] + g[20] + g[21];
         G6 = 2.0 * (g[6] - 2.0 * g[1] + g[9]);
         G8 = 0.5 * (g[14] - g[15] + g[16] - g[17] - g[18] + g[19] - g[20] + g[21]);
         G9 = 0.5 * (g[14] - g[15] - g[16] + g[17] + g[18] - g[19] - g[20] + g[21]);
@@ -93,9 +111,9 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         PG15 = 0.5 * (gq5 - gq6) - 2.0 * (g[10] - g[13]);
         PG16 = 0.5 * (gq1 - gq2) - 2.0 * (g[2] - g[5]);
         QG34 = gq3 - gq4;
-        const V hq1 = h[14] + h[15] + h[16] + h[17], hq2 = h[18] + h[19] + h[20] + h[21];
-        const V hq3 = h[14] + h[16] + h[18] + h[20], hq4 = h[15] + h[17] + h[19] + h[21];
-        const V hq5 = h[14] + h[15] + h[18] + h[19], hq6 = h[16] + h[17] + h[20] + h[21];
+        const VF hq1 = h[14] + h[15] + h[16] + h[17], hq2 = h[18] + h[19] + h[20] + h[21];
+        const VF hq3 = h[14] + h[16] + h[18] + h[20], hq4 = h[15] + h[17] + h[19] + h[21];
+        const VF hq5 = h[14] + h[15] + h[18] + h[19], hq6 = h[16] + h[17] + h[20] + h[21];
         H7 = 2.0 * (h[10] - 2.0 * h[1] + h[13]);
         H9 = 0.5 * (h[14] - h[15] - h[16] + h[17] + h[18] - h[19] - h[20] + h[21]);
         H10 = 0.5 * (h[14] + h[15] - h[16] - h[17] - h[18] - h[19] + h[20] + h[21]);
@@ -217,10 +235,11 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         for (int k = 23; k <= (SRC ? 42 : 41); ++k) out[k] = fw.leave(x[k]);
     };
     // Eq. 45 without sources: the modes fed by tau = 0 fluxes only
-    const V e21 = -(scale(cx, F2 + 0.1 * F11) + scale(cy, G3 + 0.1 * G12) + scale(cz, H4 + 0.1 * H13));
-    const V e24 = -(scale(cx, 2.0 * F5) + scale(cy, G8) + scale(cz, H10));
-    const V e25 = -(scale(cx, F8) + scale(cy, 2.0 * G6) + scale(cz, H9));
-    const V e26 = -(scale(cx, F10) + scale(cy, G9) + scale(cz, 2.0 * H7));
+    const FF fo = c.out(ff);
+    const V e21 = fo.leave(-(c.template times<0>(F2 + 0.1 * F11) + c.template times<1>(G3 + 0.1 * G12) + c.template times<2>(H4 + 0.1 * H13)));
+    const V e24 = fo.leave(-(c.template times<0>(2.0 * F5) + c.template times<1>(G8) + c.template times<2>(H10)));
+    const V e25 = fo.leave(-(c.template times<0>(F8) + c.template times<1>(2.0 * G6) + c.template times<2>(H9)));
+    const V e26 = fo.leave(-(c.template times<0>(F10) + c.template times<1>(G9) + c.template times<2>(2.0 * H7)));
 
     const bool conv = positive_arg(ctl.tol);
     const int cap = conv ? ctl.max_iter : ctl.n_iter;
@@ -232,80 +251,98 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         V w[43];
         build_w(w);
         // fluxes at nodes 23..35 (all three directions) and the axis nodes 36..41
-        V f[38], g[38], h[38];
-        t.template fluxes<13, 2, false>(w + 23, f + 23, g + 23, h + 23);
-        const V f36 = f[36], f37 = f[37], g38 = g[36], g39 = g[37], h40 = h[36], h41 = h[37];
+        V fn[38], gn[38], hn[38];
+        t.template fluxes<13, 2, false>(w + 23, fn + 23, gn + 23, hn + 23);
+        FF fi;
+        VF f[38], g[38], h[38];
+#pragma unroll
+        for (int k = 23; k <= 37; ++k) {
+            fi.include(fn[k]);
+            fi.include(gn[k]);
+            fi.include(hn[k]);
+        }
+        fi.close();
+        fi.join(ff);
+#pragma unroll
+        for (int k = 23; k <= 37; ++k) {
+            f[k] = fi.enter(fn[k]);
+            g[k] = fi.enter(gn[k]);
+            h[k] = fi.enter(hn[k]);
+        }
+        const FF fio = c.out(fi);
+        auto keep = [&](const VF& x) { return fi.from(ff, x); };      // a tau = 0 part in this iterate's frame
+        const VF f36 = f[36], f37 = f[37], g38 = g[36], g39 = g[37], h40 = h[36], h41 = h[37];
         // Eq. 49 (x)
-        V F14, F15, F16, F18, F24, F27, F30, F33, F35;
+        VF F14, F15, F16, F18, F24, F27, F30, F33, F35;
         {
-            const V q7 = f[23] + f[24] - f[25] - f[26] - f[27] - f[28] + f[29] + f[30];
-            const V q8 = f[23] + f[27] - f[24] - f[28] - f[31] - f[33] + f[32] + f[34];
-            const V q9 = f[25] + f[29] - f[26] - f[30] - f[31] - f[32] + f[33] + f[34];
-            const V q10 = f[23] + f[24] + f[25] + f[26] - f[27] - f[28] - f[29] - f[30];
-            F14 = q8 + PF14;
-            F15 = q9 + PF15;
-            F16 = q7 + PF16;
+            const VF q7 = f[23] + f[24] - f[25] - f[26] - f[27] - f[28] + f[29] + f[30];
+            const VF q8 = f[23] + f[27] - f[24] - f[28] - f[31] - f[33] + f[32] + f[34];
+            const VF q9 = f[25] + f[29] - f[26] - f[30] - f[31] - f[32] + f[33] + f[34];
+            const VF q10 = f[23] + f[24] + f[25] + f[26] - f[27] - f[28] - f[29] - f[30];
+            F14 = q8 + keep(PF14);
+            F15 = q9 + keep(PF15);
+            F16 = q7 + keep(PF16);
             F18 = -2.0 * q7 + F16;
-            F27 = 1.125 * QF12 + 4.5 * (f36 - f37) - 2.25 * q10;
+            F27 = 1.125 * keep(QF12) + 4.5 * (f36 - f37) - 2.25 * q10;
             F24 = 3.0 * (f36 - f37) - 0.75 * q10 + 0.375 * (F16 + F18) - F27;
-            F30 = 3.0 * (f36 - 2.0 * f[35] + f37) - 1.5 * F5;
-            F33 = 3.0 * (f[23] - f[27] - f[24] + f[28]) - 3.0 * F8;
-            F35 = 3.0 * (f[25] - f[29] - f[26] + f[30]) - 3.0 * F10;
+            F30 = 3.0 * (f36 - 2.0 * f[35] + f37) - 1.5 * keep(F5);
+            F33 = 3.0 * (f[23] - f[27] - f[24] + f[28]) - 3.0 * keep(F8);
+            F35 = 3.0 * (f[25] - f[29] - f[26] + f[30]) - 3.0 * keep(F10);
         }
         // Eq. 50 (y)
-        V G14, G16, G17, G19, G25, G28, G31, G33, G34;
+        VF G14, G16, G17, G19, G25, G28, G31, G33, G34;
         {
-            const V q7 = g[23] + g[24] - g[25] - g[26] - g[27] - g[28] + g[29] + g[30];
-            const V q8 = g[23] + g[27] - g[24] - g[28] - g[31] - g[33] + g[32] + g[34];
-            const V q9 = g[25] + g[29] - g[26] - g[30] - g[31] - g[32] + g[33] + g[34];
-            const V q11 = g[23] - g[24] + g[27] - g[28] + g[31] - g[32] + g[33] - g[34];
-            G14 = q8 + PG14;
-            const V G15 = q9 + PG15;
-            G16 = q7 + PG16;
+            const VF q7 = g[23] + g[24] - g[25] - g[26] - g[27] - g[28] + g[29] + g[30];
+            const VF q8 = g[23] + g[27] - g[24] - g[28] - g[31] - g[33] + g[32] + g[34];
+            const VF q9 = g[25] + g[29] - g[26] - g[30] - g[31] - g[32] + g[33] + g[34];
+            const VF q11 = g[23] - g[24] + g[27] - g[28] + g[31] - g[32] + g[33] - g[34];
+            G14 = q8 + keep(PG14);
+            const VF G15 = q9 + keep(PG15);
+            G16 = q7 + keep(PG16);
             G17 = -2.0 * q9 + G15;
             G19 = -2.0 * q8 + G14;
-            G28 = 1.125 * QG34 + 4.5 * (g38 - g39) - 2.25 * q11;
+            G28 = 1.125 * keep(QG34) + 4.5 * (g38 - g39) - 2.25 * q11;
             G25 = 3.0 * (g38 - g39) - 0.75 * q11 + 0.375 * (G14 + G19) - G28;
-            G31 = 3.0 * (g38 - 2.0 * g[35] + g39) - 1.5 * G6;
-            G33 = 3.0 * (g[23] - g[27] - g[24] + g[28]) - 3.0 * G8;
-            G34 = 3.0 * (g[31] - g[32] - g[33] + g[34]) - 3.0 * G9;
+            G31 = 3.0 * (g38 - 2.0 * g[35] + g39) - 1.5 * keep(G6);
+            G33 = 3.0 * (g[23] - g[27] - g[24] + g[28]) - 3.0 * keep(G8);
+            G34 = 3.0 * (g[31] - g[32] - g[33] + g[34]) - 3.0 * keep(G9);
         }
         // Eq. 51 (z)
-        V H15, H17, H18, H19, H26, H29, H32, H34, H35;
+        VF H15, H17, H18, H19, H26, H29, H32, H34, H35;
         {
-            const V q7 = h[23] + h[24] - h[25] - h[26] - h[27] - h[28] + h[29] + h[30];
-            const V q8 = h[23] + h[27] - h[24] - h[28] - h[31] - h[33] + h[32] + h[34];
-            const V q9 = h[25] + h[29] - h[26] - h[30] - h[31] - h[32] + h[33] + h[34];
-            const V q12 = h[25] - h[26] + h[29] - h[30] + h[31] + h[32] - h[33] - h[34];
-            const V H14 = q8 + PH14;
-            H15 = q9 + PH15;
-            const V H16 = q7 + PH16;
+            const VF q7 = h[23] + h[24] - h[25] - h[26] - h[27] - h[28] + h[29] + h[30];
+            const VF q8 = h[23] + h[27] - h[24] - h[28] - h[31] - h[33] + h[32] + h[34];
+            const VF q9 = h[25] + h[29] - h[26] - h[30] - h[31] - h[32] + h[33] + h[34];
+            const VF q12 = h[25] - h[26] + h[29] - h[30] + h[31] + h[32] - h[33] - h[34];
+            const VF H14 = q8 + keep(PH14);
+            H15 = q9 + keep(PH15);
+            const VF H16 = q7 + keep(PH16);
             H17 = -2.0 * q9 + H15;
             H18 = -2.0 * q7 + H16;
             H19 = -2.0 * q8 + H14;
-            H29 = 1.125 * QH56 + 4.5 * (h40 - h41) - 2.25 * q12;
+            H29 = 1.125 * keep(QH56) + 4.5 * (h40 - h41) - 2.25 * q12;
             H26 = 3.0 * (h40 - h41) - 0.75 * q12 + 0.375 * (H15 + H17) - H29;
-            H32 = 3.0 * (h40 - 2.0 * h[35] + h41) - 1.5 * H7;
-            H34 = 3.0 * (h[31] - h[32] - h[33] + h[34]) - 3.0 * H9;
-            H35 = 3.0 * (h[25] - h[26] - h[29] + h[30]) - 3.0 * H10;
+            H32 = 3.0 * (h40 - 2.0 * h[35] + h41) - 1.5 * keep(H7);
+            H34 = 3.0 * (h[31] - h[32] - h[33] + h[34]) - 3.0 * keep(H9);
+            H35 = 3.0 * (h[25] - h[26] - h[29] + h[30]) - 3.0 * keep(H10);
         }
         // Eq. 45 without sources
         V n[16];
         n[0] = e21;
-        n[1] = -0.5 * (scale(cx, F24) + scale(cy, G25) + scale(cz, H26));
-        n[2] = -(1.0 / 3.0) * (scale(cx, F27) + scale(cy, G28) + scale(cz, H29));
+        n[1] = fio.leave(-0.5 * (c.template times<0>(F24) + c.template times<1>(G25) + c.template times<2>(H26)));
+        n[2] = fio.leave(-(1.0 / 3.0) * (c.template times<0>(F27) + c.template times<1>(G28) + c.template times<2>(H29)));
         n[3] = e24;
         n[4] = e25;
         n[5] = e26;
-        n[6] = -(scale(cx, F30) + scale(cy, 0.5 * G33) + scale(cz, 0.5 * H35));
-        n[7] = -(scale(cx, 0.5 * F33) + scale(cy, G31) + scale(cz, 0.5 * H34));
-        n[8] = -(scale(cx, 0.5 * F35) + scale(cy, 0.5 * G34) + scale(cz, H32));
-        n[9] = -(scale(cx, 3.0 * F11) + scale(cy, G14) + scale(cz, H15));
-        n[10] = -(scale(cx, F16) + scale(cy, 3.0 * G12) + scale(cz, H17));
-        n[11] = -(scale(cx, F18) + scale(cy, G19) + scale(cz, 3.0 * H13));
-        n[12] = -(scale(cx, 2.0 * F14) + scale(cy, 2.0 * G16) + scale(cz, H20));
-        n[13] = -(scale(cx, F20) + scale(cy, 2.0 * G17) + scale(cz, 2.0 * H19));
-        n[14] = -(scale(cx, 2.0 * F15) + scale(cy, G20) + scale(cz, 2.0 * H18));
+        n[6] = fio.leave(-(c.template times<0>(F30) + c.template times<1>(0.5 * G33) + c.template times<2>(0.5 * H35)));
+        n[7] = fio.leave(-(c.template times<0>(0.5 * F33) + c.template times<1>(G31) + c.template times<2>(0.5 * H34)));
+        n[8] = fio.leave(-(c.template times<0>(0.5 * F35) + c.template times<1>(0.5 * G34) + c.template times<2>(H32)));
+        n[9] = fio.leave(-(c.template times<0>(3.0 * keep(F11)) + c.template times<1>(G14) + c.template times<2>(H15)));
+        n[10] = fio.leave(-(c.template times<0>(F16) + c.template times<1>(3.0 * keep(G12)) + c.template times<2>(H17)));
+        n[11] = fio.leave(-(c.template times<0>(F18) + c.template times<1>(G19) + c.template times<2>(3.0 * keep(H13))));
+        n[12] = fio.leave(-(c.template times<0>(2.0 * F14) + c.template times<1>(2.0 * G16) + c.template times<2>(keep(H20))));
+        n[13] = fio.leave(-(c.template times<0>(keep(F20)) + c.template times<1>(2.0 * G17) + c.template times<2>(2.0 * H19)));
+        n[14] = fio.leave(-(c.template times<0>(2.0 * F15) + c.template times<1>(keep(G20)) + c.template times<2>(2.0 * H18)));
         if constexpr (SRC) {        // Eq. 45, source terms
             V ts[15];
             time_source_modes(w, ts);
@@ -521,8 +558,8 @@ ADER_DEV constexpr int mean_node(int k) {
     constexpr int n[12] = {1, 2, 5, 6, 9, 14, 15, 16, 17, 18, 19, 24};
     return n[k];
 }
-template <class V>
-ADER_DEV V face_mean(const V* F) {
+template <class F_>
+ADER_DEV auto face_mean(const F_& F) {
     return (11.0 * F[1] - 2.0 * (F[2] + F[5] + F[6] + F[9]) - 3.0 * F[14] + 3.0 * (F[15] + F[16] + F[17] + F[18]) +
             9.0 * F[19] + 3.0 * F[24]) / 24.0;
 }
