@@ -173,10 +173,24 @@ __global__ void __launch_bounds__(256) kb_flux_update(BatchGroupDev g) {
         const long long z = batch_block_item(g, base, it) + threadIdx.x;
         if (z >= it.a.grid.n) continue;
         double* U = it.U;
-        if constexpr (sizeof(R) == 4)
+        if constexpr (NV == 8) {                        // from the fluxes of kb_mhd_faces
+            float chi[3], clo[3];
+            split_scales(it.a, 1.0, 1, chi, clo);
+            zone_flux_update_stored_pair(it.a, U, U, chi, clo, z);
+        } else {
             zone_flux_update_pair<SOLVER, NV>(it.a, U, U, 1.0, 1, z);
-        else
-            zone_flux_update<SOLVER, NV, R>(it.a, U, U, 1.0, 1, z);
+        }
+    }
+}
+
+// MHD: every face solved once, with its edge fluxes
+template <int SOLVER, class R>
+__global__ void __launch_bounds__(128) kb_mhd_faces(BatchGroupDev g) {
+    __shared__ BatchItem it;
+    for (long long base = (long long)blockIdx.x * blockDim.x; base < g.total; base += batch_stride()) {
+        const long long z = batch_block_item(g, base, it) + threadIdx.x;
+        if (z >= it.a.grid.n) continue;
+        zone_face_fluxes<SOLVER, 8, R>(it.a, z);
     }
 }
 
@@ -201,8 +215,8 @@ __global__ void __launch_bounds__(256) kb_ct(BatchGroupDev g) {
 }
 
 // Phases of one step, in order; a group runs those that apply to it.
-enum BatchPhase { PH_TO_F32 = 0, PH_FACE_B, PH_WENO1D, PH_CROSS1, PH_CROSS2, PH_PREDICT, PH_UPDATE, PH_EMF, PH_CT,
-                  PH_COUNT };
+enum BatchPhase { PH_TO_F32 = 0, PH_FACE_B, PH_WENO1D, PH_CROSS1, PH_CROSS2, PH_PREDICT, PH_FACES, PH_UPDATE, PH_EMF,
+                  PH_CT, PH_COUNT };
 
 // whether a phase's kernel walks the group's range with a grid-stride loop (any grid size), or needs a
 // thread for every padded zone
@@ -210,12 +224,13 @@ inline bool batch_phase_persistent(int ph) { return ph != PH_PREDICT; }
 
 // the largest block a phase's kernel is compiled for (its launch bounds)
 inline int batch_phase_max_threads(int ph) {
-    return ph == PH_PREDICT ? BATCH_PREDICT_MAX_THREADS : (ph == PH_WENO1D || ph == PH_CROSS1) ? 128 : 256;
+    return ph == PH_PREDICT ? BATCH_PREDICT_MAX_THREADS : (ph == PH_WENO1D || ph == PH_CROSS1 || ph == PH_FACES) ? 128 : 256;
 }
 
 inline bool batch_phase_applies(int ph, int order, int mhd) {
     switch (ph) {
-        case PH_FACE_B: return mhd != 0;
+        case PH_FACE_B:
+        case PH_FACES: return mhd != 0;
         case PH_CROSS1: return order >= 3;
         case PH_CROSS2: return order == 4;
         case PH_EMF:

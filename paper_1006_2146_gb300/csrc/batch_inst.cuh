@@ -47,6 +47,11 @@ int batch_phase(int ph, const BatchGroupDev& g, int form, int solver, int thread
                     return -1;
             }
             break;
+        case PH_FACES:
+            if constexpr (NV == 8)
+                k = solver == SOLVER_LINEARIZED ? (const void*)kb_mhd_faces<SOLVER_LINEARIZED, R>
+                                                : (const void*)kb_mhd_faces<SOLVER_HLL, R>;
+            break;
         case PH_UPDATE:
             k = solver == SOLVER_LINEARIZED ? (const void*)kb_flux_update<SOLVER_LINEARIZED, NV, R>
                                             : (const void*)kb_flux_update<SOLVER_HLL, NV, R>;

@@ -34,7 +34,7 @@ struct StepArgs {
     double dt;          // used when dt_dev is null
     const double* dt_dev;
     void* S1;           // 1-D WENO moments          (R)
-    void* S2;           // cross moments             (R)
+    void* S2;           // cross moments, then MHD's edge fluxes (R)
     void* S3;           // face-side data             (R)
     unsigned* flag;     // device error flag
     int mhd;            // 1: ideal MHD (8 variables, face-centred B)
@@ -49,8 +49,9 @@ struct StepArgs {
     int emf_transonic;  // MHD: twice the dissipative term of the EMF fluxes at transonic faces
     int defer_nonfinite;  // the positivity fallback checks the updated state itself (after its passes)
     int wait_test;      // the learned-guess kernel's test of its bounded waits (ader_test_bounded_wait)
-    int tiled;          // Euler, orders 2-3: predictor and face solves per 2.5-D tile (k_pf_tile), fluxes
-                        // stored once per face in S1; 0: face data of every zone through S3 (MHD, order 4)
+    int tiled;          // FP32 Euler, orders 2-3: predictor and face solves per 2.5-D tile (k_pf_tile), fluxes stored
+                        // once per face in S1; 0 (and FP64, MHD, order 4): face data of every zone through S3.
+                        // Also the WENO tiles (recon.cu)
 };
 
 // gamma, gamma - 1 and 1 / dx_d in the bulk precision R
@@ -77,7 +78,8 @@ inline void finish_args(StepArgs& a) {
 // Number of R values per zone in each scratch array.
 inline int nvar(int mhd) { return mhd ? 8 : 5; }
 inline int s1_per_zone(int order, int mhd) { return nvar(mhd) * 3 * (order - 1); }
-inline int s2_per_zone(int order, int mhd) { return order == 2 ? 0 : nvar(mhd) * (order == 3 ? 3 : 10); }
+// (S2 also takes the edge fluxes of MHD's faces, 12 values, once the cross moments have been read)
+inline int s2_per_zone(int order, int mhd) { return order == 2 ? (mhd ? 12 : 0) : nvar(mhd) * (order == 3 ? 3 : 10); }
 // face-side values per side: u_b, <u>, <F> (NV each) and, for MHD, 4 edges x (<u_c>, <F_c>)
 ADER_DEV constexpr int side_values(int nv) { return 3 * nv + (nv == 8 ? 8 : 0); }
 // MHD with the linearized solver also keeps every edge's full averaged state: a second block of

@@ -263,22 +263,25 @@ int launch_flux_update(const StepArgs& a, double* out, const double* base, doubl
             return 1;
         }
     }
+    if (a.mhd) {                               // each face and its edge fluxes solved once, then the update
+        if (a.solver == SOLVER_HLL)
+            k_face_fluxes<SOLVER_HLL, 8, R><<<blocks, T, 0, st>>>(a);
+        else
+            k_face_fluxes<SOLVER_LINEARIZED, 8, R><<<blocks, T, 0, st>>>(a);
+        if constexpr (sizeof(R) == 4)
+            k_flux_update_stored_pair<R><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
+        else
+            k_flux_update_stored<R><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
+        return 2;
+    }
     if constexpr (sizeof(R) == 4) {           // fused, both faces of each direction per zone, FP32 pairs
-        if (a.mhd && a.solver == SOLVER_HLL)
-            k_flux_update_pair<SOLVER_HLL, 8><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
-        else if (a.mhd)
-            k_flux_update_pair<SOLVER_LINEARIZED, 8><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
-        else if (a.solver == SOLVER_HLL)
+        if (a.solver == SOLVER_HLL)
             k_flux_update_pair<SOLVER_HLL, 5><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
         else
             k_flux_update_pair<SOLVER_LINEARIZED, 5><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
         return 1;
     } else {                                   // each face solved once, then the update
-        if (a.mhd && a.solver == SOLVER_HLL)
-            k_face_fluxes<SOLVER_HLL, 8, R><<<blocks, T, 0, st>>>(a);
-        else if (a.mhd)
-            k_face_fluxes<SOLVER_LINEARIZED, 8, R><<<blocks, T, 0, st>>>(a);
-        else if (a.solver == SOLVER_HLL)
+        if (a.solver == SOLVER_HLL)
             k_face_fluxes<SOLVER_HLL, 5, R><<<blocks, T, 0, st>>>(a);
         else
             k_face_fluxes<SOLVER_LINEARIZED, 5, R><<<blocks, T, 0, st>>>(a);

@@ -10,6 +10,8 @@
 // edge averages <u_c> and <F_c> (Eq. 57, Eqs. D.5/D.10/D.15) of the field
 // component c = 5 + t the edge's EMF needs.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 #include "fixed.cuh"
 #include "kernels.cuh"
@@ -560,28 +562,128 @@ __global__ void __launch_bounds__(128) k_flux_update_pair(StepArgs a, double* ou
     store_pair_update(a, out, base, hi, lo, z);
 }
 
-// The same update for one zone whose block may not share its problem (the batched kernels): c_d's FP32
+// The same updates for one zone whose block may not share its problem (the batched kernels): c_d's FP32
 // head and tail taken per zone, the split by integer conversions (one FP64 product and one difference
 // per direction).
-template <int SOLVER, int NV>
-__device__ __forceinline__ void zone_flux_update_pair(const StepArgs& a, double* out, const double* base,
-                                                      double c_host, int use_dt_dev, long long z) {
-    int i, j, k;
-    zone_ijk(a.grid, z, i, j, k);
+__device__ __forceinline__ void split_scales(const StepArgs& a, double c_host, int use_dt_dev, float* chi, float* clo) {
     const double c = use_dt_dev ? c_host * (*a.dt_dev) : c_host;
-    float chi[3], clo[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const double cd = c * a.idx[d];
         chi[d] = f32_of_f64(cd);
         clo[d] = f32_of_f64(cd - f64_of_f32(chi[d]));
     }
+}
+
+template <int SOLVER, int NV>
+__device__ __forceinline__ void zone_flux_update_pair(const StepArgs& a, double* out, const double* base,
+                                                      double c_host, int use_dt_dev, long long z) {
+    int i, j, k;
+    zone_ijk(a.grid, z, i, j, k);
+    float chi[3], clo[3];
+    split_scales(a, c_host, use_dt_dev, chi, clo);
     const float gamma = a.gamma_f, gm1 = a.gm1_f;
     float hi[5] = {0, 0, 0, 0, 0}, lo[5] = {0, 0, 0, 0, 0};
     flux_difference_pair<SOLVER, 0, NV>(a, z, i, j, k, gamma, gm1, chi[0], clo[0], hi, lo);
     flux_difference_pair<SOLVER, 1, NV>(a, z, i, j, k, gamma, gm1, chi[1], clo[1], hi, lo);
     flux_difference_pair<SOLVER, 2, NV>(a, z, i, j, k, gamma, gm1, chi[2], clo[2], hi, lo);
     store_pair_update(a, out, base, hi, lo, z);
+}
+
+// Eq. 6 from the stored face fluxes: the differences in FP32 pairs, the accumulation in FP64
+__device__ __forceinline__ void zone_flux_update_stored_pair(const StepArgs& a, double* out, const double* base,
+                                                             const float* c_hi, const float* c_lo, long long z) {
+    int i, j, k;
+    zone_ijk(a.grid, z, i, j, k);
+    const float* F = (const float*)a.S1;
+    const long long N = a.grid.n;
+    float hi[5] = {0, 0, 0, 0, 0}, lo[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+    for (int D = 0; D < 3; ++D) {
+        const long long zm = nbr_along(a.grid, z, i, j, k, D, -1);
+        const float chi = c_hi[D], clo = c_lo[D];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+            float s, e;
+            two_sum(F[(D * 5 + v) * N + zm], -F[(D * 5 + v) * N + z], s, e);
+            const float p = s * chi;
+            const float pe = fmaf(s, chi, -p);
+            const float t = pe + fmaf(s, clo, e * chi);
+            float h, he;
+            two_sum(hi[v], p, h, he);
+            hi[v] = h;
+            lo[v] += he + t;
+        }
+    }
+    store_pair_update(a, out, base, hi, lo, z);
+}
+
+// ------------------------------------------------------------------ MHD: faces and their edge fluxes (Sec. II.3, Eq. 7)
+// A face's Riemann problem is transonic when a fast wave speed changes sign between its two states.
+template <class R>
+ADER_DEV bool transonic(R vl, R cl, R vr, R cr) {
+    return (vl - cl) * (vr - cr) < R(0) || (vl + cl) * (vr + cr) < R(0);
+}
+
+// The flux of the face of direction D between the states L and Rt with its edge values uL, FL and uR, FR (of the field
+// component the edge's EMF needs): HLL with the face's own frozen wave speeds.
+template <int D, class R>
+ADER_DEV R edge_hll(const Vec<8, R>& ubl, const Vec<8, R>& ubr, int emf_transonic, R uL, R FL, R uR, R FR, R gamma, R gm1) {
+    const Prim<8, R> pl = primitives(ubl, gm1), pr = primitives(ubr, gm1);
+    const R vl = D == 0 ? pl.vx : (D == 1 ? pl.vy : pl.vz);
+    const R vr = D == 0 ? pr.vx : (D == 1 ? pr.vy : pr.vz);
+    const R cl = fast_speed<D>(ubl, pl, gamma), cr = fast_speed<D>(ubr, pr, gamma);
+    const R lamL = fmin(fmin(vl - cl, vr - cr), R(0));
+    const R lamR = fmax(fmax(vl + cl, vr + cr), R(0));
+    // optional: twice the third (dissipative) term of Eq. 17 where a fast speed changes sign (Sec. V)
+    const R w = (emf_transonic && transonic(vl, cl, vr, cr)) ? R(2) : R(1);
+    return (lamR * FL - lamL * FR + (w * lamR) * lamL * (uR - uL)) * rcp(lamR - lamL);
+}
+
+// The same flux with the linearized solver: |A| at the mean of the face's two
+// barycentre states applied to the jump dU of the full edge-averaged states.
+template <int D, class R>
+ADER_DEV R edge_linearized(const Vec<8, R>& ubl, const Vec<8, R>& ubr, int emf_transonic, int c, const Vec<8, R>& dU, R FL,
+                           R FR, R gamma, R gm1) {
+    const MeanState<R> m = mhd_mean_state(ubl, ubr, gm1);
+    const Vec<8, R> diss = mhd_abs_jacobian_apply<D, R>(m.rho, m.v, m.p, m.B, gamma, gm1, dU);
+    R w = R(1);
+    if (emf_transonic) {           // optional doubled dissipation at transonic faces (Sec. V)
+        const Prim<8, R> pl = primitives(ubl, gm1), pr = primitives(ubr, gm1);
+        const R vl = D == 0 ? pl.vx : (D == 1 ? pl.vy : pl.vz);
+        const R vr = D == 0 ? pr.vx : (D == 1 ? pr.vy : pr.vz);
+        if (transonic(vl, fast_speed<D>(ubl, pl, gamma), vr, fast_speed<D>(ubr, pr, gamma))) w = R(2);
+    }
+    return R(0.5) * (FL + FR) - (R(0.5) * w) * diss[c];
+}
+
+// The upper face of zone z in direction D (zp the zone above it): its flux into F and the fluxes of its four edges
+// (t1+, t1-, t2+, t2-) into q, the wave speeds or eigenvectors taken once.  A zone's EMFs used to solve each face
+// again for every edge that met it, twelve solves a zone beside the update's.
+template <int SOLVER, int D, class R>
+ADER_DEV void mhd_face(const StepArgs& a, long long z, long long zp, R gamma, R gm1, Vec<8, R>& f, R* q) {
+    constexpr int NQ = side_values(8);
+    constexpr int T1 = D == 0 ? 1 : 0, T2 = D == 2 ? 1 : 2;
+    const long long N = a.grid.n;
+    const R* S3 = (const R*)a.S3;
+    const FaceSide<8, R> L = load_side<8, R>(a, 2 * D, z), Rt = load_side<8, R>(a, 2 * D + 1, zp);
+    f = riemann<SOLVER, D>(L, Rt, gamma, gm1);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const R* pl = S3 + (long long)(2 * D * NQ + 24 + 2 * e) * N + z;
+        const R* pr = S3 + (long long)((2 * D + 1) * NQ + 24 + 2 * e) * N + zp;
+        if constexpr (SOLVER == SOLVER_HLL) {
+            q[e] = edge_hll<D>(L.ub, Rt.ub, a.emf_transonic, pl[0], pl[N], pr[0], pr[N], gamma, gm1);
+        } else {
+            const R* X = S3 + (long long)6 * NQ * N;
+            Vec<8, R> dU;
+#pragma unroll
+            for (int v = 0; v < 8; ++v)
+                dU[v] = X[(long long)((2 * D + 1) * EDGE_STATE_VALUES + e * 8 + v) * N + zp] -
+                        X[(long long)(2 * D * EDGE_STATE_VALUES + e * 8 + v) * N + z];
+            q[e] = edge_linearized<D>(L.ub, Rt.ub, a.emf_transonic, 5 + (e < 2 ? T1 : T2), dU, pl[N], pr[N], gamma, gm1);
+        }
+    }
 }
 
 template <int SOLVER, int NV, class R>
@@ -591,15 +693,26 @@ ADER_DEV void zone_face_fluxes(const StepArgs& a, long long z) {
     const R gamma = arg_gamma<R>(a), gm1 = arg_gm1<R>(a);
     R* F = (R*)a.S1;
     const long long N = a.grid.n;
-    const Vec<NV, R> f0 = upper_face_flux<SOLVER, 0, NV, R>(a, z, i, j, k, gamma, gm1);
+    auto face = [&](auto dir) {
+        constexpr int D = decltype(dir)::value;
+        if constexpr (NV == 8) {
+            Vec<8, R> f;
+            R q[4];
+            mhd_face<SOLVER, D, R>(a, z, nbr_along(a.grid, z, i, j, k, D, 1), gamma, gm1, f, q);
+            R* Q = (R*)a.S2;            // the cross moments, read by now
 #pragma unroll
-    for (int v = 0; v < 5; ++v) F[(0 * 5 + v) * N + z] = f0[v];
-    const Vec<NV, R> f1 = upper_face_flux<SOLVER, 1, NV, R>(a, z, i, j, k, gamma, gm1);
+            for (int e = 0; e < 4; ++e) Q[(long long)(D * 4 + e) * N + z] = q[e];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) F[(1 * 5 + v) * N + z] = f1[v];
-    const Vec<NV, R> f2 = upper_face_flux<SOLVER, 2, NV, R>(a, z, i, j, k, gamma, gm1);
+            for (int v = 0; v < 5; ++v) F[(D * 5 + v) * N + z] = f[v];
+        } else {
+            const Vec<NV, R> f = upper_face_flux<SOLVER, D, NV, R>(a, z, i, j, k, gamma, gm1);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) F[(2 * 5 + v) * N + z] = f2[v];
+            for (int v = 0; v < 5; ++v) F[(D * 5 + v) * N + z] = f[v];
+        }
+    };
+    face(std::integral_constant<int, 0>{});
+    face(std::integral_constant<int, 1>{});
+    face(std::integral_constant<int, 2>{});
 }
 
 template <int SOLVER, int NV, class R>
@@ -894,8 +1007,7 @@ void launch_pf_tile(const StepArgs& a, const double* U, cudaStream_t st) {
     }
 }
 
-// FP32 bulk, Eq. 6 from the stored face fluxes (tiled path): the differences in FP32 pairs as in
-// k_flux_update_pair, the accumulation in FP64
+// FP32 bulk, Eq. 6 from the stored face fluxes (the tiles' or MHD's)
 template <class R>
 __global__ void __launch_bounds__(128) k_flux_update_stored_pair(StepArgs a, double* out, const double* base,
                                                                  double c_host, int use_dt_dev) {
@@ -910,105 +1022,10 @@ __global__ void __launch_bounds__(128) k_flux_update_stored_pair(StepArgs a, dou
     }
     __syncthreads();
     const long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (z >= a.grid.n) return;
-    int i, j, k;
-    zone_ijk(a.grid, z, i, j, k);
-    const float* F = (const float*)a.S1;
-    const long long N = a.grid.n;
-    float hi[5] = {0, 0, 0, 0, 0}, lo[5] = {0, 0, 0, 0, 0};
-#pragma unroll
-    for (int D = 0; D < 3; ++D) {
-        const long long zm = nbr_along(a.grid, z, i, j, k, D, -1);
-        const float chi = c_hi[D], clo = c_lo[D];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {
-            float s, e;
-            two_sum(F[(D * 5 + v) * N + zm], -F[(D * 5 + v) * N + z], s, e);
-            const float p = s * chi;
-            const float pe = fmaf(s, chi, -p);
-            const float t = pe + fmaf(s, clo, e * chi);
-            float h, he;
-            two_sum(hi[v], p, h, he);
-            hi[v] = h;
-            lo[v] += he + t;
-        }
-    }
-    store_pair_update(a, out, base, hi, lo, z);
+    if (z < a.grid.n) zone_flux_update_stored_pair(a, out, base, c_hi, c_lo, z);
 }
 
 // ------------------------------------------------------------------ MHD: edge EMFs (Sec. II.3, Eq. 7)
-// HLL flux of the face of direction D between zones zl (lower) and zr,
-// evaluated with its edge slot e (0: t1+, 1: t1-, 2: t2+, 3: t2-): the face's
-// own frozen wave speeds (from its barycentre states) applied to the edge
-// averages of its two sides.
-// A face's Riemann problem is transonic when a fast wave speed changes sign between its two states.
-template <class R>
-ADER_DEV bool transonic(R vl, R cl, R vr, R cr) {
-    return (vl - cl) * (vr - cr) < R(0) || (vl + cl) * (vr + cr) < R(0);
-}
-
-template <int D, class R>
-ADER_DEV R edge_hll(const StepArgs& a, long long zl, long long zr, int e, R gamma, R gm1) {
-    constexpr int NQ = side_values(8);
-    const R* S3 = (const R*)a.S3;
-    const long long N = a.grid.n;
-    const int sl = 2 * D, sr = 2 * D + 1;
-    Vec<8, R> ubl, ubr;
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        ubl[v] = S3[(sl * NQ + v) * N + zl];
-        ubr[v] = S3[(sr * NQ + v) * N + zr];
-    }
-    const Prim<8, R> pl = primitives(ubl, gm1), pr = primitives(ubr, gm1);
-    const R vl = D == 0 ? pl.vx : (D == 1 ? pl.vy : pl.vz);
-    const R vr = D == 0 ? pr.vx : (D == 1 ? pr.vy : pr.vz);
-    const R cl = fast_speed<D>(ubl, pl, gamma), cr = fast_speed<D>(ubr, pr, gamma);
-    const R lamL = fmin(fmin(vl - cl, vr - cr), R(0));
-    const R lamR = fmax(fmax(vl + cl, vr + cr), R(0));
-    const R uL = S3[(sl * NQ + 24 + 2 * e) * N + zl], FL = S3[(sl * NQ + 25 + 2 * e) * N + zl];
-    const R uR = S3[(sr * NQ + 24 + 2 * e) * N + zr], FR = S3[(sr * NQ + 25 + 2 * e) * N + zr];
-    // optional: twice the third (dissipative) term of Eq. 17 where a fast speed changes sign (Sec. V)
-    const R w = (a.emf_transonic && transonic(vl, cl, vr, cr)) ? R(2) : R(1);
-    return (lamR * FL - lamL * FR + (w * lamR) * lamL * (uR - uL)) / (lamR - lamL);
-}
-
-// The same flux with the linearized solver: |A| at the mean of the face's two
-// barycentre states applied to the jump of the full edge-averaged states.
-template <int D, class R>
-ADER_DEV R edge_linearized(const StepArgs& a, long long zl, long long zr, int e, R gamma, R gm1) {
-    constexpr int NQ = side_values(8);
-    constexpr int T1 = D == 0 ? 1 : 0, T2 = D == 2 ? 1 : 2;
-    const R* S3 = (const R*)a.S3;
-    const R* X = S3 + (long long)6 * NQ * a.grid.n;
-    const long long N = a.grid.n;
-    const int sl = 2 * D, sr = 2 * D + 1;
-    Vec<8, R> ubl, ubr, dU;
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        ubl[v] = S3[(sl * NQ + v) * N + zl];
-        ubr[v] = S3[(sr * NQ + v) * N + zr];
-        dU[v] = X[(sr * EDGE_STATE_VALUES + e * 8 + v) * N + zr] - X[(sl * EDGE_STATE_VALUES + e * 8 + v) * N + zl];
-    }
-    const MeanState<R> m = mhd_mean_state(ubl, ubr, gm1);
-    const Vec<8, R> diss = mhd_abs_jacobian_apply<D, R>(m.rho, m.v, m.p, m.B, gamma, gm1, dU);
-    const int c = 5 + (e < 2 ? T1 : T2);
-    const R FL = S3[(sl * NQ + 25 + 2 * e) * N + zl], FR = S3[(sr * NQ + 25 + 2 * e) * N + zr];
-    R w = R(1);
-    if (a.emf_transonic) {           // optional doubled dissipation at transonic faces (Sec. V)
-        const Prim<8, R> pl = primitives(ubl, gm1), pr = primitives(ubr, gm1);
-        const R vl = D == 0 ? pl.vx : (D == 1 ? pl.vy : pl.vz);
-        const R vr = D == 0 ? pr.vx : (D == 1 ? pr.vy : pr.vz);
-        if (transonic(vl, fast_speed<D>(ubl, pl, gamma), vr, fast_speed<D>(ubr, pr, gamma))) w = R(2);
-    }
-    return R(0.5) * (FL + FR) - (R(0.5) * w) * diss[c];
-}
-
-template <int D, class R>
-ADER_DEV R edge_flux(const StepArgs& a, long long zl, long long zr, int e, R gamma, R gm1) {
-    return a.solver == SOLVER_LINEARIZED ? edge_linearized<D, R>(a, zl, zr, e, gamma, gm1)
-                                         : edge_hll<D, R>(a, zl, zr, e, gamma, gm1);
-}
-
 // EMFs at the three upper edges of zone (i, j, k): Ez on (i+1/2, j+1/2),
 // Ey on (i+1/2, k+1/2), Ex on (j+1/2, k+1/2); each the mean of the four
 // adjacent faces' edge fluxes with Eq. 7's signs (Ez = -F7 = G6,
@@ -1018,16 +1035,14 @@ ADER_DEV void zone_emf(const StepArgs& a, long long z) {
     const Grid& g = a.grid;
     int i, j, k;
     zone_ijk(g, z, i, j, k);
-    const R gamma = arg_gamma<R>(a), gm1 = arg_gm1<R>(a);
     const long long zx = nbr(g, i, j, k, 1, 0, 0), zy = nbr(g, i, j, k, 0, 1, 0), zz = nbr(g, i, j, k, 0, 0, 1);
-    const long long zxy = nbr(g, i, j, k, 1, 1, 0), zxz = nbr(g, i, j, k, 1, 0, 1), zyz = nbr(g, i, j, k, 0, 1, 1);
-    // x-faces: t1 = y (slots 0, 1), t2 = z (2, 3); y-faces: t1 = x, t2 = z; z-faces: t1 = x, t2 = y
-    const R Ez = R(0.25) * (-edge_flux<0, R>(a, z, zx, 0, gamma, gm1) - edge_flux<0, R>(a, zy, zxy, 1, gamma, gm1) +
-                            edge_flux<1, R>(a, z, zy, 0, gamma, gm1) + edge_flux<1, R>(a, zx, zxy, 1, gamma, gm1));
-    const R Ey = R(0.25) * (edge_flux<0, R>(a, z, zx, 2, gamma, gm1) + edge_flux<0, R>(a, zz, zxz, 3, gamma, gm1) -
-                            edge_flux<2, R>(a, z, zz, 0, gamma, gm1) - edge_flux<2, R>(a, zx, zxz, 1, gamma, gm1));
-    const R Ex = R(0.25) * (-edge_flux<1, R>(a, z, zy, 2, gamma, gm1) - edge_flux<1, R>(a, zz, zyz, 3, gamma, gm1) +
-                            edge_flux<2, R>(a, z, zz, 2, gamma, gm1) + edge_flux<2, R>(a, zy, zyz, 3, gamma, gm1));
+    // the edge fluxes of zone_face_fluxes, stored at the zone below the face.  x-faces: t1 = y (slots 0, 1), t2 = z
+    // (2, 3); y-faces: t1 = x, t2 = z; z-faces: t1 = x, t2 = y
+    const R* Q = (const R*)a.S2;
+    auto q = [&](int d, int e, long long at) { return Q[(long long)(d * 4 + e) * g.n + at]; };
+    const R Ez = R(0.25) * (-q(0, 0, z) - q(0, 1, zy) + q(1, 0, z) + q(1, 1, zx));
+    const R Ey = R(0.25) * (q(0, 2, z) + q(0, 3, zz) - q(2, 0, z) - q(2, 1, zx));
+    const R Ex = R(0.25) * (-q(1, 2, z) - q(1, 3, zz) + q(2, 2, z) + q(2, 3, zy));
     R* E = (R*)a.E;
     E[z] = Ex;
     E[g.n + z] = Ey;
