@@ -176,6 +176,62 @@ def _terms(C, k, lo, hi, f_name, idx_shift):
     return out
 
 
+def _grouped(terms):
+    """Terms {name: coefficient} as a sum of c * (a - b + ...), one product per distinct |c|."""
+    groups = {}
+    for name, c in terms.items():
+        if c != 0:
+            groups.setdefault(abs(c), []).append(("-" if c < 0 else "+", name))
+    out = []
+    for c, ts in groups.items():
+        if ts[0][0] == "-":
+            sign, ts = "-", [("+" if x == "-" else "-", n) for x, n in ts]
+        else:
+            sign = "+"
+        body = ts[0][1] + "".join(" %s %s" % t for t in ts[1:])
+        if len(ts) > 1:
+            body = "(%s)" % body
+        out.append("%s %s" % (sign, body if c == 1 else "%.17g * %s" % (float(c), body)))
+    return "\n        ".join(out)
+
+
+def mode_coefficients(C):
+    """D[d][k][m] (exact): response of node k to mode m = 2..20 of the tau = 0 interpolant of scaled flux d."""
+    V0 = [[_phi(m, p) for m in MODES[:20]] for p in NODES[:20]]
+    return [{k: {m + 1: sum(C[d][k][j + 1] * V0[j][m] for j in range(20)) for m in range(20)} for k in range(21, 36)}
+            for d in range(3)]
+
+
+def emit_modes(C):
+    """The update for scalars whose sums cost less than their products (zone-scaled integers)."""
+    D = mode_coefficients(C)
+    lines = ["// the tau = 0 node at the spatial point of node 21 + k",
+             "ADER_DEV constexpr int nodal_o4_base(int k) {",
+             "    constexpr int b[15] = {%s};" % ", ".join(str(base_node(k)) for k in range(21, 36)),
+             "    return b[k];",
+             "}",
+             "",
+             "// The same update where additions are cheap (fixed.cuh).  The tau = 0 terms from the flux modes of the",
+             "// twenty nodes, f[m], g[m], h[m] (scaled, m = 2..20): dq[k-21], without u[base(k)].",
+             "template <class V>",
+             "ADER_DEV void nodal_o4_qterms_modes(const V* f, const V* g, const V* h, V* dq) {"]
+    row = {k: {"%s[%d]" % (a, m): D[d][k][m] for d, a in enumerate("fgh") for m in range(1, 21)} for k in range(21, 36)}
+    for base, name, ks in ((21, "q1", range(21, 31)), (31, "q2", range(31, 35))):     # tau = 1/3 and tau = 2/3
+        lines.append("    const V %s = %s;" % (name, _grouped(row[base]).lstrip("+ ")))
+        for k in ks:
+            d = {n: row[k][n] - row[base][n] for n in row[k]}
+            lines.append("    dq[%d] = %s%s;" % (k - 21, name, "".join("\n        " + x for x in [_grouped(d)] if x)))
+    lines.append("    dq[14] = %s;" % _grouped(row[35]).lstrip("+ "))
+    lines += ["}", "",
+              "// one Picard step without qt: de[k-21], from the scaled fluxes at the nodes tau > 0 (index node - 21)",
+              "template <class V>",
+              "ADER_DEV void nodal_o4_update_terms(const V* f, const V* g, const V* h, V* de) {"]
+    for k in range(21, 36):
+        t = {"%s[%d]" % (a, j - 21): C[d][k][j] for d, a in enumerate("fgh") for j in range(21, 36)}
+        lines.append("    de[%d] = %s;" % (k - 21, _grouped(t).lstrip("+ ")))
+    return lines + ["}", ""]
+
+
 def emit():
     C = coefficients()
     lines = [
@@ -219,9 +275,9 @@ def emit():
         t = _terms(C, k, 21, 35, None, 21)
         assert all("[14]" not in s for s in t), "node 35 flux must not enter the update"
         lines.append("    e[%d] = qt[%d]%s;" % (k - 21, k - 21, "".join("\n        + " + s for s in t)))
+    lines += ["}", ""] + emit_modes(C)
     CS, W = source_coefficients()
-    lines += ["}", "",
-              "// the source terms of Eq. C.2: qt[k-21] += tau = 0 node sources s[1..20] (s = dt S)",
+    lines += ["// the source terms of Eq. C.2: qt[k-21] += tau = 0 node sources s[1..20] (s = dt S)",
               "template <int NV, class R>",
               "ADER_DEV void nodal_o4_qterms_src(const Vec<NV, R>* s, Vec<NV, R>* qt) {"]
     for k in range(21, 36):

@@ -411,6 +411,38 @@ ADER_DEV void nodal_o4_to_modes(const Vec<NV, R>* u, const Vec<NV, R>* e, Vec<NV
 #undef UB
 }
 
+// The modes 2..20 of the polynomial through the values n[1..20] at the tau = 0 nodes of Eq. C.1: Eq. C.4 solved for the
+// modes, about 100 additions and 15 products.  The nodes' quarter points couple w14, w17 and w18 in a ring.
+template <class V>
+ADER_DEV void nodal_o4_flux_modes(const V* n, V* m) {
+    m[5] = 2.0 * (n[3] + n[4] - 2.0 * n[1]);
+    m[6] = 2.0 * (n[5] + n[6] - 2.0 * n[1]);
+    m[7] = 2.0 * (n[7] + n[8] - 2.0 * n[1]);
+    m[15] = 4.0 * (n[10] - 2.0 * n[7] + n[11]) - 2.0 * m[5];
+    m[16] = 4.0 * (n[12] - 2.0 * n[3] + n[13]) - 2.0 * m[6];
+    m[19] = 4.0 * (n[14] - 2.0 * n[5] + n[9]) - 2.0 * m[7];
+    const V b8 = n[13] - n[3] - n[5] + n[1], b9 = n[9] - n[5] - n[7] + n[1], b10 = n[11] - n[3] - n[7] + n[1];
+    m[20] = 8.0 * (n[2] - n[11] - n[9] + n[7] - b8);
+    const V k1 = 8.0 * n[8] - 4.0 * n[14] + 0.25 * m[5] + 2.0 * m[6] - 0.125 * m[15] - 2.0 * (n[15] + n[16]);
+    const V k2 = 8.0 * n[4] - 4.0 * n[10] + 0.25 * m[6] + 2.0 * m[7] - 0.125 * m[16] - 2.0 * (n[17] + n[18]);
+    const V k3 = 8.0 * n[6] - 4.0 * n[12] + 2.0 * m[5] + 0.25 * m[7] - 0.125 * m[19] - 2.0 * (n[19] + n[20]);
+    m[14] = (512.0 / 513.0) * (k3 - 0.125 * k2 + 0.015625 * k1);
+    m[17] = k1 - 0.125 * m[14];
+    m[18] = k2 - 0.125 * m[17];
+    m[8] = 4.0 * b8 - 0.5 * (m[14] + m[16]);
+    m[9] = 4.0 * b9 - 0.5 * (m[17] + m[19]);
+    m[10] = 4.0 * b10 - 0.5 * (m[15] + m[18]);
+    const V h1 = 0.5 * (n[3] - n[1]) - 0.125 * m[5], h2 = 0.5 * (n[5] - n[1]) - 0.125 * m[6],
+            h3 = 0.5 * (n[7] - n[1]) - 0.125 * m[7];
+    const V g1 = m[16] + m[18], g2 = m[14] + m[19], g3 = m[15] + m[17];
+    m[11] = (64.0 / 3.0) * (h1 + 0.0625 * (g1 + m[20]) - 0.125 * (m[8] + m[10]) - 0.5 * (n[16] - n[15]));
+    m[12] = (64.0 / 3.0) * (h2 + 0.0625 * (g2 + m[20]) - 0.125 * (m[8] + m[9]) - 0.5 * (n[18] - n[17]));
+    m[13] = (64.0 / 3.0) * (h3 + 0.0625 * (g3 + m[20]) - 0.125 * (m[9] + m[10]) - 0.5 * (n[20] - n[19]));
+    m[2] = 4.0 * h1 + g1 / 12.0 - 0.1 * m[11];
+    m[3] = 4.0 * h2 + g2 / 12.0 - 0.1 * m[12];
+    m[4] = 4.0 * h3 + g3 / 12.0 - 0.1 * m[13];
+}
+
 // SRC: with a non-stiff source (s = dt S at nodes 1..20 once and at the tau > 0 nodes of the current
 // iterate; the source terms of Eqs. C.2-C.3); sdt receives dt S-bar of Eq. C.6 from the final iterate.
 template <class T, bool SRC = false>
@@ -457,18 +489,74 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
 #pragma unroll
         for (int k = 1; k <= 20; ++k) u[k] = fr.leave(s[k]);
     }
-    // Eq. C.2 without sources: q-terms of the tau = 0 fluxes
+    // Eq. C.2 without sources: q-terms of the tau = 0 fluxes.  FP64 takes them from the fluxes' modes, in integers
+    // (sums of up to 210 fluxes); the sums over nodes took 879 multiply-adds a variable, an iteration's 282.
+    constexpr bool INTS = !std::is_same<typename FR::S, R>::value;
+    using FF = FR;
+    using VF = VS;
+    const AxisScale<FF> c(t.cx, t.cy, t.cz);
     V qt[16];
     {
         V f[21], g[21], h[21];
-        t.template fluxes<20, 0, true>(u + 1, f + 1, g + 1, h + 1);
-        nodal_o4_qterms(u, f, g, h, qt);
+        t.template fluxes<20, 0, !INTS>(u + 1, f + 1, g + 1, h + 1);
+        if constexpr (INTS) {
+            FF ff;
+#pragma unroll
+            for (int k = 1; k <= 20; ++k) {
+                ff.include(f[k]);
+                ff.include(g[k]);
+                ff.include(h[k]);
+            }
+            ff.close();
+            VF n[21], F[21], G[21], H[21], dq[15];
+#pragma unroll
+            for (int k = 1; k <= 20; ++k) n[k] = ff.enter(f[k]);
+            nodal_o4_flux_modes(n, F);
+#pragma unroll
+            for (int k = 1; k <= 20; ++k) n[k] = ff.enter(g[k]);
+            nodal_o4_flux_modes(n, G);
+#pragma unroll
+            for (int k = 1; k <= 20; ++k) n[k] = ff.enter(h[k]);
+            nodal_o4_flux_modes(n, H);
+#pragma unroll
+            for (int k = 2; k <= 20; ++k) {
+                F[k] = c.template times<0>(F[k]);
+                G[k] = c.template times<1>(G[k]);
+                H[k] = c.template times<2>(H[k]);
+            }
+            nodal_o4_qterms_modes(F, G, H, dq);
+            const FF fo = c.out(ff);
+#pragma unroll
+            for (int k = 0; k < 15; ++k) qt[k] = u[nodal_o4_base(k)] + fo.leave(dq[k]);
+        } else {
+            nodal_o4_qterms(u, f, g, h, qt);
+        }
     }
     V s0[21];              // with a source: s at the tau = 0 nodes, built once
     if constexpr (SRC) {
         t.template sources<20>(u + 1, *src, s0 + 1);
         nodal_o4_qterms_src(s0, qt);
     }
+    auto to_modes = [&](const V* ev) {           // sums of up to 96 node values
+        if constexpr (INTS) {
+            FR ft;
+            VS us[21], es[15], ms[36];
+#pragma unroll
+            for (int k = 1; k <= 20; ++k) ft.include(u[k]);
+#pragma unroll
+            for (int k = 0; k < 15; ++k) ft.include(ev[k]);
+            ft.close();
+#pragma unroll
+            for (int k = 1; k <= 20; ++k) us[k] = ft.enter(u[k]);
+#pragma unroll
+            for (int k = 0; k < 15; ++k) es[k] = ft.enter(ev[k]);
+            nodal_o4_to_modes(us, es, ms);
+#pragma unroll
+            for (int k = 21; k <= 35; ++k) m[k] = ft.leave(ms[k]);
+        } else {
+            nodal_o4_to_modes(u, ev, m);
+        }
+    };
     // initial guess: the evolutionary modes in m[21..35] (zero: no time evolution) at the
     // tau > 0 nodes of Eq. C.1
     V e[16];
@@ -481,11 +569,33 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
     bool done = false;                  // this zone has converged (others of the team may go on)
     for (int it = 0; it < cap; ++it) {
         V f[15], g[15], h[15];          // index k - 21 for nodes 21..34
-        t.template fluxes<14, 0, true>(e, f, g, h);
+        t.template fluxes<14, 0, !INTS>(e, f, g, h);
         V se[15];
         if constexpr (SRC) t.template sources<15>(e, *src, se);
-        if (!t.waits(done)) {
-            nodal_o4_update(qt, f, g, h, e);   // Eq. C.3
+        if (!t.waits(done)) {                  // Eq. C.3
+            if constexpr (INTS) {
+                FF fi;
+                VF F[15], G[15], H[15], de[15];
+#pragma unroll
+                for (int k = 0; k < 14; ++k) {
+                    fi.include(f[k]);
+                    fi.include(g[k]);
+                    fi.include(h[k]);
+                }
+                fi.close();
+#pragma unroll
+                for (int k = 0; k < 14; ++k) {
+                    F[k] = c.template times<0>(fi.enter(f[k]));
+                    G[k] = c.template times<1>(fi.enter(g[k]));
+                    H[k] = c.template times<2>(fi.enter(h[k]));
+                }
+                nodal_o4_update_terms(F, G, H, de);
+                const FF fo = c.out(fi);
+#pragma unroll
+                for (int k = 0; k < 15; ++k) e[k] = qt[k] + fo.leave(de[k]);
+            } else {
+                nodal_o4_update(qt, f, g, h, e);
+            }
             if constexpr (SRC) nodal_o4_update_src(se, e);
             ++ctl.iters;
         }
@@ -495,7 +605,7 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
                 V old[15];
 #pragma unroll
                 for (int k = 0; k < 15; ++k) old[k] = m[21 + k];
-                nodal_o4_to_modes(u, e, m);
+                to_modes(e);
 #pragma unroll
                 for (int k = 0; k < 15; ++k) change = fmax(change, max_abs_diff(old[k], m[21 + k]));
             }
@@ -505,7 +615,7 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         }
     }
     ctl.capped = conv && !done;
-    if (!conv) nodal_o4_to_modes(u, e, m);
+    if (!conv) to_modes(e);
     if constexpr (SRC) {            // Eq. C.6 from the source at the final iterate (times dt)
         V se[15];
         t.template sources<15>(e, *src, se);
