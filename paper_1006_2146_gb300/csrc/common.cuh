@@ -76,17 +76,47 @@ ADER_DEV Vec<NV, R> scale(R s, const Vec<NV, R>& a) {
 
 template <class R> ADER_DEV R rcp(R x) { return R(1) / x; }
 
-// FP64 reciprocal: the hardware's approximate reciprocal (relative error up to 2^-19.9) seeds r, and one step of
-// third order, r + r (e + e^2) with e = 1 - x r, takes it to a rounding of the last place (e^3 < 2^-59; |1 - x r| at
-// most 1.12e-16 over 8 10^8 arguments, 1.11e-16 for two Newton steps).  On GB300 the FP64 units are scarce; this
-// costs one seed and three FMAs instead of a correctly rounded division.  Zero, infinite and subnormal arguments do
-// not occur where it is used (densities, positive sums of weights and wave-speed spans).
+// FP64 reciprocal on the integer units: the hardware's approximate reciprocal (relative error up to 2^-19.9) seeds r0,
+// and one step of third order, r0 + r0 (e + e^2) with e = 1 - x r0, takes it below a rounding of the last place.  x's
+// mantissa has 53 bits and r0's 22, so that 1 - x r0 is their product modulo 2^64 exactly (x r0 = 1 at 2^74), and e^2
+// needs its upper 32 bits.  GB300 has one FP64 unit for 32 integer ones, and as three FMAs this step was a seventh of
+// an FP64 step's FP64 instructions: on the integer units the 96^3 step takes 1.78 ms against 2.02 (second order), 3.89
+// against 4.22 (third), the 64^3 MHD step 3.47 against 3.73.  |1 - x r| at most 1.121e-16 over 1.6 10^9 arguments, as
+// the FMAs had (a half unit of the last place is 1.110e-16).
+
+// 1 / m in units of 2^-63, in [2^62, 2^63], for x = m 2^k, 1 <= |m| < 2, normal
+ADER_DEV unsigned long long inverse_mantissa(double x) {
+#ifdef __CUDA_ARCH__
+    double seed;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(seed) : "d"(x));
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), sh = (unsigned)__double2hiint(seed);
+    const unsigned ex = (hi >> 20) & 0x7ffu;
+    // r0 in units of 2^-22: the seed's exponent is that of 1 / m, one above or one below
+    const unsigned r0 = ((sh & 0xfffffu) | 0x100000u) << ((((sh >> 20) & 0x7ffu) + ex - 2044u) & 31u);
+    const unsigned long long X = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    const long long e = (long long)(0ull - X * r0);                                     // units of 2^-74
+    const int eh = (int)(e >> 32);
+    const long long s = e + (((long long)eh * eh + (0x2000ll << 10)) >> 10);
+    const long long p = (long long)((unsigned long long)(s >> 14) * r0);                // units of 2^-82
+    return ((unsigned long long)r0 << 41) + (unsigned long long)(p >> 19);
+#else
+    unsigned long long b;
+    __builtin_memcpy(&b, &x, 8);
+    return (unsigned long long)(((unsigned __int128)1 << 115) / ((b & 0xfffffffffffffull) | 0x10000000000000ull));
+#endif
+}
+
+// Zero, infinite, NaN and subnormal arguments give NaN; where 1 / x is below the normal range the result is zero.
 template <> ADER_DEV double rcp<double>(double x) {
 #ifdef __CUDA_ARCH__
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
+    const unsigned hi = (unsigned)__double2hiint(x), ex = (hi >> 20) & 0x7ffu;
+    const unsigned long long m = (inverse_mantissa(x) + 0x200ull) >> 10;                // bit 52 is the leading one
+    unsigned h = (unsigned)(m >> 32) + ((2044u - ex) << 20), l = (unsigned)m;
+    if (ex - 1u >= 2044u) {
+        h = ex - 2045u < 2u ? 0u : 0x7ff80000u;
+        l = 0u;
+    }
+    return __hiloint2double((int)(h | (hi & 0x80000000u)), (int)l);
 #else
     return 1.0 / x;
 #endif

@@ -161,12 +161,13 @@ ADER_DEV double unit_of(unsigned long long w) {
 }
 
 // the candidates' weights g_s prod_{r != s} t_r^2 without the gains g (1, 10, 1 or 1, 10, 10, 1), their largest exponent
-// and 2^63 / sum g_s w_s 2^-(GUARD + em)
+// and the reciprocal of sum g_s w_s 2^-(GUARD + em + 63): its mantissa in units of 2^-63 and the sum's exponent field
 template <int S>
 struct IntWeights {
     Scaled w[S];
     int em;
-    double inv;
+    unsigned long long inv;
+    int ei;
 
     ADER_DEV explicit IntWeights(const double* t) {
         Scaled q[S];
@@ -192,7 +193,9 @@ struct IntWeights {
         unsigned long long sum = 0;
 #pragma unroll
         for (int s = 0; s < S; ++s) sum += gain(s, down(w[s].m, em - w[s].e));
-        inv = rcp(unit_of(sum));
+        const double u = unit_of(sum);
+        inv = inverse_mantissa(u);
+        ei = (int)(bits_of(u) >> 52);
     }
     // m 2^-(GUARD + d): places for the sum of gains (12 or 22 times the largest term, and a sign)
     static constexpr int GUARD = S == 3 ? 5 : 6;
@@ -218,15 +221,17 @@ struct IntWeights {
             const unsigned long long sg = (unsigned long long)(bits_of(x[s]) >> 63);
             n += (g ^ sg) - sg;
         }
-        // n 2^(tm - em - 1086) times inv is the result
+        // n 2^(tm - em - 1086) times the reciprocal
         const unsigned long long sg = (unsigned long long)((long long)n >> 63), a = (n ^ sg) - sg;
         const unsigned hi = (unsigned)(a >> 32), top = hi ? hi : (unsigned)a;
         const int lz = u32_clz(top | 1u) + (hi ? 0 : 32);
-        const int be = tm - em - lz;                         // the exponent field
-        unsigned long long r = (((a << (lz - 1 & 63)) + 0x200ull) >> 10) + ((unsigned long long)(unsigned)(be - 1) << 52);
+        const unsigned long long p = u64_mulhi(a << (lz & 63), inv);         // the leading one at bit 62 or 61
+        const int up = (int)(~p >> 62) & 1;
+        const int be = tm - em - lz - ei + 1023 - up;                        // the exponent field
+        unsigned long long r = (((p << up) + 0x200ull) >> 10) + ((unsigned long long)(unsigned)(be - 1) << 52);
         r = a && be > 0 && ex > 0 ? r : 0ull;                // zero where all candidates are zero or subnormal
         r |= (sg & 0x8000000000000000ull) | (ex == 0x7ff ? 0x7ff8000000000000ull : 0ull);
-        return rn_mul(of_bits((long long)r), inv);
+        return of_bits((long long)r);
     }
 };
 
