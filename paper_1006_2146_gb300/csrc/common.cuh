@@ -122,6 +122,17 @@ template <> ADER_DEV double rcp<double>(double x) {
 #endif
 }
 
+// x / 2: FP64 by the exponent field (zero, the last normal binade and what is not finite stay as they are)
+template <class R> ADER_DEV R halved(R x) { return R(0.5) * x; }
+template <> ADER_DEV double halved<double>(double x) {
+#ifdef __CUDA_ARCH__
+    const unsigned h = (unsigned)__double2hiint(x), ex = h & 0x7ff00000u;
+    return __hiloint2double((int)(ex - 0x00200000u < 0x7fd00000u ? h - 0x00100000u : h), __double2loint(x));
+#else
+    return 0.5 * x;
+#endif
+}
+
 // The square root of a wave speed's square (FP64, not negative): the approximate reciprocal root y
 // (2^-19.9) seeds s = x y, and one step of third order, s + s (e / 2 + 3 e^2 / 8) with e = 1 - s y, takes it to
 // about one unit in the last place; five FP64 instructions.
@@ -250,6 +261,25 @@ ADER_DEV Vec<NV, R> flux_from(const Vec<NV, R>& u, const Prim<NV, R>& q) {
     return f;
 }
 
+// The fluxes of all three directions.  FP64 takes the products they share once: the momentum flux is symmetric and
+// MHD's electric field antisymmetric (18 FP64 instructions a node instead of 21, MHD 44 instead of 58).
+template <int NV, class R>
+ADER_DEV void fluxes_from(const Vec<NV, R>& u, const Prim<NV, R>& q, Vec<NV, R>& f, Vec<NV, R>& g, Vec<NV, R>& h) {
+    f = flux_from<0>(u, q);
+    g = flux_from<1>(u, q);
+    h = flux_from<2>(u, q);
+    if constexpr (sizeof(R) == 8) {
+        g[1] = f[2];
+        h[1] = f[3];
+        h[2] = g[3];
+        if constexpr (NV == 8) {
+            g[5] = -f[6];
+            h[5] = -f[7];
+            h[6] = -g[7];
+        }
+    }
+}
+
 // the physical flux of one direction from the conserved state; Euler takes only what that direction
 // needs (the normal velocity and P = (gamma - 1)(eps - |rho v|^2 / 2 rho), no transverse velocities)
 template <int D, int NV, class R>
@@ -258,7 +288,7 @@ ADER_DEV Vec<NV, R> flux(const Vec<NV, R>& u, R gm1) {
         const R irho = rcp(u[0]);
         const R vn = u[1 + D] * irho;
         const R m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
-        const R p = gm1 * (u[4] - R(0.5) * irho * m2);
+        const R p = gm1 * (u[4] - halved(irho) * m2);
         Vec<NV, R> f;
         f[0] = u[1 + D];
         f[1] = u[1] * vn;

@@ -40,9 +40,11 @@ struct SerialTeam {
 #pragma unroll
         for (int k = 0; k < N; ++k) {
             const Prim<NV, R> q = primitives(u[k], gm1);
-            f[k] = SC ? scale(kx, flux_from<0>(u[k], q)) : flux_from<0>(u[k], q);
-            g[k] = SC ? scale(ky, flux_from<1>(u[k], q)) : flux_from<1>(u[k], q);
-            h[k] = SC ? scale(kz, flux_from<2>(u[k], q)) : flux_from<2>(u[k], q);
+            V fx, fy, fz;
+            fluxes_from(u[k], q, fx, fy, fz);
+            f[k] = SC ? scale(kx, fx) : fx;
+            g[k] = SC ? scale(ky, fy) : fy;
+            h[k] = SC ? scale(kz, fz) : fz;
         }
 #pragma unroll
         for (int k = 0; k < A; ++k) f[N + k] = SC ? flux_scaled<0>(u[N + k], gm1, kx) : flux<0>(u[N + k], gm1);
@@ -122,9 +124,11 @@ struct WarpTeam {
                 const int at = k * 3 * NV;
                 const Vec<NV, R> x = load(at);
                 const Prim<NV, R> q = primitives(x, gm1);
-                store(at, SC ? scale(cx, flux_from<0>(x, q)) : flux_from<0>(x, q));
-                store(at + NV, SC ? scale(cy, flux_from<1>(x, q)) : flux_from<1>(x, q));
-                store(at + 2 * NV, SC ? scale(cz, flux_from<2>(x, q)) : flux_from<2>(x, q));
+                Vec<NV, R> fx, fy, fz;
+                fluxes_from(x, q, fx, fy, fz);
+                store(at, SC ? scale(cx, fx) : fx);
+                store(at + NV, SC ? scale(cy, fy) : fy);
+                store(at + 2 * NV, SC ? scale(cz, fz) : fz);
             } else if (A > 0) {
                 const int at = AX + (k - N) * NV, d = (k - N) / (A > 0 ? A : 1);
                 const Vec<NV, R> x = load(at);
