@@ -40,16 +40,17 @@ ADER_DEV Vec<NV, R> riemann_hll(const FaceSide<NV, R>& L, const FaceSide<NV, R>&
     return out;
 }
 
-// Euler: the textbook eigenvectors
+// Euler: the textbook eigenvectors.  (FP64 quotients and roots in the short forms of common.cuh: the four divisions and
+// the root of a face took about fifty FP64 instructions as IEEE sequences.)
 template <int D, class R>
 ADER_DEV Vec<5, R> riemann_linearized(const FaceSide<5, R>& L, const FaceSide<5, R>& Rt, R gamma, R gm1) {
     const Prim<5, R> pl = primitives(L.ub, gm1), pr = primitives(Rt.ub, gm1);
     const R rho = R(0.5) * (L.ub[0] + Rt.ub[0]);
     const R v[3] = {R(0.5) * (pl.vx + pr.vx), R(0.5) * (pl.vy + pr.vy), R(0.5) * (pl.vz + pr.vz)};
     const R p = R(0.5) * (pl.p + pr.p);
-    const R a2 = gamma * p / rho, a = sqrt(a2);
+    const R a2 = quot(gamma * p, rho), a = speed_root(a2);
     const R q2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    const R H = a2 / gm1 + R(0.5) * q2;
+    const R H = quot(a2, gm1) + R(0.5) * q2;
     constexpr int T1 = D == 0 ? 1 : 0, T2 = D == 2 ? 1 : 2;
     const R un = v[D], ut1 = v[T1], ut2 = v[T2];
     Vec<5, R> dU;
@@ -59,8 +60,8 @@ ADER_DEV Vec<5, R> riemann_linearized(const FaceSide<5, R>& L, const FaceSide<5,
     const R at1 = dU[1 + T1] - ut1 * dU[0];
     const R at2 = dU[1 + T2] - ut2 * dU[0];
     const R d5 = dU[4] - at1 * ut1 - at2 * ut2;
-    const R a2s = gm1 / a2 * (dU[0] * (H - un * un) + un * dU[1 + D] - d5);
-    const R a1s = (dU[0] * (un + a) - dU[1 + D] - a * a2s) / (R(2) * a);
+    const R a2s = quot(gm1, a2) * (dU[0] * (H - un * un) + un * dU[1 + D] - d5);
+    const R a1s = quot(dU[0] * (un + a) - dU[1 + D] - a * a2s, R(2) * a);
     const R a5s = dU[0] - a1s - a2s;
     const R l1 = fabs(un - a), l2 = fabs(un), l5 = fabs(un + a);
     const R s1 = l1 * a1s, s2 = l2 * a2s, s5 = l5 * a5s, st1 = l2 * at1, st2 = l2 * at2;
@@ -112,8 +113,8 @@ ADER_DEV Vec<8, R> mhd_abs_jacobian_apply(R rho, const R* v, R p, const R* B, R 
     const R bt = speed_root(by * by + bz * bz);
     R ey = R(0.70710678118654752), ez = R(0.70710678118654752);
     if (bt > tiny * speed_root(rho * sum)) {
-        ey = by / bt;
-        ez = bz / bt;
+        ey = quot(by, bt);
+        ez = quot(bz, bt);
     }
     const R sg = bx >= R(0) ? R(1) : R(-1);
     // primitive jump
@@ -130,9 +131,9 @@ ADER_DEV Vec<8, R> mhd_abs_jacobian_apply(R rho, const R* v, R p, const R* B, R 
     const R fc = af * cf, sc = as * cs;
     const R idet = rcp(fc * fc + sc * sc);
     const R Fd = (fc * du - sc * sg * dvpar) * idet, Sd = (sc * du + fc * sg * dvpar) * idet;
-    const R X = dp * irho / a2, Y = dbpar * isr / a;
+    const R X = quot(dp * irho, a2), Y = quot(dbpar * isr, a);
     const R Fs = af * X + as * Y, Ss = as * X - af * Y;
-    const R E = drho - dp / a2;
+    const R E = drho - quot(dp, a2);
     // scaled by |lambda|
     const R wE = fabs(u) * E;
     const R wFp = fabs(u + cf) * R(0.5) * (Fs + Fd), wFm = fabs(u - cf) * R(0.5) * (Fs - Fd);
@@ -153,10 +154,10 @@ ADER_DEV Vec<8, R> mhd_abs_jacobian_apply(R rho, const R* v, R p, const R* B, R 
     out[1 + D] = u * Drho + rho * Du;
     out[1 + T1] = vt1 * Drho + rho * Dv;
     out[1 + T2] = vt2 * Drho + rho * Dw;
-    out[4] = R(0.5) * q2 * Drho + rho * (u * Du + vt1 * Dv + vt2 * Dw) + Dp / gm1 + by * Dby + bz * Dbz;
+    out[4] = R(0.5) * q2 * Drho + rho * (u * Du + vt1 * Dv + vt2 * Dw) + quot(Dp, gm1) + by * Dby + bz * Dbz;
     out[5 + D] = R(0);
-    out[5 + T1] = Dby / k;
-    out[5 + T2] = Dbz / k;
+    out[5 + T1] = quot(Dby, k);
+    out[5 + T2] = quot(Dbz, k);
     return out;
 }
 
