@@ -972,6 +972,8 @@ def gpu_arm(args):
         bound, peak = "alu", alu_peak_tflops(args.fp32, 2070.0)
         basis = "derived: 152 SM x %s at 2070 MHz max clock" % (
             "128 FFMA/clk" if args.fp32 else "2 DFMA/clk (1.25 TFLOP/s nominal FP64)")
+        if not args.fp32:     # the count is of the formulas' FLOPs
+            basis += "; most sums, the WENO weights and the reciprocals run on the integer units, so frac may pass 1"
     total_ms = sum(v[1] for v in prof.values())
     roofline = {"bound": bound, "kernel": kname, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak if achieved else None,

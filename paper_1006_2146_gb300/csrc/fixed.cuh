@@ -10,9 +10,10 @@
 // unit, 2^-(53 + LSH) of the largest.  A node state then carries an error of a few such units before it is
 // rounded once to FP64, where the FP64 sum rounds at every operation to 2^-53 of its partial sums.
 //
-// Measured (FP64, face states): the third-order tile kernel of 64 x 128 x 128 zones 6.28 -> 4.71 ms, 3224 -> 2116
-// FP64 instructions a zone; the step of 256^3 zones 147.7 -> 124.7 ms, of 93 x 75 x 110 zones at second order
-// 3.10 -> 2.74 ms.
+// Measured (FP64): face states alone took the third-order predictor of 64 x 128 x 128 zones, one thread a zone, from
+// 6.28 to 4.71 ms (3224 -> 2116 FP64 instructions a zone); with the sums of flux modes, teams of warps (team.cuh) and
+// the reciprocals (common.cuh) it takes 2.5 ms and about 1000.  The nodal fourth-order step of 56^3 zones fell from
+// 5.60 to 3.19 ms when its tables moved here.
 //
 // Range.  HEADROOM = 10 - LSH bits are left above the largest mode for sums; intermediate sums may wrap (the
 // arithmetic is modulo 2^64) as long as no wrapped value is shifted or scaled by a fraction.  Modes of magnitude
@@ -247,11 +248,11 @@ struct AxisScale<FixFrame<NV, LSH>> {
     }
 };
 
-// Sum of the Euler flux of direction D over face nodes, kept by its factors so that a node costs few FP64
-// instructions: with r = 1 / rho, v = m_D r and w = |m|^2 r (twice the kinetic energy) the node adds m_i v to the
+// Sum of the Euler flux of direction D over face nodes, kept by its factors so that a node costs few
+// instructions (FP32 faces, one thread a zone): with r = 1 / rho, v = m_D r and w = |m|^2 r (twice the kinetic energy) the node adds m_i v to the
 // momentum products, E v and w v to the energy's and w to the pressure's.  The pressure P = (gamma - 1)(E - w / 2)
 // is applied to the sums, and the weighted sums of m_D and E themselves are the face averages of the state (the
-// facial quadrature is exact on its basis).  14 FP64 instructions a node where the flux and its addition took 22.
+// facial quadrature is exact on its basis).  14 instructions a node where the flux and its addition took 22.
 template <int D, class R>
 struct FluxSum {
     R p[3] = {R(0), R(0), R(0)}, w = R(0), ev = R(0), wv = R(0);

@@ -449,6 +449,8 @@ ADER_DEV void store_update(const StepArgs& a, double* out, const double* base, d
     if (bad && !a.defer_nonfinite) raise_flag(a.flag, FLAG_NONFINITE);
 }
 
+// both faces of each direction solved for one zone (the form zone_flux_update_pair carries in FP32 pairs; counted by
+// flopcount)
 template <int SOLVER, int NV, class R>
 ADER_DEV void zone_flux_update(const StepArgs& a, double* out, const double* base, double c_host, int use_dt_dev,
                                long long z) {
