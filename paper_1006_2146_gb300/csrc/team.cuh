@@ -42,11 +42,17 @@ struct SerialTeam {
 #pragma unroll
         for (int k = 0; k < N; ++k) {
             const Prim<NV, R> q = primitives(u[k], gm1);
-            V fx, fy, fz;
-            fluxes_from(u[k], q, fx, fy, fz);
-            f[k] = SC ? scale(kx, fx) : fx;
-            g[k] = SC ? scale(ky, fy) : fy;
-            h[k] = SC ? scale(kz, fz) : fz;
+            if constexpr (sizeof(R) == 4) {     // (the three-way form costs 4% of a nodal fourth-order step here)
+                f[k] = SC ? scale(kx, flux_from<0>(u[k], q)) : flux_from<0>(u[k], q);
+                g[k] = SC ? scale(ky, flux_from<1>(u[k], q)) : flux_from<1>(u[k], q);
+                h[k] = SC ? scale(kz, flux_from<2>(u[k], q)) : flux_from<2>(u[k], q);
+            } else {
+                V fx, fy, fz;
+                fluxes_from(u[k], q, fx, fy, fz);
+                f[k] = SC ? scale(kx, fx) : fx;
+                g[k] = SC ? scale(ky, fy) : fy;
+                h[k] = SC ? scale(kz, fz) : fz;
+            }
         }
 #pragma unroll
         for (int k = 0; k < A; ++k) f[N + k] = SC ? flux_scaled<0>(u[N + k], gm1, kx) : flux<0>(u[N + k], gm1);
