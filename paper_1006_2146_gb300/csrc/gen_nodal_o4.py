@@ -202,8 +202,31 @@ def mode_coefficients(C):
             for d in range(3)]
 
 
+HEADROOM = 256          # the integer frame of the update's sums holds this many times the largest entered flux (fixed.cuh)
+
+
+def _flux_functional(terms, functionals):
+    """The linear combination {name: coefficient} in terms of the node fluxes."""
+    out = {}
+    for name, c in terms.items():
+        for j, x in functionals[name].items():
+            out[j] = out.get(j, Fr(0)) + c * x
+    return out
+
+
+def _check_headroom(terms, functionals):
+    """Every operand of a product with a fraction, and the sum itself, stays inside the frame for any signs of the fluxes."""
+    norm = lambda t: sum(abs(x) for x in _flux_functional(t, functionals).values())
+    assert norm(terms) < HEADROOM
+    for c in set(abs(x) for x in terms.values() if x != 0):
+        operand = {n: x / c for n, x in terms.items() if abs(x) == c}
+        if c.denominator != 1:
+            assert norm(operand) < HEADROOM, (operand, float(norm(operand)))
+
+
 def emit_modes(C):
-    """The update for scalars whose sums cost less than their products (zone-scaled integers)."""
+    """The update for scalars whose sums cost less than their products (zone-scaled integers), one flux direction at a
+    time: the sums of one direction stay inside the integers' headroom, those of all three would not."""
     D = mode_coefficients(C)
     lines = ["// the tau = 0 node at the spatial point of node 21 + k",
              "ADER_DEV constexpr int nodal_o4_base(int k) {",
@@ -211,25 +234,37 @@ def emit_modes(C):
              "    return b[k];",
              "}",
              "",
-             "// The same update where additions are cheap (fixed.cuh).  The tau = 0 terms from the flux modes of the",
-             "// twenty nodes, f[m], g[m], h[m] (scaled, m = 2..20): dq[k-21], without u[base(k)].",
-             "template <class V>",
-             "ADER_DEV void nodal_o4_qterms_modes(const V* f, const V* g, const V* h, V* dq) {"]
-    row = {k: {"%s[%d]" % (a, m): D[d][k][m] for d, a in enumerate("fgh") for m in range(1, 21)} for k in range(21, 36)}
-    for base, name, ks in ((21, "q1", range(21, 31)), (31, "q2", range(31, 35))):     # tau = 1/3 and tau = 2/3
-        lines.append("    const V %s = %s;" % (name, _grouped(row[base]).lstrip("+ ")))
-        for k in ks:
-            d = {n: row[k][n] - row[base][n] for n in row[k]}
-            lines.append("    dq[%d] = %s%s;" % (k - 21, name, "".join("\n        " + x for x in [_grouped(d)] if x)))
-    lines.append("    dq[14] = %s;" % _grouped(row[35]).lstrip("+ "))
-    lines += ["}", "",
-              "// one Picard step without qt: de[k-21], from the scaled fluxes at the nodes tau > 0 (index node - 21)",
-              "template <class V>",
-              "ADER_DEV void nodal_o4_update_terms(const V* f, const V* g, const V* h, V* de) {"]
-    for k in range(21, 36):
-        t = {"%s[%d]" % (a, j - 21): C[d][k][j] for d, a in enumerate("fgh") for j in range(21, 36)}
-        lines.append("    de[%d] = %s;" % (k - 21, _grouped(t).lstrip("+ ")))
-    return lines + ["}", ""]
+             "// The same update where additions are cheap (fixed.cuh), for the flux of direction DIR alone.  The tau = 0 terms",
+             "// from the flux modes f[2..20] of the twenty nodes: dq[k-21], without u[base(k)] and the scale dt / dx.",
+             "template <int DIR, class V>",
+             "ADER_DEV void nodal_o4_qterms_modes(const V* f, V* dq) {"]
+    V0i = _inverse([[_phi(m, p) for m in MODES[:20]] for p in NODES[:20]])
+    modes = {"f[%d]" % (m + 1): {j: V0i[m][j] for j in range(20)} for m in range(20)}
+    for d in range(3):
+        row = {k: {"f[%d]" % m: D[d][k][m] for m in range(1, 21)} for k in range(21, 36)}
+        lines.append("    %sif constexpr (DIR == %d) {" % ("} else " if d else "", d) if d < 2 else "    } else {")
+        for base, name, ks in ((21, "q1", range(21, 31)), (31, "q2", range(31, 35))):     # tau = 1/3 and tau = 2/3
+            _check_headroom(row[base], modes)
+            lines.append("        const V %s = %s;" % (name, _grouped(row[base]).lstrip("+ ")))
+            for k in ks:
+                t = {n: row[k][n] - row[base][n] for n in row[k]}
+                _check_headroom(t, modes)
+                _check_headroom(row[k], modes)
+                lines.append("        dq[%d] = %s%s;" % (k - 21, name, "".join("\n        " + x for x in [_grouped(t)] if x)))
+        _check_headroom(row[35], modes)
+        lines.append("        dq[14] = %s;" % _grouped(row[35]).lstrip("+ "))
+    lines += ["    }", "}", "",
+              "// one Picard step without qt: de[k-21], from the fluxes of direction DIR at the nodes tau > 0 (index node - 21)",
+              "template <int DIR, class V>",
+              "ADER_DEV void nodal_o4_update_terms(const V* f, V* de) {"]
+    nodes = {"f[%d]" % j: {j: Fr(1)} for j in range(15)}
+    for d in range(3):
+        lines.append("    %sif constexpr (DIR == %d) {" % ("} else " if d else "", d) if d < 2 else "    } else {")
+        for k in range(21, 36):
+            t = {"f[%d]" % (j - 21): C[d][k][j] for j in range(21, 36)}
+            _check_headroom(t, nodes)
+            lines.append("        de[%d] = %s;" % (k - 21, _grouped(t).lstrip("+ ")))
+    return [x.replace("\n", "\n    ") for x in lines] + ["    }", "}", ""]
 
 
 def emit():

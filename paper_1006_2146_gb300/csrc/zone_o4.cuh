@@ -412,7 +412,8 @@ ADER_DEV void nodal_o4_to_modes(const Vec<NV, R>* u, const Vec<NV, R>* e, Vec<NV
 }
 
 // The modes 2..20 of the polynomial through the values n[1..20] at the tau = 0 nodes of Eq. C.1: Eq. C.4 solved for the
-// modes, about 100 additions and 15 products.  The nodes' quarter points couple w14, w17 and w18 in a ring.
+// modes, about 100 additions and 15 products, up to 209 times the largest value.  The nodes' quarter points couple w14,
+// w17 and w18 in a ring.
 template <class V>
 ADER_DEV void nodal_o4_flux_modes(const V* n, V* m) {
     m[5] = 2.0 * (n[3] + n[4] - 2.0 * n[1]);
@@ -489,45 +490,40 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
 #pragma unroll
         for (int k = 1; k <= 20; ++k) u[k] = fr.leave(s[k]);
     }
-    // Eq. C.2 without sources: q-terms of the tau = 0 fluxes.  FP64 takes them from the fluxes' modes, in integers
-    // (sums of up to 210 fluxes); the sums over nodes took 879 multiply-adds a variable, an iteration's 282.
+    // Eq. C.2 without sources: q-terms of the tau = 0 fluxes.  FP64 takes them from the fluxes' modes, in integers; the
+    // sums over nodes took 879 multiply-adds a variable, an iteration's 282.  Each direction has a frame of its own: its
+    // sums reach 209 times the largest flux of the frame's 256 (the three directions together 627), and fluxes of
+    // different size keep their own bits.  dt / dx enters in FP64, as the directions' sums are added.
     constexpr bool INTS = !std::is_same<typename FR::S, R>::value;
     using FF = FR;
     using VF = VS;
-    const AxisScale<FF> c(t.cx, t.cy, t.cz);
     V qt[16];
     {
         V f[21], g[21], h[21];
         t.template fluxes<20, 0, !INTS>(u + 1, f + 1, g + 1, h + 1);
         if constexpr (INTS) {
-            FF ff;
+            auto terms = [&](auto dir, const V* x, R c) {
+                constexpr int DIR = decltype(dir)::value;
+                FF ff;
 #pragma unroll
-            for (int k = 1; k <= 20; ++k) {
-                ff.include(f[k]);
-                ff.include(g[k]);
-                ff.include(h[k]);
-            }
-            ff.close();
-            VF n[21], F[21], G[21], H[21], dq[15];
+                for (int k = 1; k <= 20; ++k) ff.include(x[k]);
+                ff.close();
+                VF n[21], F[21], dq[15];
 #pragma unroll
-            for (int k = 1; k <= 20; ++k) n[k] = ff.enter(f[k]);
-            nodal_o4_flux_modes(n, F);
+                for (int k = 1; k <= 20; ++k) n[k] = ff.enter(x[k]);
+                nodal_o4_flux_modes(n, F);
+                nodal_o4_qterms_modes<DIR>(F, dq);
 #pragma unroll
-            for (int k = 1; k <= 20; ++k) n[k] = ff.enter(g[k]);
-            nodal_o4_flux_modes(n, G);
+                for (int k = 0; k < 15; ++k) {
+                    const V s = scale(c, ff.leave(dq[k]));
+                    qt[k] = DIR == 0 ? s : qt[k] + s;
+                }
+            };
+            terms(std::integral_constant<int, 0>{}, f, t.cx);
+            terms(std::integral_constant<int, 1>{}, g, t.cy);
+            terms(std::integral_constant<int, 2>{}, h, t.cz);
 #pragma unroll
-            for (int k = 1; k <= 20; ++k) n[k] = ff.enter(h[k]);
-            nodal_o4_flux_modes(n, H);
-#pragma unroll
-            for (int k = 2; k <= 20; ++k) {
-                F[k] = c.template times<0>(F[k]);
-                G[k] = c.template times<1>(G[k]);
-                H[k] = c.template times<2>(H[k]);
-            }
-            nodal_o4_qterms_modes(F, G, H, dq);
-            const FF fo = c.out(ff);
-#pragma unroll
-            for (int k = 0; k < 15; ++k) qt[k] = u[nodal_o4_base(k)] + fo.leave(dq[k]);
+            for (int k = 0; k < 15; ++k) qt[k] = u[nodal_o4_base(k)] + qt[k];
         } else {
             nodal_o4_qterms(u, f, g, h, qt);
         }
@@ -574,25 +570,27 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         if constexpr (SRC) t.template sources<15>(e, *src, se);
         if (!t.waits(done)) {                  // Eq. C.3
             if constexpr (INTS) {
-                FF fi;
-                VF F[15], G[15], H[15], de[15];
+                auto terms = [&](auto dir, const V* x, R c) {
+                    constexpr int DIR = decltype(dir)::value;
+                    FF fi;
 #pragma unroll
-                for (int k = 0; k < 14; ++k) {
-                    fi.include(f[k]);
-                    fi.include(g[k]);
-                    fi.include(h[k]);
-                }
-                fi.close();
+                    for (int k = 0; k < 14; ++k) fi.include(x[k]);
+                    fi.close();
+                    VF F[15], de[15];
 #pragma unroll
-                for (int k = 0; k < 14; ++k) {
-                    F[k] = c.template times<0>(fi.enter(f[k]));
-                    G[k] = c.template times<1>(fi.enter(g[k]));
-                    H[k] = c.template times<2>(fi.enter(h[k]));
-                }
-                nodal_o4_update_terms(F, G, H, de);
-                const FF fo = c.out(fi);
+                    for (int k = 0; k < 14; ++k) F[k] = fi.enter(x[k]);
+                    nodal_o4_update_terms<DIR>(F, de);
 #pragma unroll
-                for (int k = 0; k < 15; ++k) e[k] = qt[k] + fo.leave(de[k]);
+                    for (int k = 0; k < 15; ++k) {
+                        const V s = scale(c, fi.leave(de[k]));
+                        e[k] = DIR == 0 ? s : e[k] + s;
+                    }
+                };
+                terms(std::integral_constant<int, 0>{}, f, t.cx);
+                terms(std::integral_constant<int, 1>{}, g, t.cy);
+                terms(std::integral_constant<int, 2>{}, h, t.cz);
+#pragma unroll
+                for (int k = 0; k < 15; ++k) e[k] = qt[k] + e[k];
             } else {
                 nodal_o4_update(qt, f, g, h, e);
             }
