@@ -6,9 +6,15 @@
 // of one variable share the exponent of the largest of them, q = mode * 2^s, and sums and differences of q are
 // exact.  Only the products and quotients of the fluxes stay FP64.
 //
-// Precision.  The largest mode keeps all its 53 bits and LSH more below them; the others are cut at the same
-// unit, 2^-(53 + LSH) of the largest.  A node state then carries an error of a few such units before it is
-// rounded once to FP64, where the FP64 sum rounds at every operation to 2^-53 of its partial sums.
+// Precision.  The largest value of a frame keeps all its 53 bits and LSH more below them; the others are cut at the same
+// unit, 2^-(53 + LSH) of the largest.  A sum then carries an error of a few such units before it is rounded once to
+// FP64, where an FP64 sum rounds at every operation to 2^-53 of its partial sums.  With the frame's largest value among
+// a sum's terms the integers' error is the smaller one.  A sum of terms that are all small beside the largest value of
+// the frame keeps that absolute error, where FP64 would keep a relative one.  Frames therefore hold values that enter
+// the same sums: the modes of one variable of a zone (every node state has the mean in it), the fluxes of one variable
+// in one direction (the pressure sets the size of one direction's momentum flux and is absent from the others'), and
+// the differences of one WENO stencil.  What is left: a variable whose mean is far below its variation along one axis
+// holds its variation along another to 2^-58 of the larger one (order 4: 2^-56) instead of to its own last place.
 //
 // Measured (FP64): face states alone took the third-order predictor of 64 x 128 x 128 zones, one thread a zone, from
 // 6.28 to 4.71 ms (3224 -> 2116 FP64 instructions a zone); with the sums of flux modes, teams of warps (team.cuh) and
@@ -198,16 +204,11 @@ struct FixFrame {
     }
 };
 
-// Multiplication of flux modes by c_d = dt / dx_d inside a frame.  For integers c_d is a 63-bit integer with the
-// exponent of the largest of the three, the product the upper half of 128 bits; out() is the frame of the products.
+// Multiplication of integers by c_d = dt / dx_d inside a frame: c_d is a 63-bit integer with the exponent of the largest
+// of the three, the product the upper half of 128 bits; out() is the frame of the products.  The bits of an axis are cut
+// at the unit of the largest c (an axis 2^10 times wider loses one and more), so the predictors scale in FP64, behind a
+// direction's sum; the host check of the frames holds this form.
 template <class FR> struct AxisScale;
-template <int NV, class R>
-struct AxisScale<PlainFrame<NV, R>> {
-    R c[3];
-    ADER_DEV AxisScale(R cx, R cy, R cz) : c{cx, cy, cz} {}
-    template <int D> ADER_DEV Vec<NV, R> times(const Vec<NV, R>& f) const { return ader::scale(c[D], f); }
-    ADER_DEV PlainFrame<NV, R> out(const PlainFrame<NV, R>& f) const { return f; }
-};
 template <int NV, int LSH>
 struct AxisScale<FixFrame<NV, LSH>> {
     long long c[3];

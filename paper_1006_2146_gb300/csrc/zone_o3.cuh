@@ -64,50 +64,52 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
 #pragma unroll
         for (int k = 1; k <= 13; ++k) u[k] = fr.leave(s[k]);
     }
-    // fluxes at the tau = 0 nodes, built once (Sec. IV.2); the sums of Eqs. 40-42 and 36 in the state scalar (up to
-    // 32 times a flux)
+    // fluxes at the tau = 0 nodes, built once (Sec. IV.2); the sums of Eqs. 40-42 in the state scalar (up to 16 times a
+    // flux), one frame per direction, and Eq. 36's sum over the directions in R
     V e11, e13, e14, e15;       // Eq. 36 without sources: the modes fed by tau = 0 fluxes alone
     {
         using FF = typename FrameAt<2, NL, R>::T;
         using VF = Vec<NL, typename FF::S>;
         V fn[14], gn[14], hn[14];
         t.template fluxes<13, 0, false>(u + 1, fn + 1, gn + 1, hn + 1);
-        FF ff;
-        VF f[14], g[14], h[14];
+        // one direction after the other: the values of one frame at a time
+        auto enter = [&](const V* x, FF& ff, VF* f) {
 #pragma unroll
-        for (int n = 1; n <= 13; ++n) {
-            ff.include(fn[n]);
-            ff.include(gn[n]);
-            ff.include(hn[n]);
-        }
-        ff.close();
+            for (int n = 1; n <= 13; ++n) ff.include(x[n]);
+            ff.close();
 #pragma unroll
-        for (int n = 1; n <= 13; ++n) {
-            f[n] = ff.enter(fn[n]);
-            g[n] = ff.enter(gn[n]);
-            h[n] = ff.enter(hn[n]);
+            for (int n = 1; n <= 13; ++n) f[n] = ff.enter(x[n]);
+        };
+        {
+            FF ff;
+            VF f[14];
+            enter(fn, ff, f);
+            const VF q1 = f[2] + f[3] + f[4] + f[5], q2 = f[6] + f[7] + f[8] + f[9], q3 = f[10] + f[11] + f[12] + f[13];
+            e11 = scale(cx, ff.leave(0.25 * (q1 - q2)));                                // F2
+            e13 = scale(cx, ff.leave(2.0 * (0.5 * (q1 + q2 - q3) - 2.0 * f[1])));       // 2 F5
+            e14 = scale(cx, ff.leave(f[2] - f[3] - f[6] + f[7]));                       // F8
+            e15 = scale(cx, ff.leave(f[4] - f[5] - f[8] + f[9]));                       // F10
         }
-        const AxisScale<FF> c(cx, cy, cz);
-        const FF fo = c.out(ff);
-        const VF q1 = f[2] + f[3] + f[4] + f[5], q2 = f[6] + f[7] + f[8] + f[9], q3 = f[10] + f[11] + f[12] + f[13];
-        const VF F2 = c.template times<0>(0.25 * (q1 - q2));
-        const VF F5 = c.template times<0>(0.5 * (q1 + q2 - q3) - 2.0 * f[1]);
-        const VF F8 = c.template times<0>(f[2] - f[3] - f[6] + f[7]);
-        const VF F10 = c.template times<0>(f[4] - f[5] - f[8] + f[9]);
-        const VF q4 = g[2] + g[6] + g[10] + g[12], q5 = g[3] + g[7] + g[11] + g[13], q6 = g[4] + g[5] + g[8] + g[9];
-        const VF G3 = c.template times<1>(0.25 * (q4 - q5));
-        const VF G6 = c.template times<1>(0.5 * (q4 + q5 - q6) - 2.0 * g[1]);
-        const VF G8 = c.template times<1>(g[2] - g[3] - g[6] + g[7]);
-        const VF G9 = c.template times<1>(g[10] - g[11] - g[12] + g[13]);
-        const VF q7 = h[4] + h[8] + h[10] + h[11], q8 = h[5] + h[9] + h[12] + h[13], q9 = h[2] + h[3] + h[6] + h[7];
-        const VF H4 = c.template times<2>(0.25 * (q7 - q8));
-        const VF H7 = c.template times<2>(0.5 * (q7 + q8 - q9) - 2.0 * h[1]);
-        const VF H9 = c.template times<2>(h[10] - h[11] - h[12] + h[13]);
-        const VF H10 = c.template times<2>(h[4] - h[5] - h[8] + h[9]);
-        e11 = fo.leave(-(F2 + G3 + H4));
-        e13 = fo.leave(-(2.0 * F5 + G8 + H10));
-        e14 = fo.leave(-(F8 + 2.0 * G6 + H9));
-        e15 = fo.leave(-(F10 + G9 + 2.0 * H7));
+        {
+            FF ff;
+            VF g[14];
+            enter(gn, ff, g);
+            const VF q4 = g[2] + g[6] + g[10] + g[12], q5 = g[3] + g[7] + g[11] + g[13], q6 = g[4] + g[5] + g[8] + g[9];
+            e11 += scale(cy, ff.leave(0.25 * (q4 - q5)));                               // G3
+            e13 += scale(cy, ff.leave(g[2] - g[3] - g[6] + g[7]));                      // G8
+            e14 += scale(cy, ff.leave(2.0 * (0.5 * (q4 + q5 - q6) - 2.0 * g[1])));      // 2 G6
+            e15 += scale(cy, ff.leave(g[10] - g[11] - g[12] + g[13]));                  // G9
+        }
+        {
+            FF ff;
+            VF h[14];
+            enter(hn, ff, h);
+            const VF q7 = h[4] + h[8] + h[10] + h[11], q8 = h[5] + h[9] + h[12] + h[13], q9 = h[2] + h[3] + h[6] + h[7];
+            e11 = -(e11 + scale(cz, ff.leave(0.25 * (q7 - q8))));                       // H4
+            e13 = -(e13 + scale(cz, ff.leave(h[4] - h[5] - h[8] + h[9])));              // H10
+            e14 = -(e14 + scale(cz, ff.leave(h[10] - h[11] - h[12] + h[13])));          // H9
+            e15 = -(e15 + scale(cz, ff.leave(2.0 * (0.5 * (q7 + q8 - q9) - 2.0 * h[1]))));   // 2 H7
+        }
     }
     // source modes from the tau = 0 nodes (Eqs. 40-43 with f, g, h -> s), built once
     V S1, S2, S3, S4, s1;
@@ -147,7 +149,7 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         // Eqs. 40-42 give F13 = 2 (cx (f14 - f15) - F2) and so on, and Eq. 36 u12 = -(F13 + G14 + H15) / 2 =
         // -u11 - sum_d c_d (f_d(upper) - f_d(lower))
         V n11 = e11;
-        V n12 = -e11 - (ft[0] - ft[1] + gt[0] - gt[1] + ht[0] - ht[1]);
+        V n12 = -e11 - ((ft[0] - ft[1]) + (gt[0] - gt[1]) + (ht[0] - ht[1]));
         V n13 = e13, n14 = e14, n15 = e15;
         if constexpr (SRC) {
             const V us[7] = {ut[0], ut[1], ut[2], ut[3], ut[4], ut[5], u[1] + m[11] + m[12]};
@@ -238,42 +240,40 @@ ADER_DEV void predict_nodal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
     // (1.5 f1 - f2 - f3 / 2 = -A and f2 + f3 - 2 f1 = A + X / 2), for y and z the same with the axes exchanged.
     V q11, q12, q13, q14, q15;
     {
-        // all directions at nodes 1, 2, 4, 6, 8, 9, 10; x alone at 3, y at 5, z at 7; the sums in the state scalar
+        // all directions at nodes 1, 2, 4, 6, 8, 9, 10; x alone at 3, y at 5, z at 7; the differences of a direction in
+        // the state scalar, one frame per direction, and their sum in R
         using FF = typename FrameAt<2, NL, R>::T;
         using VF = Vec<NL, typename FF::S>;
         const V un[10] = {u[1], u[2], u[4], u[6], u[8], u[9], u[10], u[3], u[5], u[7]};
         V fn[8], gn[8], hn[8];
         t.template fluxes<7, 1, false>(un, fn, gn, hn);
-        FF ff;
+        FF ff, fg, fh;
         VF f[8], g[8], h[8];
 #pragma unroll
         for (int n = 0; n < 8; ++n) {
             if (n != 4) ff.include(fn[n]);
-            if (n != 5) ff.include(gn[n]);
-            if (n != 6) ff.include(hn[n]);
+            if (n != 5) fg.include(gn[n]);
+            if (n != 6) fh.include(hn[n]);
         }
         ff.close();
+        fg.close();
+        fh.close();
 #pragma unroll
         for (int n = 0; n < 8; ++n) {
             if (n != 4) f[n] = ff.enter(fn[n]);
-            if (n != 5) g[n] = ff.enter(gn[n]);
-            if (n != 6) h[n] = ff.enter(hn[n]);
+            if (n != 5) g[n] = fg.enter(gn[n]);
+            if (n != 6) h[n] = fh.enter(hn[n]);
         }
-        const AxisScale<FF> c(cx, cy, cz);
-        const FF fo = c.out(ff);
-        const VF X = c.template times<0>(f[7] - f[0]), Y = c.template times<1>(g[7] - g[0]);
-        const VF Z = c.template times<2>(h[7] - h[0]), half = 0.5 * (X + Y + Z);
-        const VF ax = c.template times<0>(f[1] - f[0]) + 0.5 * X, ay = c.template times<1>(g[2] - g[0]) + 0.5 * Y;
-        const VF az = c.template times<2>(h[3] - h[0]) + 0.5 * Z;
-        // the mixed differences of q12, q13, q14
-        const VF d12 = c.template times<1>(g[1] - g[6]) + c.template times<2>(h[1] - h[5]);
-        const VF d13 = c.template times<0>(f[2] - f[6]) + c.template times<2>(h[2] - h[4]);
-        const VF d14 = c.template times<0>(f[3] - f[5]) + c.template times<1>(g[3] - g[4]);
-        q11 = u[1] + fo.leave(half);
-        q12 = u[2] + fo.leave(d12 + (ay + az - ax));
-        q13 = u[4] + fo.leave(d13 + (ax + az - ay));
-        q14 = u[6] + fo.leave(d14 + (ax + ay - az));
-        q15 = u[1] + fo.leave(half + (ax + ay + az));   // u1 + sum_d c_d (A + X / 2)
+        auto sum = [&](const VF& x, const VF& y, const VF& z) {
+            return scale(cx, ff.leave(x)) + scale(cy, fg.leave(y)) + scale(cz, fh.leave(z));
+        };
+        const VF X = f[7] - f[0], Y = g[7] - g[0], Z = h[7] - h[0];
+        const VF ax = f[1] - f[0] + 0.5 * X, ay = g[2] - g[0] + 0.5 * Y, az = h[3] - h[0] + 0.5 * Z;
+        q11 = u[1] + 0.5 * sum(X, Y, Z);
+        q12 = u[2] + sum(-ax, g[1] - g[6] + ay, h[1] - h[5] + az);
+        q13 = u[4] + sum(f[2] - f[6] + ax, -ay, h[2] - h[4] + az);
+        q14 = u[6] + sum(f[3] - f[5] + ax, g[3] - g[4] + ay, -az);
+        q15 = u[1] + sum(0.5 * X + ax, 0.5 * Y + ay, 0.5 * Z + az);   // u1 + sum_d c_d (A + X / 2)
     }
     V s0sum, s1;         // with a source: s2 + ... + s7 and s1 (nodes 1-7, built once)
     if constexpr (SRC) {          // Eq. B.2, source terms

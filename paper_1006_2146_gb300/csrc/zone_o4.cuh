@@ -57,11 +57,10 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         s[21] = s[19] + s[20] - s[18] + w[9] - 0.5 * w[20];
     }
 
-    // tau = 0 parts of Eqs. 49-51 (built once), in the state scalar: sums of up to 110 fluxes
+    // tau = 0 parts of Eqs. 49-51 (built once), in the state scalar: sums of up to 212 fluxes, a frame per direction
     using FF = typename FrameAt<2, NL, R>::T;
     using VF = Vec<NL, typename FF::S>;
-    const AxisScale<FF> c(cx, cy, cz);
-    FF ff;
+    FF ff, fg, fh;
     VF F2, F5, F8, F10, F11, F20, PF14, PF15, PF16, QF12;
     VF G3, G6, G8, G9, G12, G20, PG14, PG15, PG16, QG34;
     VF H4, H7, H9, H10, H13, H20, PH14, PH15, PH16, QH56;
@@ -74,15 +73,17 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
 #pragma unroll
         for (int k = 1; k <= 21; ++k) {
             ff.include(fn[k]);
-            ff.include(gn[k]);
-            ff.include(hn[k]);
+            fg.include(gn[k]);
+            fh.include(hn[k]);
         }
         ff.close();
+        fg.close();
+        fh.close();
 #pragma unroll
         for (int k = 1; k <= 21; ++k) {
             f[k] = ff.enter(fn[k]);
-            g[k] = ff.enter(gn[k]);
-            h[k] = ff.enter(hn[k]);
+            g[k] = fg.enter(gn[k]);
+            h[k] = fh.enter(hn[k]);
         }
         // q1..q6 of Eqs. 49-51 (corner sums), per flux
         const VF fq1 = f[14] + f[15] + f[16] + f[17], fq2 = f[18] + f[19] + f[20] + f[21];
@@ -235,11 +236,16 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         for (int k = 23; k <= (SRC ? 42 : 41); ++k) out[k] = fw.leave(x[k]);
     };
     // Eq. 45 without sources: the modes fed by tau = 0 fluxes only
-    const FF fo = c.out(ff);
-    const V e21 = fo.leave(-(c.template times<0>(F2 + 0.1 * F11) + c.template times<1>(G3 + 0.1 * G12) + c.template times<2>(H4 + 0.1 * H13)));
-    const V e24 = fo.leave(-(c.template times<0>(2.0 * F5) + c.template times<1>(G8) + c.template times<2>(H10)));
-    const V e25 = fo.leave(-(c.template times<0>(F8) + c.template times<1>(2.0 * G6) + c.template times<2>(H9)));
-    const V e26 = fo.leave(-(c.template times<0>(F10) + c.template times<1>(G9) + c.template times<2>(2.0 * H7)));
+    V e21, e24, e25, e26;
+    {
+        auto sum = [&](const VF& x, const VF& y, const VF& z) {
+            return scale(cx, ff.leave(x)) + scale(cy, fg.leave(y)) + scale(cz, fh.leave(z));
+        };
+        e21 = -sum(F2 + 0.1 * F11, G3 + 0.1 * G12, H4 + 0.1 * H13);
+        e24 = -sum(2.0 * F5, G8, H10);
+        e25 = -sum(F8, 2.0 * G6, H9);
+        e26 = -sum(F10, G9, 2.0 * H7);
+    }
 
     const bool conv = positive_arg(ctl.tol);
     const int cap = conv ? ctl.max_iter : ctl.n_iter;
@@ -253,24 +259,33 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
         // fluxes at nodes 23..35 (all three directions) and the axis nodes 36..41
         V fn[38], gn[38], hn[38];
         t.template fluxes<13, 2, false>(w + 23, fn + 23, gn + 23, hn + 23);
-        FF fi;
+        FF fi, gi, hi;
         VF f[38], g[38], h[38];
 #pragma unroll
         for (int k = 23; k <= 37; ++k) {
             fi.include(fn[k]);
-            fi.include(gn[k]);
-            fi.include(hn[k]);
+            gi.include(gn[k]);
+            hi.include(hn[k]);
         }
         fi.close();
+        gi.close();
+        hi.close();
         fi.join(ff);
+        gi.join(fg);
+        hi.join(fh);
 #pragma unroll
         for (int k = 23; k <= 37; ++k) {
             f[k] = fi.enter(fn[k]);
-            g[k] = fi.enter(gn[k]);
-            h[k] = fi.enter(hn[k]);
+            g[k] = gi.enter(gn[k]);
+            h[k] = hi.enter(hn[k]);
         }
-        const FF fio = c.out(fi);
-        auto keep = [&](const VF& x) { return fi.from(ff, x); };      // a tau = 0 part in this iterate's frame
+        // a tau = 0 part in this iterate's frame
+        auto keepx = [&](const VF& x) { return fi.from(ff, x); };
+        auto keepy = [&](const VF& x) { return gi.from(fg, x); };
+        auto keepz = [&](const VF& x) { return hi.from(fh, x); };
+        auto sum = [&](const VF& x, const VF& y, const VF& z) {
+            return scale(cx, fi.leave(x)) + scale(cy, gi.leave(y)) + scale(cz, hi.leave(z));
+        };
         const VF f36 = f[36], f37 = f[37], g38 = g[36], g39 = g[37], h40 = h[36], h41 = h[37];
         // Eq. 49 (x)
         VF F14, F15, F16, F18, F24, F27, F30, F33, F35;
@@ -279,15 +294,15 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
             const VF q8 = f[23] + f[27] - f[24] - f[28] - f[31] - f[33] + f[32] + f[34];
             const VF q9 = f[25] + f[29] - f[26] - f[30] - f[31] - f[32] + f[33] + f[34];
             const VF q10 = f[23] + f[24] + f[25] + f[26] - f[27] - f[28] - f[29] - f[30];
-            F14 = q8 + keep(PF14);
-            F15 = q9 + keep(PF15);
-            F16 = q7 + keep(PF16);
+            F14 = q8 + keepx(PF14);
+            F15 = q9 + keepx(PF15);
+            F16 = q7 + keepx(PF16);
             F18 = -2.0 * q7 + F16;
-            F27 = 1.125 * keep(QF12) + 4.5 * (f36 - f37) - 2.25 * q10;
+            F27 = 1.125 * keepx(QF12) + 4.5 * (f36 - f37) - 2.25 * q10;
             F24 = 3.0 * (f36 - f37) - 0.75 * q10 + 0.375 * (F16 + F18) - F27;
-            F30 = 3.0 * (f36 - 2.0 * f[35] + f37) - 1.5 * keep(F5);
-            F33 = 3.0 * (f[23] - f[27] - f[24] + f[28]) - 3.0 * keep(F8);
-            F35 = 3.0 * (f[25] - f[29] - f[26] + f[30]) - 3.0 * keep(F10);
+            F30 = 3.0 * (f36 - 2.0 * f[35] + f37) - 1.5 * keepx(F5);
+            F33 = 3.0 * (f[23] - f[27] - f[24] + f[28]) - 3.0 * keepx(F8);
+            F35 = 3.0 * (f[25] - f[29] - f[26] + f[30]) - 3.0 * keepx(F10);
         }
         // Eq. 50 (y)
         VF G14, G16, G17, G19, G25, G28, G31, G33, G34;
@@ -296,16 +311,16 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
             const VF q8 = g[23] + g[27] - g[24] - g[28] - g[31] - g[33] + g[32] + g[34];
             const VF q9 = g[25] + g[29] - g[26] - g[30] - g[31] - g[32] + g[33] + g[34];
             const VF q11 = g[23] - g[24] + g[27] - g[28] + g[31] - g[32] + g[33] - g[34];
-            G14 = q8 + keep(PG14);
-            const VF G15 = q9 + keep(PG15);
-            G16 = q7 + keep(PG16);
+            G14 = q8 + keepy(PG14);
+            const VF G15 = q9 + keepy(PG15);
+            G16 = q7 + keepy(PG16);
             G17 = -2.0 * q9 + G15;
             G19 = -2.0 * q8 + G14;
-            G28 = 1.125 * keep(QG34) + 4.5 * (g38 - g39) - 2.25 * q11;
+            G28 = 1.125 * keepy(QG34) + 4.5 * (g38 - g39) - 2.25 * q11;
             G25 = 3.0 * (g38 - g39) - 0.75 * q11 + 0.375 * (G14 + G19) - G28;
-            G31 = 3.0 * (g38 - 2.0 * g[35] + g39) - 1.5 * keep(G6);
-            G33 = 3.0 * (g[23] - g[27] - g[24] + g[28]) - 3.0 * keep(G8);
-            G34 = 3.0 * (g[31] - g[32] - g[33] + g[34]) - 3.0 * keep(G9);
+            G31 = 3.0 * (g38 - 2.0 * g[35] + g39) - 1.5 * keepy(G6);
+            G33 = 3.0 * (g[23] - g[27] - g[24] + g[28]) - 3.0 * keepy(G8);
+            G34 = 3.0 * (g[31] - g[32] - g[33] + g[34]) - 3.0 * keepy(G9);
         }
         // Eq. 51 (z)
         VF H15, H17, H18, H19, H26, H29, H32, H34, H35;
@@ -314,35 +329,35 @@ ADER_DEV void predict_modal(const T& t, typename T::V* m, PredCtl& ctl, const Sr
             const VF q8 = h[23] + h[27] - h[24] - h[28] - h[31] - h[33] + h[32] + h[34];
             const VF q9 = h[25] + h[29] - h[26] - h[30] - h[31] - h[32] + h[33] + h[34];
             const VF q12 = h[25] - h[26] + h[29] - h[30] + h[31] + h[32] - h[33] - h[34];
-            const VF H14 = q8 + keep(PH14);
-            H15 = q9 + keep(PH15);
-            const VF H16 = q7 + keep(PH16);
+            const VF H14 = q8 + keepz(PH14);
+            H15 = q9 + keepz(PH15);
+            const VF H16 = q7 + keepz(PH16);
             H17 = -2.0 * q9 + H15;
             H18 = -2.0 * q7 + H16;
             H19 = -2.0 * q8 + H14;
-            H29 = 1.125 * keep(QH56) + 4.5 * (h40 - h41) - 2.25 * q12;
+            H29 = 1.125 * keepz(QH56) + 4.5 * (h40 - h41) - 2.25 * q12;
             H26 = 3.0 * (h40 - h41) - 0.75 * q12 + 0.375 * (H15 + H17) - H29;
-            H32 = 3.0 * (h40 - 2.0 * h[35] + h41) - 1.5 * keep(H7);
-            H34 = 3.0 * (h[31] - h[32] - h[33] + h[34]) - 3.0 * keep(H9);
-            H35 = 3.0 * (h[25] - h[26] - h[29] + h[30]) - 3.0 * keep(H10);
+            H32 = 3.0 * (h40 - 2.0 * h[35] + h41) - 1.5 * keepz(H7);
+            H34 = 3.0 * (h[31] - h[32] - h[33] + h[34]) - 3.0 * keepz(H9);
+            H35 = 3.0 * (h[25] - h[26] - h[29] + h[30]) - 3.0 * keepz(H10);
         }
         // Eq. 45 without sources
         V n[16];
         n[0] = e21;
-        n[1] = fio.leave(-0.5 * (c.template times<0>(F24) + c.template times<1>(G25) + c.template times<2>(H26)));
-        n[2] = fio.leave(-(1.0 / 3.0) * (c.template times<0>(F27) + c.template times<1>(G28) + c.template times<2>(H29)));
+        n[1] = -0.5 * sum(F24, G25, H26);
+        n[2] = -(1.0 / 3.0) * sum(F27, G28, H29);
         n[3] = e24;
         n[4] = e25;
         n[5] = e26;
-        n[6] = fio.leave(-(c.template times<0>(F30) + c.template times<1>(0.5 * G33) + c.template times<2>(0.5 * H35)));
-        n[7] = fio.leave(-(c.template times<0>(0.5 * F33) + c.template times<1>(G31) + c.template times<2>(0.5 * H34)));
-        n[8] = fio.leave(-(c.template times<0>(0.5 * F35) + c.template times<1>(0.5 * G34) + c.template times<2>(H32)));
-        n[9] = fio.leave(-(c.template times<0>(3.0 * keep(F11)) + c.template times<1>(G14) + c.template times<2>(H15)));
-        n[10] = fio.leave(-(c.template times<0>(F16) + c.template times<1>(3.0 * keep(G12)) + c.template times<2>(H17)));
-        n[11] = fio.leave(-(c.template times<0>(F18) + c.template times<1>(G19) + c.template times<2>(3.0 * keep(H13))));
-        n[12] = fio.leave(-(c.template times<0>(2.0 * F14) + c.template times<1>(2.0 * G16) + c.template times<2>(keep(H20))));
-        n[13] = fio.leave(-(c.template times<0>(keep(F20)) + c.template times<1>(2.0 * G17) + c.template times<2>(2.0 * H19)));
-        n[14] = fio.leave(-(c.template times<0>(2.0 * F15) + c.template times<1>(keep(G20)) + c.template times<2>(2.0 * H18)));
+        n[6] = -sum(F30, 0.5 * G33, 0.5 * H35);
+        n[7] = -sum(0.5 * F33, G31, 0.5 * H34);
+        n[8] = -sum(0.5 * F35, 0.5 * G34, H32);
+        n[9] = -sum(3.0 * keepx(F11), G14, H15);
+        n[10] = -sum(F16, 3.0 * keepy(G12), H17);
+        n[11] = -sum(F18, G19, 3.0 * keepz(H13));
+        n[12] = -sum(2.0 * F14, 2.0 * G16, keepz(H20));
+        n[13] = -sum(keepx(F20), 2.0 * G17, 2.0 * H19);
+        n[14] = -sum(2.0 * F15, keepy(G20), 2.0 * H18);
         if constexpr (SRC) {        // Eq. 45, source terms
             V ts[15];
             time_source_modes(w, ts);

@@ -97,19 +97,6 @@ struct SymFrame {
     }
 };
 template <int LSH, int NV> struct FrameAt<LSH, NV, Sym> { using T = SymFrame<NV, LSH>; };
-template <int NV, int LSH>
-struct AxisScale<SymFrame<NV, LSH>> {
-    AxisScale(Sym, Sym, Sym) {}
-    template <int D> Vec<NV, SymFix<LSH>> times(const Vec<NV, SymFix<LSH>>& f) const {
-        Vec<NV, SymFix<LSH>> r;
-        for (int i = 0; i < NV; ++i) {
-            operand(f[i].c, std::ldexp(1.0, 10 - LSH));
-            r[i] = combine(f[i], 0.5, f[i], 0);
-        }
-        return r;
-    }
-    SymFrame<NV, LSH> out(const SymFrame<NV, LSH>&) const { return {}; }
-};
 }  // namespace ader
 
 // input n: a mode (n below 1000) or the j-th flux of the k-th exchange (1000 k + j)
