@@ -119,9 +119,9 @@ ADER_DEV R w3_curv(R D2) { return fma(rn_mul(R(13.0 / 3.0), D2), D2, R(4.0 * WEN
 // part: squares and products of the t (the cleared denominators), a reciprocal and the weighted sum, 17 FP64
 // instructions for S = 3 and one output.  Here the products run as 64 x 64-bit integer products of normalised
 // mantissas (upper halves; 7.4 a clock and SM against 1.7 FP64 multiplications) with their exponents apart, and the
-// two sums are integers aligned to their largest term with 57 bits or more (56 for S = 4).  What stays FP64 is the quotient of the
-// sums: one reciprocal for all outputs and one product each.  Errors against 80-bit arithmetic are smaller than the
-// FP64 form's, and no intermediate value overflows.
+// two sums are integers aligned to their largest term with 57 bits or more (56 for S = 4).  What stays FP64 is the
+// quotient of the sums: one reciprocal for all outputs and one product each.  A sum's error is relative to its largest
+// term, as the FP64 form's was, and smaller; no intermediate value overflows.
 ADER_DEV unsigned long long u64_mulhi(unsigned long long a, unsigned long long b) {
 #ifdef __CUDA_ARCH__
     return __umul64hi(a, b);
@@ -285,33 +285,34 @@ ADER_DEV void weno3(const R* a, R& b, R& c) {
 template <class R>
 ADER_DEV void weno4(const R* a, R& b, R& c, R& d) {
     if constexpr (std::is_same<R, double>::value) {
-        // The candidates from the six neighbour differences e, as integers of a common exponent: 60 b, 2 c and 6 d
-        // of each stencil (sums of up to 200 e), and 3600 (EPS + IS) = T^2 + 3900 (2 c)^2 + 3905 (6 d)^2 + 3600 EPS
-        // with T = 60 b + 6 d.  34 FP64 instructions; all in FP64 it took 135.
-        FixFrame<1, 2> fr;
+        // The candidates from the six neighbour differences e, as integers with one exponent per stencil (three
+        // differences: the values of a smooth stencil beside a jump keep all their bits): 60 b, 2 c and 6 d of each
+        // stencil (sums of up to 200 e), and 3600 (EPS + IS) = T^2 + 3900 (2 c)^2 + 3905 (6 d)^2 + 3600 EPS with
+        // T = 60 b + 6 d.  35 FP64 instructions; all in FP64 it took 135.
         Vec<1, double> e[6];
 #pragma unroll
-        for (int j = 0; j < 6; ++j) {
-            e[j][0] = a[j + 1] - a[j];
-            fr.include(e[j]);
-        }
-        fr.close();
-        Fix x[6];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) x[j] = fr.enter(e[j])[0];
-        const Fix cb[4] = {109.0 * x[2] - 68.0 * x[1] + 19.0 * x[0], 19.0 * x[3] + 52.0 * x[2] - 11.0 * x[1],
-                           52.0 * x[3] + 19.0 * x[2] - 11.0 * x[4], 109.0 * x[3] - 68.0 * x[4] + 19.0 * x[5]};
-        const Fix cc[3] = {2.0 * x[2] - 3.0 * x[1] + x[0], x[3] - x[2], 3.0 * x[4] - 2.0 * x[3] - x[5]};
+        for (int j = 0; j < 6; ++j) e[j][0] = a[j + 1] - a[j];
         double B[4], C[4], D[4], t[4];
-        C[0] = fr.leave_one(0, cc[0]);
-        C[1] = C[2] = fr.leave_one(0, cc[1]);
-        C[3] = fr.leave_one(0, cc[2]);
+        C[1] = C[2] = e[3][0] - e[2][0];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const Fix cd = x[q + 2] - 2.0 * x[q + 1] + x[q];
-            B[q] = fr.leave_one(0, cb[q]);
+            FixFrame<1, 2> fr;
+            Fix x[3];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) fr.include(e[q + j]);
+            fr.close();
+#pragma unroll
+            for (int j = 0; j < 3; ++j) x[j] = fr.enter(e[q + j])[0];
+            const Fix cb = q == 0 ? 109.0 * x[2] - 68.0 * x[1] + 19.0 * x[0]
+                         : q == 1 ? 19.0 * x[2] + 52.0 * x[1] - 11.0 * x[0]
+                         : q == 2 ? 52.0 * x[1] + 19.0 * x[0] - 11.0 * x[2]
+                                  : 109.0 * x[0] - 68.0 * x[1] + 19.0 * x[2];
+            const Fix cd = x[2] - 2.0 * x[1] + x[0];
+            if (q == 0) C[0] = fr.leave_one(0, 2.0 * x[2] - 3.0 * x[1] + x[0]);
+            if (q == 3) C[3] = fr.leave_one(0, 3.0 * x[1] - 2.0 * x[0] - x[2]);
+            B[q] = fr.leave_one(0, cb);
             D[q] = fr.leave_one(0, cd);
-            const double T = fr.leave_one(0, cb[q] + cd);
+            const double T = fr.leave_one(0, cb + cd);
             t[q] = fma(T, T, fma(3900.0 * C[q], C[q], fma(3905.0 * D[q], D[q], 3600.0 * WENO_EPS)));
         }
         const IntWeights<4> w(t);

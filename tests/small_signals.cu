@@ -55,6 +55,29 @@ static void transverse(const char* name, double bound) {
     std::printf("%s %.17g %.17g\n", name, worst, bound);
 }
 
+// A smooth signal of size s beside a jump of 1 at one or two of the stencil's end values: the blend is of the stencils
+// that the jump does not reach.
+static void beside_a_jump(const char* name, double bound) {
+    const double x[7] = {0.31, 0.62, 0.90, 1.27, 1.75, 2.31, 2.96};
+    double worst = 0;
+    for (double s : {1e-4, 1e-6, 1e-10, 1e-14, 1e-17})
+        for (int n = 1; n <= 2; ++n)
+            for (int end = 0; end < 2; ++end) {
+                double a[7], b, c, d;
+                LD l[7], bl, cl, dl;
+                for (int k = 0; k < 7; ++k) {
+                    a[k] = (end ? k >= 7 - n : k < n) ? 1.0 + 0.1 * k : s * x[k];
+                    l[k] = a[k];
+                }
+                weno4(a, b, c, d);
+                weno4(l, bl, cl, dl);
+                worst = std::fmax(worst, (double)std::fabs((b - bl) / bl));
+                worst = std::fmax(worst, (double)std::fabs((c - cl) / bl));
+                worst = std::fmax(worst, (double)std::fabs((d - dl) / bl));
+            }
+    std::printf("%s %.17g %.17g\n", name, worst, bound);
+}
+
 int main() {
     // A flux carries four roundings, a mode's sums amplify them by at most 16 (order 3) and 212 (order 4), and the
     // order's further iterations add the same again.
@@ -63,5 +86,7 @@ int main() {
     transverse<3, FORM_MODAL, 8>("modal3_mhd", b3);
     transverse<4, FORM_MODAL, 5>("modal4", b4);
     transverse<4, FORM_MODAL, 8>("modal4_mhd", b4);
+    // 60 b sums up to 196 differences of a unit and more; a blend's weights carry a few roundings and move it by its spread
+    beside_a_jump("weno4", std::ldexp(1.0, -53 + 6));
     return 0;
 }

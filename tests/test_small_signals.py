@@ -16,7 +16,7 @@ def test_small_signals_against_long_double(tmp_path):
     subprocess.run([nvcc, "-O1", "-std=c++17", "--expt-relaxed-constexpr", "-gencode", "arch=compute_103a,code=sm_103a",
                     os.path.join(HERE, "small_signals.cu"), "-o", exe], check=True, capture_output=True, timeout=900)
     lines = subprocess.run([exe], check=True, capture_output=True, text=True, timeout=600).stdout.splitlines()
-    assert len(lines) == 4
+    assert len(lines) == 5
     for text in lines:
         name, value, bound = text.split()
         assert float(value) <= float(bound), text
