@@ -335,28 +335,6 @@ ADER_DEV Vec<NV, R> flux_scaled(const Vec<NV, R>& u, R gm1, R c) {
     }
 }
 
-// cx F + cy G + cz H: the flux along the vector (cx, cy, cz), for Euler in the work of one direction
-template <int NV, class R>
-ADER_DEV Vec<NV, R> flux_along(const Vec<NV, R>& u, R gm1, R cx, R cy, R cz) {
-    if constexpr (NV == 5) {
-        const R irho = rcp(u[0]);
-        const R mc = cx * u[1] + cy * u[2] + cz * u[3];
-        const R vc = mc * irho;
-        const R w = (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * irho;
-        const R p = gm1 * (u[4] - R(0.5) * w);
-        Vec<NV, R> f;
-        f[0] = mc;
-        f[1] = u[1] * vc + cx * p;
-        f[2] = u[2] * vc + cy * p;
-        f[3] = u[3] * vc + cz * p;
-        f[4] = (u[4] + p) * vc;
-        return f;
-    } else {
-        const Prim<NV, R> q = primitives(u, gm1);
-        return scale(cx, flux_from<0>(u, q)) + scale(cy, flux_from<1>(u, q)) + scale(cz, flux_from<2>(u, q));
-    }
-}
-
 // fast magnetosonic speed in direction D (the sound speed for Euler)
 template <int D, int NV, class R>
 ADER_DEV R fast_speed(const Vec<NV, R>& u, const Prim<NV, R>& q, R gamma) {

@@ -62,10 +62,12 @@ struct SerialTeam {
         for (int k = 0; k < A; ++k)
             h[N + k] = SC ? flux_scaled<2>(u[N + 2 * A + k], gm1, kz) : flux<2>(u[N + 2 * A + k], gm1);
     }
-    // sum over d of c_d (F_d(u[0]) - F_d(u[1 + d])), times k
+    // sum over d of c_d (F_d(u[0]) - F_d(u[1 + d])), times k.  Direction by direction, with the same flux on both sides:
+    // equal states give exactly zero (one flux along (cx, cy, cz) for u[0] rounds unlike the three it meets).
     ADER_DEV V axis_differences(const V* u, R k) const {
-        return flux_along(u[0], gm1, k * cx, k * cy, k * cz) - flux_scaled<0>(u[1], gm1, k * cx) -
-               flux_scaled<1>(u[2], gm1, k * cy) - flux_scaled<2>(u[3], gm1, k * cz);
+        return scale(k * cx, flux<0>(u[0], gm1) - flux<0>(u[1], gm1)) +
+               scale(k * cy, flux<1>(u[0], gm1) - flux<1>(u[2], gm1)) +
+               scale(k * cz, flux<2>(u[0], gm1) - flux<2>(u[3], gm1));
     }
     // fluxes of direction D at N nodes; ok[s]: whether the M states ub[s] are physical
     template <int D, int N, int M>
@@ -164,16 +166,16 @@ struct WarpTeam {
 #pragma unroll
         for (int n = 0; n < 4; ++n) sh[(n * NV + v) * 32] = u[n][0];
         __syncthreads();
-        if (v < 4) {
-            const Vec<NV, R> x = load(v * NV);
-            if (v == 0) store(0, flux_along(x, gm1, k * cx, k * cy, k * cz));
-            else if (v == 1) store(NV, flux_scaled<0>(x, gm1, k * cx));
-            else if (v == 2) store(2 * NV, flux_scaled<1>(x, gm1, k * cy));
-            else store(3 * NV, flux_scaled<2>(x, gm1, k * cz));
+        if (v < 3) {                        // warp d takes the direction d: node 0 against node 1 + d
+            const int at = (v + 1) * NV;
+            const Vec<NV, R> x = load(0), y = load(at);
+            if (v == 0) store(at, scale(k * cx, flux<0>(x, gm1) - flux<0>(y, gm1)));
+            else if (v == 1) store(at, scale(k * cy, flux<1>(x, gm1) - flux<1>(y, gm1)));
+            else store(at, scale(k * cz, flux<2>(x, gm1) - flux<2>(y, gm1)));
         }
         __syncthreads();
         V r;
-        r[0] = sh[v * 32] - sh[(NV + v) * 32] - sh[(2 * NV + v) * 32] - sh[(3 * NV + v) * 32];
+        r[0] = sh[(NV + v) * 32] + sh[(2 * NV + v) * 32] + sh[(3 * NV + v) * 32];
         return r;
     }
     template <int D, int N, int M>

@@ -55,6 +55,20 @@ static void transverse(const char* name, double bound) {
     std::printf("%s %.17g %.17g\n", name, worst, bound);
 }
 
+// The largest time mode of a uniform oblique flow: exactly zero.
+template <int ORDER, int FORM, int NV, class R>
+static void uniform(const char* name) {
+    constexpr int L = ModeCount<ORDER>::L;
+    const double c[3] = {0.21, 0.17, 0.13}, state[8] = {1.1, 0.37, -0.53, 0.71, 2.6, 0.9, -0.4, 0.7};
+    double w[36][8] = {}, worst = 0;
+    for (int v = 0; v < NV; ++v) w[1][v] = state[v];
+    Vec<NV, R> m[L + 1];
+    predict<ORDER, FORM, NV, R>(w, c, m);
+    for (int k = ModeCount<ORDER>::LS + 1; k <= L; ++k)
+        for (int v = 0; v < NV; ++v) worst = std::fmax(worst, (double)std::fabs(m[k][v]));
+    std::printf("%s %.17g 0\n", name, worst);
+}
+
 // A smooth signal of size s beside a jump of 1 at one or two of the stencil's end values: the blend is of the stencils
 // that the jump does not reach.
 static void beside_a_jump(const char* name, double bound) {
@@ -82,10 +96,20 @@ int main() {
     // A flux carries four roundings, a mode's sums amplify them by at most 16 (order 3) and 212 (order 4), and the
     // order's further iterations add the same again.
     const double b3 = std::ldexp(1.0, -53 + 2 + 4 + 1), b4 = std::ldexp(1.0, -53 + 2 + 8 + 2);
+    transverse<2, FORM_MODAL, 5>("modal2", b3);
+    transverse<2, FORM_NODAL, 5>("nodal2", b3);
+    // (the nodal form takes its time modes from differences of node values: their last places too)
+    transverse<3, FORM_NODAL, 5>("nodal3", b3 + std::ldexp(1.0, -53 + 4) / (3e-5 * 0.37 / 1.1));
     transverse<3, FORM_MODAL, 5>("modal3", b3);
     transverse<3, FORM_MODAL, 8>("modal3_mhd", b3);
     transverse<4, FORM_MODAL, 5>("modal4", b4);
     transverse<4, FORM_MODAL, 8>("modal4_mhd", b4);
+    uniform<2, FORM_NODAL, 5, double>("uniform2");
+    uniform<2, FORM_NODAL, 8, double>("uniform2_mhd");
+    uniform<2, FORM_NODAL, 5, float>("uniform2_f32");
+    uniform<3, FORM_NODAL, 5, double>("uniform3");
+    uniform<3, FORM_NODAL, 8, double>("uniform3_mhd");
+    uniform<3, FORM_NODAL, 5, float>("uniform3_f32");
     // 60 b sums up to 196 differences of a unit and more; a blend's weights carry a few roundings and move it by its spread
     beside_a_jump("weno4", std::ldexp(1.0, -53 + 6));
     return 0;
