@@ -344,6 +344,9 @@ void ader_destroy(ader_ctx* ctx);
  *   ader_batch_tune: optional; times each (group, phase) over block sizes
  *     64/128/256 and persistent grid sizes on private copies of the given
  *     states (allocated and freed inside the call) and keeps the fastest.
+ *     Predictors that run by teams of warps (Euler at modal order 4, MHD at
+ *     orders 3-4) have one launch shape, 32 zones a block: they are not
+ *     timed or listed.
  *   ader_batch_step: U[p] (device, 5 x zones, in/out), Bface[p] (device,
  *     3 x zones for MHD problems, else ignored), dt_dev[p] (device, n doubles).
  *   ader_batch_advance: dt_dev[p] = cfl / max over zones of sum_d (|v_d| +
@@ -353,7 +356,8 @@ void ader_destroy(ader_ctx* ctx);
  *   ader_batch_status: synchronises the stream; codes_host[p] (n ints, may be
  *     NULL) gets each problem's code; returns the first non-OK code.
  *   ader_batch_tuning: writes (group, phase, threads, blocks) quadruples
- *     (blocks 0 = one block per `threads` zones) to out_host (cap ints);
+ *     (blocks 0 = one block per `threads` zones) of the phases with a choice to
+ *     out_host (cap ints);
  *     returns the number of quadruples.
  * The pointer arrays are host arrays; the pointers they hold are device
  * pointers and stay owned by the caller. */

@@ -363,7 +363,8 @@ def ader_batch_status(b, n, stream=None):
 
 
 def ader_batch_tuning(b):
-    """[(group, phase, threads, blocks)] chosen by ader_batch_tune (blocks 0: one block per `threads` zones)."""
+    """[(group, phase, threads, blocks)] chosen by ader_batch_tune (blocks 0: one block per `threads` zones); phases
+    of one launch shape are left out."""
     cap = 4 * 512
     out = (ctypes.c_int * cap)()
     k = load().ader_batch_tuning(b, out, cap)

@@ -179,6 +179,9 @@ int run_phase(const Group& gr, int ph, int T, int B, cudaStream_t st, bool go, c
     }
 }
 
+// whether a phase's kernel has one launch shape, whatever block size it is asked for (teams of warps)
+bool one_shape(const Group& g, int ph) { return run_phase(g, ph, 128, 0, nullptr, false, nullptr) == 2; }
+
 // Uploads the items (state pointers set) and padded offsets of every group and of the whole batch.
 int upload(ader_batch* b, double* const* U, double* const* Bf, const double* dt_dev) {
     for (int p = 0; p < b->n; ++p) {
@@ -462,7 +465,7 @@ int ader_batch_tune(ader_batch* b, double* const* U, double* const* Bface, void*
     const int Ts[3] = {64, 128, 256};
     for (auto& g : b->groups) {
         for (int ph = 0; ph < PH_COUNT && rc == ADER_OK; ++ph) {
-            if (!batch_phase_applies(ph, g.order, g.mhd)) continue;
+            if (!batch_phase_applies(ph, g.order, g.mhd) || one_shape(g, ph)) continue;
             Tuned best;
             for (int T : Ts) {
                 if (T > batch_phase_max_threads(ph)) continue;
@@ -526,7 +529,7 @@ int ader_batch_tuning(const ader_batch* b, int* out_host, int cap) {
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         const Group& g = b->groups[gi];
         for (int ph = 0; ph < PH_COUNT; ++ph) {
-            if (!batch_phase_applies(ph, g.order, g.mhd)) continue;
+            if (!batch_phase_applies(ph, g.order, g.mhd) || one_shape(g, ph)) continue;
             if (k + 4 <= cap) {
                 out_host[k] = (int)gi;
                 out_host[k + 1] = ph;

@@ -240,8 +240,8 @@ inline bool batch_phase_applies(int ph, int order, int mhd) {
 }
 
 // Launches phase ph of a group of (ORDER, NV) problems with `threads` zones per
-// block and `blocks` blocks; returns the kernel (for occupancy queries) through
-// *fn when launch is false.  Instantiated per (ORDER, NV) in batch_o*_*.cu (FP32 bulk).
+// block and `blocks` blocks (a team of warps: its own shape); returns the kernel (for occupancy queries) through
+// *fn, and when launch is false 2 for a kernel of one launch shape, 1 for one with a choice.  Instantiated per (ORDER, NV) in batch_o*_*.cu (FP32 bulk).
 template <int ORDER, int NV>
 int batch_phase(int ph, const BatchGroupDev& g, int form, int solver, int threads, int blocks, cudaStream_t st,
                 bool launch, const void** fn);

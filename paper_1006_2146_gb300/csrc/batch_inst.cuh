@@ -65,7 +65,8 @@ int batch_phase(int ph, const BatchGroupDev& g, int form, int solver, int thread
         default: break;
     }
     if (fn) *fn = k;
-    if (!k || !launch) return k ? 1 : 0;
+    if (!k) return 0;
+    if (!launch) return team ? 2 : 1;
     void* args[] = {(void*)&g};
     return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3((unsigned)threads), args, smem, st) == cudaSuccess ? 1 : -1;
 }
