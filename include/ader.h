@@ -187,11 +187,15 @@ int ader_set_predictor(ader_ctx* ctx, double tol, int max_iter);
  * on = 1 also computes the moments of the reconstruction in shared-memory
  * tiles of 32 x 8 columns, each WENO term of a position once for all the
  * zones that use it: FP64 1-D and cross moments of orders 2-3 (Euler and MHD)
- * on every grid that fills at least half of its tiles' columns, FP32 cross
- * moments of order 3 where nx is a multiple of 32 and ny of 8; on = 0 takes
- * the per-zone kernels, with the same bits in FP64 (FP32 to FP32 rounding).
+ * on every grid that fills at least half of its tiles' columns and has two
+ * planes of tiles for every SM (tiles x nz >= 2 SMs), FP32 cross moments of
+ * order 3 where nx is a multiple of 32 and ny of 8; on = 0 takes the per-zone
+ * kernels, with the same bits in FP64 (FP32 to FP32 rounding).
  * ADER_ERR_ARG for a NULL context. */
 int ader_set_tiled(ader_ctx* ctx, int on);
+/* Planes a block of the FP64 reconstruction tiles marches through on this
+ * context's grid (1 to 8), 0 where the per-zone kernels run. */
+int ader_weno_tile_planes(const ader_ctx* ctx);
 
 /* Box faces (Euler contexts).  bc[6] = {x-, x+, y-, y+, z-, z+}, each
  * ADER_BC_PERIODIC (the default), ADER_BC_OUTFLOW or ADER_BC_REFLECTIVE; an

@@ -539,6 +539,10 @@ int ader_set_tiled(ader_ctx* c, int on) {
     return ADER_OK;
 }
 
+int ader_weno_tile_planes(const ader_ctx* c) {
+    return c ? recon_tile_planes(make_args(c->inner ? c->inner : c, 0.0, nullptr, 0)) : 0;
+}
+
 int ader_set_boundary(ader_ctx* c, const int* bc) {
     if (!c) return ADER_ERR_ARG;
     if (!bc) return fail(c, ADER_ERR_ARG, "bc is null");

@@ -90,6 +90,8 @@ inline int s3_per_zone(int mhd, int linearized = 0) {
 }
 
 template <class R> int launch_recon(const StepArgs& a, const double* U, cudaStream_t st);
+// FP64: planes a block of the WENO tiles marches through, 0 where the per-zone kernels run
+int recon_tile_planes(const StepArgs& a);
 // out[i] = (float)U[i], i < count (the FP32 copy of the state the FP32 WENO reads)
 int launch_to_f32(float* out, const double* U, long long count, cudaStream_t st);
 // FP64: first-order fluxes on the faces of zones left non-physical, conservative re-update; MHD (Bold: the face

@@ -509,6 +509,12 @@ static bool tiles64(const Grid& g, dim3& grid, int& cz) {
     return grid.y <= 65535u;
 }
 
+int recon_tile_planes(const StepArgs& a) {
+    dim3 grid;
+    int cz;
+    return a.tiled && !a.fp32 && a.order <= 3 && tiles64(a.grid, grid, cz) ? cz : 0;
+}
+
 template <int ORDER, int NV>
 static bool launch_weno1d_tiled64(const Grid& g, const double* U, const double* ZB, double* S1, cudaStream_t st) {
     dim3 grid;
