@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(256) kb_flux_update(BatchGroupDev g) {
             split_scales(it.a, 1.0, 1, chi, clo);
             zone_flux_update_stored_pair(it.a, U, U, chi, clo, z);
         } else {
-            zone_flux_update_pair<SOLVER, NV>(it.a, U, U, 1.0, 1, z);
+            zone_flux_update_pair<SOLVER>(it.a, U, U, 1.0, 1, z);
         }
     }
 }

@@ -53,7 +53,8 @@ ADER_DEV long long fix_mulhi(long long a, long long b) {
 }
 
 // c a for a literal c (folded at compile time): the nearest integer by a multiplication, a fractional power of
-// two by a shift, any other fraction by the upper half of a product with its 64-bit expansion
+// two by a shift, any other fraction by the upper half of a product with it (c's FP64 value less the integer, at
+// most 53 bits)
 ADER_DEV Fix fix_times(double c, Fix a) {          // c >= 0
     const long long i = (long long)(c + 0.49999999);
     const double f = c - (double)i;                 // in (-1/2, 1/2]
@@ -258,30 +259,15 @@ template <int D, class R>
 struct FluxSum {
     R p[3] = {R(0), R(0), R(0)}, w = R(0), ev = R(0), wv = R(0);
 
-    template <int SIGN = 1>
     ADER_DEV void add(const Vec<5, R>& u) {
         const R r = rcp(u[0]);
-        const R v = SIGN > 0 ? u[1 + D] * r : -(u[1 + D] * r);
+        const R v = u[1 + D] * r;
         const R k = (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * r;
 #pragma unroll
         for (int c = 0; c < 3; ++c) p[c] += u[1 + c] * v;
-        w = SIGN > 0 ? w + k : w - k;
+        w += k;
         ev += u[4] * v;
         wv += k * v;
-    }
-    ADER_DEV void scale(R c) {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) p[i] = c * p[i];
-        w = c * w;
-        ev = c * ev;
-        wv = c * wv;
-    }
-    ADER_DEV void merge(R c, const FluxSum& o) {      // this + c o
-#pragma unroll
-        for (int i = 0; i < 3; ++i) p[i] += c * o.p[i];
-        w += c * o.w;
-        ev += c * o.ev;
-        wv += c * o.wv;
     }
     // c times the sum; avg the face average of the state
     ADER_DEV Vec<5, R> mean(const Vec<5, R>& avg, R gm1, R c) const {

@@ -276,9 +276,9 @@ int launch_flux_update(const StepArgs& a, double* out, const double* base, doubl
     }
     if constexpr (sizeof(R) == 4) {           // fused, both faces of each direction per zone, FP32 pairs
         if (a.solver == SOLVER_HLL)
-            k_flux_update_pair<SOLVER_HLL, 5><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
+            k_flux_update_pair<SOLVER_HLL><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
         else
-            k_flux_update_pair<SOLVER_LINEARIZED, 5><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
+            k_flux_update_pair<SOLVER_LINEARIZED><<<blocks, T, 0, st>>>(a, out, base, c_host, dd);
         return 1;
     } else {                                   // each face solved once, then the update
         if (a.solver == SOLVER_HLL)

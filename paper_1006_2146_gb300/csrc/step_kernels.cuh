@@ -353,7 +353,7 @@ constexpr bool uses_team() {
 // what spills costs (about 12% per 256^3 step at orders 2-3); order 4 spills kilobytes per zone there and takes two
 // blocks and 255 registers.
 template <int ORDER, int FORM, int NV, class R, bool SRC = false>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? (ORDER == 4 ? 2 : 3) : 1) k_predict_faces(StepArgs a, const double* __restrict__ U) {
+__global__ void __launch_bounds__(128, ORDER == 4 ? 2 : 3) k_predict_faces(StepArgs a, const double* __restrict__ U) {
     const long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (z < a.grid.n) zone_predict_faces<ORDER, FORM, NV, R, SRC>(a, U, z);
 }
@@ -407,13 +407,16 @@ ADER_DEV FaceSide<NV, R> load_side(const StepArgs& a, int side, long long z) {
 //  * fused (zone_flux_update): each zone solves the two faces of each
 //    direction itself -- every face twice over the grid, in one pass.  The
 //    same function with the same operands gives both zones of a face the same
-//    value, so Eq. 6 telescopes exactly.  Used by the FP32-bulk kernels, whose
-//    cost there is the FP64 accumulation, not the Riemann solves.
+//    value, so Eq. 6 telescopes exactly.  Used by FP32 Euler zones whose face
+//    data lie in memory (order 4, tiles off, the batch), where the FP64
+//    accumulation is the cost, not the Riemann solves.
 //  * stored (zone_face_fluxes, then zone_flux_update_stored): every face is
 //    solved once, by the zone below it, into the WENO scratch S1 (dead once
 //    the face data exist; at least 15 values per zone at every order), and
 //    the update takes differences of stored values.  Used by FP64, where the
-//    solves are FP64 work on the critical path.
+//    solves are FP64 work on the critical path, and by MHD in both precisions,
+//    whose faces also give four edge fluxes; the FP32 Euler tiles store their
+//    fluxes in the same place.
 template <int SOLVER, int D, int NV, class R>
 ADER_DEV Vec<NV, R> upper_face_flux(const StepArgs& a, long long z, int i, int j, int k, R gamma, R gm1) {
     const long long zp = nbr_along(a.grid, z, i, j, k, D, 1);
@@ -519,13 +522,13 @@ __device__ __forceinline__ void store_pair_update(const StepArgs& a, double* out
     if (bad && !a.defer_nonfinite) raise_flag(a.flag, FLAG_NONFINITE);
 }
 
-template <int SOLVER, int D, int NV>
+template <int SOLVER, int D>
 ADER_DEV void flux_difference_pair(const StepArgs& a, long long z, int i, int j, int k, float gamma, float gm1,
                                    float chi, float clo, float* hi, float* lo) {
     const long long zm = nbr_along(a.grid, z, i, j, k, D, -1);
-    const Vec<NV, float> Fp = upper_face_flux<SOLVER, D, NV, float>(a, z, i, j, k, gamma, gm1);
-    const Vec<NV, float> Fm = riemann<SOLVER, D>(load_side<NV, float>(a, 2 * D, zm),
-                                                 load_side<NV, float>(a, 2 * D + 1, z), gamma, gm1);
+    const Vec<5, float> Fp = upper_face_flux<SOLVER, D, 5, float>(a, z, i, j, k, gamma, gm1);
+    const Vec<5, float> Fm = riemann<SOLVER, D>(load_side<5, float>(a, 2 * D, zm),
+                                                load_side<5, float>(a, 2 * D + 1, z), gamma, gm1);
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
         float s, e;
@@ -540,7 +543,7 @@ ADER_DEV void flux_difference_pair(const StepArgs& a, long long z, int i, int j,
     }
 }
 
-template <int SOLVER, int NV>
+template <int SOLVER>
 __global__ void __launch_bounds__(128) k_flux_update_pair(StepArgs a, double* out, const double* base, double c_host,
                                                           int use_dt_dev) {
     __shared__ float c_hi[3], c_lo[3];
@@ -558,9 +561,9 @@ __global__ void __launch_bounds__(128) k_flux_update_pair(StepArgs a, double* ou
     zone_ijk(a.grid, z, i, j, k);
     const float gamma = a.gamma_f, gm1 = a.gm1_f;
     float hi[5] = {0, 0, 0, 0, 0}, lo[5] = {0, 0, 0, 0, 0};
-    flux_difference_pair<SOLVER, 0, NV>(a, z, i, j, k, gamma, gm1, c_hi[0], c_lo[0], hi, lo);
-    flux_difference_pair<SOLVER, 1, NV>(a, z, i, j, k, gamma, gm1, c_hi[1], c_lo[1], hi, lo);
-    flux_difference_pair<SOLVER, 2, NV>(a, z, i, j, k, gamma, gm1, c_hi[2], c_lo[2], hi, lo);
+    flux_difference_pair<SOLVER, 0>(a, z, i, j, k, gamma, gm1, c_hi[0], c_lo[0], hi, lo);
+    flux_difference_pair<SOLVER, 1>(a, z, i, j, k, gamma, gm1, c_hi[1], c_lo[1], hi, lo);
+    flux_difference_pair<SOLVER, 2>(a, z, i, j, k, gamma, gm1, c_hi[2], c_lo[2], hi, lo);
     store_pair_update(a, out, base, hi, lo, z);
 }
 
@@ -577,7 +580,7 @@ __device__ __forceinline__ void split_scales(const StepArgs& a, double c_host, i
     }
 }
 
-template <int SOLVER, int NV>
+template <int SOLVER>
 __device__ __forceinline__ void zone_flux_update_pair(const StepArgs& a, double* out, const double* base,
                                                       double c_host, int use_dt_dev, long long z) {
     int i, j, k;
@@ -586,9 +589,9 @@ __device__ __forceinline__ void zone_flux_update_pair(const StepArgs& a, double*
     split_scales(a, c_host, use_dt_dev, chi, clo);
     const float gamma = a.gamma_f, gm1 = a.gm1_f;
     float hi[5] = {0, 0, 0, 0, 0}, lo[5] = {0, 0, 0, 0, 0};
-    flux_difference_pair<SOLVER, 0, NV>(a, z, i, j, k, gamma, gm1, chi[0], clo[0], hi, lo);
-    flux_difference_pair<SOLVER, 1, NV>(a, z, i, j, k, gamma, gm1, chi[1], clo[1], hi, lo);
-    flux_difference_pair<SOLVER, 2, NV>(a, z, i, j, k, gamma, gm1, chi[2], clo[2], hi, lo);
+    flux_difference_pair<SOLVER, 0>(a, z, i, j, k, gamma, gm1, chi[0], clo[0], hi, lo);
+    flux_difference_pair<SOLVER, 1>(a, z, i, j, k, gamma, gm1, chi[1], clo[1], hi, lo);
+    flux_difference_pair<SOLVER, 2>(a, z, i, j, k, gamma, gm1, chi[2], clo[2], hi, lo);
     store_pair_update(a, out, base, hi, lo, z);
 }
 
@@ -749,7 +752,7 @@ __global__ void __launch_bounds__(128) k_flux_update_stored(StepArgs a, double* 
     if (z < a.grid.n) zone_flux_update_stored<R>(a, out, base, c_host, use_dt_dev, z);
 }
 
-// ------------------------------------------------------------------ Euler: predictor and face solves per tile
+// ------------------------------------------------------------------ FP32 Euler: predictor and face solves per tile
 // A block owns a PT_X x PT_Y tile of (x, y) columns and marches through a chunk of z planes, one zone per
 // thread and plane.  Each zone's predictor writes its six face sides (barycentre state, <u>, <F>; 15
 // values each) to shared memory; after a barrier every face inside the tile is solved once, by the zone
@@ -769,13 +772,11 @@ constexpr int PT_X = ADER_PT_X, PT_Y = ADER_PT_Y, PT_THREADS = PT_X * PT_Y;
 constexpr int PT_NQ = 15;                     // values per Euler face side
 constexpr int PT_SLOTS = 7;                   // x+, x-, y+, y-, z+ (even planes), z-, z+ (odd planes)
 
-template <class R>
-ADER_DEV R* pt_slot(R* sh, int slot, int tid) { return sh + slot * PT_NQ * PT_THREADS + tid; }
+ADER_DEV float* pt_slot(float* sh, int slot, int tid) { return sh + slot * PT_NQ * PT_THREADS + tid; }
 
 // one side into a slot: u_b (replaced by the zone mean for the wave speeds when not physical, as
 // write_side does), <u>, <F>
-template <class R>
-ADER_DEV void pt_side(R* dst, const Vec<5, R>& mean, Vec<5, R> ub, const Vec<5, R>& avg, const Vec<5, R>& Fa, R gm1) {
+ADER_DEV void pt_side(float* dst, const Vec<5, float>& mean, Vec<5, float> ub, const Vec<5, float>& avg, const Vec<5, float>& Fa, float gm1) {
     if (!physical_state(ub, gm1)) ub = mean;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
@@ -785,18 +786,17 @@ ADER_DEV void pt_side(R* dst, const Vec<5, R>& mean, Vec<5, R> ub, const Vec<5, 
     }
 }
 
-template <int ORDER, int D, class R>
-ADER_DEV void pt_sides(R* sh, int tid, int slot_plus, int slot_minus, const Vec<5, R>* m, R gm1) {
-    Vec<5, R> ub[2], avg[2], Fa[2];
-    both_faces<ORDER, D, R>(m, gm1, ub, avg, Fa);
+template <int ORDER, int D>
+ADER_DEV void pt_sides(float* sh, int tid, int slot_plus, int slot_minus, const Vec<5, float>* m, float gm1) {
+    Vec<5, float> ub[2], avg[2], Fa[2];
+    both_faces<ORDER, D, float>(m, gm1, ub, avg, Fa);
     pt_side(pt_slot(sh, slot_plus, tid), m[1], ub[0], avg[0], Fa[0], gm1);
     pt_side(pt_slot(sh, slot_minus, tid), m[1], ub[1], avg[1], Fa[1], gm1);
 }
 
-template <class R>
-ADER_DEV FaceSide<5, R> pt_load(const R* sh, int slot, int tid) {
-    const R* s = sh + slot * PT_NQ * PT_THREADS + tid;
-    FaceSide<5, R> f;
+ADER_DEV FaceSide<5, float> pt_load(const float* sh, int slot, int tid) {
+    const float* s = sh + slot * PT_NQ * PT_THREADS + tid;
+    FaceSide<5, float> f;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
         f.ub[v] = s[v * PT_THREADS];
@@ -832,16 +832,14 @@ ADER_DEV PtBoundary pt_boundary(const Grid& g, int cz) {
 }
 
 // one side from shared memory into a packed boundary array: slice stride `slice`, position `pos`
-template <class R>
-ADER_DEV void pt_to_boundary(R* base, long long slice, long long pos, const R* sh, int slot, int tid) {
-    const R* s = sh + slot * PT_NQ * PT_THREADS + tid;
+ADER_DEV void pt_to_boundary(float* base, long long slice, long long pos, const float* sh, int slot, int tid) {
+    const float* s = sh + slot * PT_NQ * PT_THREADS + tid;
 #pragma unroll
     for (int q = 0; q < PT_NQ; ++q) base[q * slice + pos] = s[q * PT_THREADS];
 }
 
-template <class R>
-ADER_DEV FaceSide<5, R> pt_from_boundary(const R* base, long long slice, long long pos) {
-    FaceSide<5, R> f;
+ADER_DEV FaceSide<5, float> pt_from_boundary(const float* base, long long slice, long long pos) {
+    FaceSide<5, float> f;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
         f.ub[v] = base[v * slice + pos];
@@ -851,20 +849,20 @@ ADER_DEV FaceSide<5, R> pt_from_boundary(const R* base, long long slice, long lo
     return f;
 }
 
-template <int D, class R>
-ADER_DEV void pt_store_flux(const StepArgs& a, long long zl, const Vec<5, R>& f) {
-    R* F = (R*)a.S1;
+template <int D>
+ADER_DEV void pt_store_flux(const StepArgs& a, long long zl, const Vec<5, float>& f) {
+    float* F = (float*)a.S1;
 #pragma unroll
     for (int v = 0; v < 5; ++v) F[(D * 5 + v) * a.grid.n + zl] = f[v];
 }
 
-// grid: (tiles_x * tiles_y, ceil(nz / cz)); dynamic shared memory PT_SLOTS * PT_NQ * PT_THREADS values of R
-template <int ORDER, int FORM, int SOLVER, class R, bool SRC>
+// grid: (tiles_x * tiles_y, ceil(nz / cz)); dynamic shared memory PT_SLOTS * PT_NQ * PT_THREADS floats
+template <int ORDER, int FORM, int SOLVER, bool SRC>
 __global__ void __launch_bounds__(PT_THREADS, 3)
     k_pf_tile(StepArgs a, const double* __restrict__ U, int cz) {
 
     extern __shared__ __align__(16) unsigned char pt_raw[];
-    R* sh = reinterpret_cast<R*>(pt_raw);
+    float* sh = reinterpret_cast<float*>(pt_raw);
     const Grid& g = a.grid;
     const int tid = threadIdx.x, tx = tid % PT_X, ty = tid / PT_X;
     const int tiles_x = (g.nx + PT_X - 1) / PT_X;
@@ -872,21 +870,21 @@ __global__ void __launch_bounds__(PT_THREADS, 3)
     const int k0 = (int)blockIdx.y * cz, k1 = min(k0 + cz, g.nz);
     const bool valid = i < g.nx && j < g.ny;
     const bool last_x = tx == PT_X - 1 || i == g.nx - 1, last_y = ty == PT_Y - 1 || j == g.ny - 1;
-    const R gamma = arg_gamma<R>(a), gm1 = arg_gm1<R>(a);
+    const float gamma = arg_gamma<float>(a), gm1 = arg_gm1<float>(a);
     const long long nxy = (long long)g.nx * g.ny;
-    const R dt = bulk_arg<R>(a.dt_dev ? *a.dt_dev : a.dt);     // once per thread, for every plane
+    const float dt = bulk_arg<float>(a.dt_dev ? *a.dt_dev : a.dt);     // once per thread, for every plane
     const PtBoundary bd = pt_boundary(g, cz);
-    R* S3 = (R*)a.S3;
-    R* bx = S3 + bd.ox;
-    R* by = S3 + bd.oy;
-    R* bz = S3 + bd.oz;
+    float* S3 = (float*)a.S3;
+    float* bx = S3 + bd.ox;
+    float* by = S3 + bd.oy;
+    float* bz = S3 + bd.oz;
     const long long tile_x = blockIdx.x % tiles_x, tile_y = blockIdx.x / tiles_x, chunk = blockIdx.y;
     for (int k = k0; k < k1; ++k) {
         const long long z = (long long)k * nxy + (long long)j * g.nx + i;
         const int zp_slot = (k & 1) ? 6 : 4;          // this plane's z+ sides; the previous plane's in the other
         if (valid) {
-            Vec<5, R> m[ModeCount<ORDER>::L + 1];
-            SerialTeam<5, R> team;
+            Vec<5, float> m[ModeCount<ORDER>::L + 1];
+            SerialTeam<5, float> team;
             team_scales(team, a, dt);
             zone_predict<ORDER, FORM, SRC>(team, a, U, z, true, m, dt);
             pt_sides<ORDER, 0>(sh, tid, 0, 1, m, gm1);
@@ -922,14 +920,14 @@ __global__ void __launch_bounds__(PT_THREADS, 3)
 // The faces on tile and chunk boundaries, from the sides k_pf_tile packed in S3: the tile boundaries in
 // x (i = multiples of PT_X, and i = 0 against nx - 1), in y (multiples of PT_Y) and the chunk boundaries
 // in z (multiples of cz).  One thread per face, the packed arrays' fastest index fastest across threads.
-template <int SOLVER, class R>
+template <int SOLVER>
 __global__ void __launch_bounds__(128) k_tile_faces(StepArgs a, int cz, long long nfx, long long nfy, long long nfz) {
     const Grid& g = a.grid;
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const R gamma = arg_gamma<R>(a), gm1 = arg_gm1<R>(a);
+    const float gamma = arg_gamma<float>(a), gm1 = arg_gm1<float>(a);
     const long long nxy = (long long)g.nx * g.ny;
     const PtBoundary bd = pt_boundary(g, cz);
-    const R* S3 = (const R*)a.S3;
+    const float* S3 = (const float*)a.S3;
     if (t < nfx) {                      // x: t = (tile * nz + k) * ny + j; lower zone in the previous tile
         const int j = (int)(t % g.ny);
         const long long r = t / g.ny;
@@ -938,7 +936,7 @@ __global__ void __launch_bounds__(128) k_tile_faces(StepArgs a, int cz, long lon
         const int tl = tile == 0 ? ntx - 1 : tile - 1;
         const int il = tile == 0 ? g.nx - 1 : tile * PT_X - 1;
         const long long pl = ((long long)tl * g.nz + k) * g.ny + j;
-        const R* bx = S3 + bd.ox;
+        const float* bx = S3 + bd.ox;
         pt_store_flux<0>(a, (long long)k * nxy + (long long)j * g.nx + il,
                          riemann<SOLVER, 0>(pt_from_boundary(bx, bd.sx, pl),
                                             pt_from_boundary(bx + PT_NQ * bd.sx, bd.sx, t), gamma, gm1));
@@ -953,7 +951,7 @@ __global__ void __launch_bounds__(128) k_tile_faces(StepArgs a, int cz, long lon
         const int tl = tile == 0 ? nty - 1 : tile - 1;
         const int jl = tile == 0 ? g.ny - 1 : tile * PT_Y - 1;
         const long long pl = ((long long)tl * g.nz + k) * g.nx + i;
-        const R* by = S3 + bd.oy;
+        const float* by = S3 + bd.oy;
         pt_store_flux<1>(a, (long long)k * nxy + (long long)jl * g.nx + i,
                          riemann<SOLVER, 1>(pt_from_boundary(by, bd.sy, pl),
                                             pt_from_boundary(by + PT_NQ * bd.sy, bd.sy, t), gamma, gm1));
@@ -966,7 +964,7 @@ __global__ void __launch_bounds__(128) k_tile_faces(StepArgs a, int cz, long lon
         const int ncz = (g.nz + cz - 1) / cz;
         const int cl = chunk == 0 ? ncz - 1 : chunk - 1;
         const int kl = chunk == 0 ? g.nz - 1 : chunk * cz - 1;
-        const R* bz = S3 + bd.oz;
+        const float* bz = S3 + bd.oz;
         pt_store_flux<2>(a, (long long)kl * nxy + col,
                          riemann<SOLVER, 2>(pt_from_boundary(bz, bd.sz, (long long)cl * nxy + col),
                                             pt_from_boundary(bz + PT_NQ * bd.sz, bd.sz, t), gamma, gm1));
@@ -985,27 +983,27 @@ inline int pt_chunk(const Grid& g) {
     return (int)cz;
 }
 
-template <int ORDER, int FORM, class R, bool SRC>
+template <int ORDER, int FORM, bool SRC>
 void launch_pf_tile(const StepArgs& a, const double* U, cudaStream_t st) {
     const Grid& g = a.grid;
     const int cz = pt_chunk(g);
     const int ntx = (g.nx + PT_X - 1) / PT_X, nty = (g.ny + PT_Y - 1) / PT_Y, ncz = (g.nz + cz - 1) / cz;
-    const size_t smem = (size_t)PT_SLOTS * PT_NQ * PT_THREADS * sizeof(R);
+    const size_t smem = (size_t)PT_SLOTS * PT_NQ * PT_THREADS * sizeof(float);
     const dim3 grid((unsigned)(ntx * nty), (unsigned)ncz);
     const long long nfx = (long long)ntx * g.ny * g.nz, nfy = (long long)nty * g.nx * g.nz,
                     nfz = (long long)ncz * g.nx * g.ny;
     const long long nf = nfx + nfy + nfz;
     const unsigned fblocks = (unsigned)((nf + 127) / 128);
     if (a.solver == SOLVER_HLL) {
-        auto kern = k_pf_tile<ORDER, FORM, SOLVER_HLL, R, SRC>;
+        auto kern = k_pf_tile<ORDER, FORM, SOLVER_HLL, SRC>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         kern<<<grid, PT_THREADS, smem, st>>>(a, U, cz);
-        k_tile_faces<SOLVER_HLL, R><<<fblocks, 128, 0, st>>>(a, cz, nfx, nfy, nfz);
+        k_tile_faces<SOLVER_HLL><<<fblocks, 128, 0, st>>>(a, cz, nfx, nfy, nfz);
     } else {
-        auto kern = k_pf_tile<ORDER, FORM, SOLVER_LINEARIZED, R, SRC>;
+        auto kern = k_pf_tile<ORDER, FORM, SOLVER_LINEARIZED, SRC>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         kern<<<grid, PT_THREADS, smem, st>>>(a, U, cz);
-        k_tile_faces<SOLVER_LINEARIZED, R><<<fblocks, 128, 0, st>>>(a, cz, nfx, nfy, nfz);
+        k_tile_faces<SOLVER_LINEARIZED><<<fblocks, 128, 0, st>>>(a, cz, nfx, nfy, nfz);
     }
 }
 
@@ -1099,7 +1097,7 @@ template <int ORDER, int FORM, int NV, class R, bool SRC>
 void launch_pf_variant(const StepArgs& a, const double* U, cudaStream_t st) {
     if constexpr (uses_tiles<ORDER, NV, R>()) {
         if (a.tiled) {
-            launch_pf_tile<ORDER, FORM, R, SRC>(a, U, st);
+            launch_pf_tile<ORDER, FORM, SRC>(a, U, st);
             return;
         }
     }
