@@ -22,6 +22,31 @@ ADER_DEV bool physical_state(const Vec<NV, R>& u, R gm1) {
     return u[0] > R(0) && q.p > R(0);
 }
 
+// a - b, both rounded before: a subtraction that is contracted with the product behind b would leave that product's
+// rounding error where a equals b
+template <class R> ADER_DEV R apart(R a, R b) { return a - b; }
+template <> ADER_DEV float apart<float>(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fsub_rn(a, b);
+#else
+    return a - b;
+#endif
+}
+template <> ADER_DEV double apart<double>(double a, double b) {
+#ifdef __CUDA_ARCH__
+    return __dsub_rn(a, b);
+#else
+    return a - b;
+#endif
+}
+template <int NV, class R>
+ADER_DEV Vec<NV, R> apart(const Vec<NV, R>& a, const Vec<NV, R>& b) {
+    Vec<NV, R> r;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) r[i] = apart(a[i], b[i]);
+    return r;
+}
+
 template <int NV_, class R_>
 struct SerialTeam {
     static constexpr int NV = NV_, NL = NV_;
@@ -62,12 +87,13 @@ struct SerialTeam {
         for (int k = 0; k < A; ++k)
             h[N + k] = SC ? flux_scaled<2>(u[N + 2 * A + k], gm1, kz) : flux<2>(u[N + 2 * A + k], gm1);
     }
-    // sum over d of c_d (F_d(u[0]) - F_d(u[1 + d])), times k.  Direction by direction, with the same flux on both sides:
-    // equal states give exactly zero (one flux along (cx, cy, cz) for u[0] rounds unlike the three it meets).
+    // sum over d of c_d (F_d(u[0]) - F_d(u[1 + d])), times k.  Direction by direction, with the same flux on both sides
+    // and a subtraction of rounded values (apart): equal states give exactly zero.  (One flux along (cx, cy, cz) for u[0]
+    // rounds unlike the three it meets.)
     ADER_DEV V axis_differences(const V* u, R k) const {
-        return scale(k * cx, flux<0>(u[0], gm1) - flux<0>(u[1], gm1)) +
-               scale(k * cy, flux<1>(u[0], gm1) - flux<1>(u[2], gm1)) +
-               scale(k * cz, flux<2>(u[0], gm1) - flux<2>(u[3], gm1));
+        return scale(k * cx, apart(flux<0>(u[0], gm1), flux<0>(u[1], gm1))) +
+               scale(k * cy, apart(flux<1>(u[0], gm1), flux<1>(u[2], gm1))) +
+               scale(k * cz, apart(flux<2>(u[0], gm1), flux<2>(u[3], gm1)));
     }
     // fluxes of direction D at N nodes; ok[s]: whether the M states ub[s] are physical
     template <int D, int N, int M>
@@ -166,16 +192,20 @@ struct WarpTeam {
 #pragma unroll
         for (int n = 0; n < 4; ++n) sh[(n * NV + v) * 32] = u[n][0];
         __syncthreads();
-        if (v < 3) {                        // warp d takes the direction d: node 0 against node 1 + d
-            const int at = (v + 1) * NV;
-            const Vec<NV, R> x = load(0), y = load(at);
-            if (v == 0) store(at, scale(k * cx, flux<0>(x, gm1) - flux<0>(y, gm1)));
-            else if (v == 1) store(at, scale(k * cy, flux<1>(x, gm1) - flux<1>(y, gm1)));
-            else store(at, scale(k * cz, flux<2>(x, gm1) - flux<2>(y, gm1)));
+        if (v < 4) {                        // node 0: all three fluxes, in the slots 0, 4 and 5; node 1 + d: direction d's
+            const Vec<NV, R> x = load(v * NV);
+            if (v == 0) {
+                store(0, flux<0>(x, gm1));
+                store(4 * NV, flux<1>(x, gm1));
+                store(5 * NV, flux<2>(x, gm1));
+            } else if (v == 1) store(NV, flux<0>(x, gm1));
+            else if (v == 2) store(2 * NV, flux<1>(x, gm1));
+            else store(3 * NV, flux<2>(x, gm1));
         }
         __syncthreads();
         V r;
-        r[0] = sh[(NV + v) * 32] + sh[(2 * NV + v) * 32] + sh[(3 * NV + v) * 32];
+        r[0] = k * cx * (sh[v * 32] - sh[(NV + v) * 32]) + k * cy * (sh[(4 * NV + v) * 32] - sh[(2 * NV + v) * 32]) +
+               k * cz * (sh[(5 * NV + v) * 32] - sh[(3 * NV + v) * 32]);
         return r;
     }
     template <int D, int N, int M>

@@ -1,7 +1,6 @@
 """A uniform oblique flow is a fixed point of the predictor at orders 2 and 3: the space-time polynomial of a step is the
-same at its end as at its start, exactly, in both precisions, for Euler and MHD, by teams of warps and by one thread."""
-import itertools
-
+same at its end as at its start, exactly: in FP64, and in FP32 for the nodal forms (whose flux differences are
+subtractions of rounded values), for Euler and MHD, by teams of warps and by one thread."""
 import numpy as np
 import pytest
 
@@ -21,9 +20,14 @@ def ader():
     return p
 
 
-@pytest.mark.parametrize("mhd,fp32,tiled", [(False, False, True), (False, True, True), (False, True, False),
-                                            (True, False, True), (True, True, True)])
-@pytest.mark.parametrize("order,form", list(itertools.product((2, 3), ("modal", "nodal"))))
+# (form, mhd, fp32, tiled); the FP32 modal differences may be contracted with a product, to a last place of a flux
+CASES = [(form, mhd, fp32, tiled) for form in ("modal", "nodal") for mhd, fp32, tiled in
+         ((False, False, True), (True, False, True), (False, True, True), (False, True, False), (True, True, True))
+         if form == "nodal" or not fp32]
+
+
+@pytest.mark.parametrize("form,mhd,fp32,tiled", CASES)
+@pytest.mark.parametrize("order", [2, 3])
 def test_uniform_flow_has_no_time_modes(ader, order, form, mhd, fp32, tiled):
     import torch
     shape, nv = (4, 5, 33), 8 if mhd else 5
