@@ -156,10 +156,9 @@ def alu_peak_tflops(fp32, sm_mhz):
     return 152 * per_clk * sm_mhz * 1e6 / 1e12
 
 
-def traffic_per_launch(kernel, order, form, fp32, zones):
-    """DRAM bytes per launch of `kernel` from the committed ncu capture, scaled to `zones` (traffic grows
-    in proportion to the zones processed); None when the kernel's sources changed since the capture or
-    the capture was of another configuration."""
+def capture_record(kernel, order, form, fp32):
+    """The committed ncu figures of `kernel` (profiles/traffic_<kernel>.json); None when the kernel's sources
+    changed since the capture or the capture was of another configuration."""
     import hashlib
     path = os.path.join(ROOT, "profiles", "traffic_%s.json" % kernel)
     if not os.path.exists(path):
@@ -171,9 +170,22 @@ def traffic_per_launch(kernel, order, form, fp32, zones):
     for f in rec["sources"]:
         p = os.path.join(ROOT, f)
         h.update(open(p).read().encode() if os.path.exists(p) else b"")
-    if h.hexdigest() != rec["sources_sha256"]:
-        return None
-    return rec["bytes_per_zone"] * zones
+    return rec if h.hexdigest() == rec["sources_sha256"] else None
+
+
+def traffic_per_launch(kernel, order, form, fp32, zones):
+    """DRAM bytes per launch of `kernel` from its capture, scaled to `zones` (traffic grows in proportion to the
+    zones processed); None without a current capture."""
+    rec = capture_record(kernel, order, form, fp32)
+    return rec["bytes_per_zone"] * zones if rec else None
+
+
+def fp64_instruction_rate(kernel, order, form, zones, seconds):
+    """10^12 FP64 instructions a second of one launch over `zones` zones, from the count of its capture; None without
+    a current one.  The unit executes two a clock and SM, alu_peak_tflops(False, mhz) / 2 of these."""
+    rec = capture_record(kernel, order, form, False)
+    count = rec.get("fp64_instructions_per_zone") if rec else None
+    return count * zones / seconds / 1e12 if count else None
 
 
 UPDATE_FLOPS = 3 * 5 * 3 + 5 * 2      # Eq. 6 from stored fluxes: per direction and variable a subtract, a
@@ -972,10 +984,14 @@ def gpu_arm(args):
         bound, peak = "alu", alu_peak_tflops(args.fp32, 2070.0)
         basis = "derived: 152 SM x %s at 2070 MHz max clock" % (
             "128 FFMA/clk" if args.fp32 else "2 DFMA/clk (1.25 TFLOP/s nominal FP64)")
-        if not args.fp32:     # the count is of the formulas' FLOPs
-            basis += "; most sums, the WENO weights and the reciprocals run on the integer units, so frac may pass 1"
+    unit, formulas = "TFLOP/s", achieved
+    if bound == "alu" and not args.fp32:
+        # FP64: most of the formulas' FLOPs run on the integer units, so the FP64 unit's share of its rate is taken
+        # from its instructions (counted by ncu for the current sources; none without such a record)
+        unit, peak = "T FP64 instructions/s", peak / 2
+        achieved = fp64_instruction_rate(kname, args.order, args.form, units, k_avg)
     total_ms = sum(v[1] for v in prof.values())
-    roofline = {"bound": bound, "kernel": kname, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+    roofline = {"bound": bound, "kernel": kname, "achieved": achieved, "peak": peak, "unit": unit, "formula_tflops": formulas,
                 "frac": achieved / peak if achieved else None,
                 "traffic": traffic_per_launch(kname, args.order, args.form, args.fp32, zones),
                 "peak_basis": basis,

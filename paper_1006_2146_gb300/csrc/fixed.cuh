@@ -18,8 +18,9 @@
 //
 // Measured (FP64): face states alone took the third-order predictor of 64 x 128 x 128 zones, one thread a zone, from
 // 6.28 to 4.71 ms (3224 -> 2116 FP64 instructions a zone); with the sums of flux modes, teams of warps (team.cuh) and
-// the reciprocals (common.cuh) it takes 2.5 ms and about 1000.  The nodal fourth-order step of 56^3 zones fell from
-// 5.60 to 3.19 ms when its tables moved here.
+// the reciprocals (common.cuh) it takes 2.6 ms and 1053.  The nodal fourth-order step of 56^3 zones fell from 5.60 to
+// 3.0 ms when its tables moved here.  A frame per direction instead of one for all costs 2% of a third-order and 4% of a
+// fourth-order step (256^3 nodal 68.2 -> 69.6 ms, 96^3 modal 14.4 -> 14.9 ms).
 //
 // Range.  HEADROOM = 10 - LSH bits are left above the largest mode for sums; intermediate sums may wrap (the
 // arithmetic is modulo 2^64) as long as no wrapped value is shifted or scaled by a fraction.  Modes of magnitude

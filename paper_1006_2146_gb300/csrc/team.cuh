@@ -9,7 +9,7 @@
 // One thread per zone spilled 5 KB a zone to local memory in FP64 at order 4 (1.6 KB in FP32, 7-14 KB of traffic for
 // MHD), which the L1 of an SM cannot hold for 256 threads; the team spills next to nothing.  At orders 2 and 3 FP64
 // had eight warps per SM beside a tile's face data; the team has 20 to 25, and the third-order predictor and faces of
-// 256^3 zones went from 75 ms (with the states in integers) to 46.
+// 256^3 zones went from 75 ms (with the states in integers) to 42.
 #pragma once
 #include "common.cuh"
 #include "fixed.cuh"
